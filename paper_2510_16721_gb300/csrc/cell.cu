@@ -199,10 +199,10 @@ __global__ void __launch_bounds__(32) k_mapback(const ImgRef *imgs, int count, B
 // split exactly with FMA, sums with Knuth's two-sum), from the FP32 pairs
 // of D and h that k_mapback stores; bv is exact in FP32 by construction.
 // Both keep the offset to ~1e-14 relative of the cell size, far below the
-// FP32 leading part's rounding.
+// FP32 leading part's rounding.  FP64 bands get the FP32 copy in lo.
 __device__ inline void refresh_offset(const ImgScalars &sc, const BandParams *bp, const double *X,
                                       const int *wr, const int *bi, double4_32a &o,
-                                      double4_32a &lo) {
+                                      float4 &lo) {
     double off[3];
     double s[3];
     for (int a = 0; a < 3; ++a)
@@ -218,7 +218,7 @@ __device__ inline void refresh_offset(const ImgScalars &sc, const BandParams *bp
     o.y = off[1];
     o.z = off[2];
     o.w = (double)bi[2];
-    lo.x = lo.y = lo.z = lo.w = 0.0;
+    lo = make_float4((float)off[0], (float)off[1], (float)off[2], (float)bi[2]);
 }
 
 struct F2 {  // unevaluated sum hi + lo of two floats
@@ -351,10 +351,11 @@ __global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev 
         unpack_bin(b.slot_bin[st], bi[0], bi[1], bi[2]);
         const int *wr = b.atom_wrap + ((size_t)tl.img * b.n + i) * 3;
         const T *Xi = (const T *)b.X + ((size_t)tl.img * b.rows + i) * 3;
-        T4 o, lo;
+        T4 o;
+        float4 lo;
         refresh_offset(sc, bp, Xi, wr, bi, o, lo);
         ((T4 *)b.slot_off)[st] = o;
-        ((T4 *)b.slot_off_lo)[st] = lo;
+        b.slot_off_lo[st] = lo;
         return;
     }
     int i = tl.t * TILE + threadIdx.x;
@@ -369,10 +370,11 @@ __global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev 
     b.atom_rank[ai] = rank;
     // offset from the bin centre (the w lane holds the innermost bin index,
     // for the row traversal of the LJ kernel)
-    T4 o, lo;
+    T4 o;
+    float4 lo;
     refresh_offset(sc, bp, Xi, wrap, bi, o, lo);
     ((T4 *)b.atom_off)[ai] = o;
-    ((T4 *)b.atom_off_lo)[ai] = lo;
+    b.atom_off_lo[ai] = lo;
     if (b.ref_X) {  // a skin: reference state of the build (row layout of X)
         T *ref = (T *)b.ref_X + ((size_t)tl.img * b.rows + i) * 3;
         ref[0] = Xi[0];
@@ -516,7 +518,7 @@ __global__ void k_bin_order(const ImgRef *imgs, BandDev *bands) {
             b.slot_bin[base + dst] = pb;
             b.atom_slot[base + idx] = dst;
             ((T4 *)b.slot_off)[base + dst] = ((const T4 *)b.atom_off)[base + idx];
-            ((T4 *)b.slot_off_lo)[base + dst] = ((const T4 *)b.atom_off_lo)[base + idx];
+            b.slot_off_lo[base + dst] = b.atom_off_lo[base + idx];
         }
     }
 }

@@ -219,7 +219,9 @@ struct BandDev {
     // (atom_bin: linear bin index; slot_bin: the bin's three indices packed
     // by pack_bin)
     void *atom_off, *slot_off;   // [ncap][n] x 4 T (x, y, z, pad): offsets, leading part
-    void *atom_off_lo, *slot_off_lo;  // [ncap][n] x 4 T: offset - leading part
+    // [ncap][n] x float4.  FP32 bands: offset - leading part.  FP64 bands: the
+    // offset rounded to FP32 (and the bin index), for distance screens
+    float4 *atom_off_lo, *slot_off_lo;
     // neighbour-list reuse: positions and periodic wraps at the last build
     void *ref_X;         // [ncap][rows][3] T: R~ at the build (the layout of X)
     int *atom_wrap;      // [ncap][n][3]: floor(s) at the build
@@ -304,6 +306,28 @@ __host__ __device__ inline void matmul3(const double *a, const double *b, double
 template <typename T> struct Vec4;
 template <> struct Vec4<float> { using type = float4; };
 template <> struct Vec4<double> { using type = double4_32a; };
+
+// FP32 offsets of one image for distance screens (list builds): an FP64
+// instruction holds a warp's pipe for ~64 cycles here, so FP64 bands screen
+// on their rounded copies and leave FP64 to the entries that remain.
+template <typename T> __device__ inline const float4 *screen_off(const BandDev &b, size_t base) {
+    return (sizeof(T) == 4 ? (const float4 *)b.slot_off : b.slot_off_lo) + base;
+}
+// Squared radius of such a screen that keeps every pair inside r.  The FP32
+// pair vector of a rounded copy is off by at most 2^-24 of the values it is
+// summed from (two offsets of about half a bin each, a bin displacement of up
+// to max m bins, their sums; 4 x 2^-24 covers the three components), and a
+// relative 5e-6 covers the rounding of the square.  FP32 bands screen the
+// offsets they compute with: their margin is 1e-5 of r^2.
+template <typename T>
+__device__ inline float screen_r2(double r, const ImgScalars &sc) {
+    if (sizeof(T) == 4) return (float)(r * r) * 1.00001f;
+    float w = 0.0f;
+    for (int k = 0; k < 9; ++k) w += fabsf(sc.bvf[k]);
+    const int m = max(sc.m[0], max(sc.m[1], sc.m[2]));
+    const float s = (float)r * 1.000005f + 2.4e-7f * (float)(m + 3) * w;
+    return s * s;
+}
 
 // packed stencil offset: 5 bits per axis, biased by 16
 __host__ __device__ inline int pack_code(int d0, int d1, int d2) {

@@ -22,13 +22,18 @@
 
 namespace cfneb {
 
-template <typename T>
-__device__ inline void pair_vec64(const typename Vec4<T>::type &oi, const typename Vec4<T>::type &oil,
-                                  const typename Vec4<T>::type &oj, const typename Vec4<T>::type &ojl,
-                                  const double *c, double *r) {
+// FP32 bands: two-term offsets (ol, jl the remainders); FP64 bands: the offsets
+__device__ inline void pair_vec64(const float4 &oi, const float4 &oil, const float4 &oj,
+                                  const float4 &ojl, const double *c, double *r) {
     r[0] = ((double)oj.x + (double)ojl.x) - ((double)oi.x + (double)oil.x) + c[0];
     r[1] = ((double)oj.y + (double)ojl.y) - ((double)oi.y + (double)oil.y) + c[1];
     r[2] = ((double)oj.z + (double)ojl.z) - ((double)oi.z + (double)oil.z) + c[2];
+}
+__device__ inline void pair_vec64(const double4_32a &oi, const float4 &, const double4_32a &oj,
+                                  const float4 &, const double *c, double *r) {
+    r[0] = oj.x - oi.x + c[0];
+    r[1] = oj.y - oi.y + c[1];
+    r[2] = oj.z - oi.z + c[2];
 }
 
 // Walk the stencil of slot t and call f(r[3]) for every neighbour entry
@@ -39,12 +44,13 @@ __device__ inline void for_neighbours64(const BandDev &b, int img, int t, const 
     using T4 = typename Vec4<T>::type;
     const size_t base = (size_t)img * b.n;
     const T4 *off = (const T4 *)b.slot_off + base;
-    const T4 *offl = (const T4 *)b.slot_off_lo + base;
+    const float4 *offl = b.slot_off_lo + base;
     const int *start = b.bin_start + (size_t)img * (b.nbins_cap + 1);
     const int nb0 = sc.nb[0], nb1 = sc.nb[1], nb2 = sc.nb[2];
     int b0, b1, b2;
     unpack_bin(b.slot_bin[base + t], b0, b1, b2);
-    const T4 oi = off[t], oil = offl[t];
+    const T4 oi = off[t];
+    const float4 oil = offl[t];
     // leading-part screen: its error (~1e-6 relative in FP32) is far inside
     // the 1e-3 margin; the FP64 test below decides
     const T screen2 = (T)(rc2 * 1.001) + (T)1e-6;
@@ -72,7 +78,7 @@ __device__ inline void for_neighbours64(const BandDev &b, int img, int t, const 
                     const T ux = oj.x + cx, uy = oj.y + cy, uz = oj.z + cz;
                     if (!(ux * ux + uy * uy + uz * uz < screen2)) continue;
                     double r[3];
-                    pair_vec64<T>(oi, oil, oj, offl[q], c, r);
+                    pair_vec64(oi, oil, oj, offl[q], c, r);
                     const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
                     if (r2 < rc2 && r2 > 0.0) f(r, r2);
                 }
@@ -114,13 +120,14 @@ __device__ inline int list_vectors64(const BandDev &b, int img, int t, const Img
     using T4 = typename Vec4<T>::type;
     const size_t base = (size_t)img * b.n;
     const T4 *off = (const T4 *)b.slot_off + base;
-    const T4 *offl = (const T4 *)b.slot_off_lo + base;
+    const float4 *offl = b.slot_off_lo + base;
     const int *nslot = b.nbr_slot + (size_t)img * MAXN_TERSOFF * b.n;
     const int *ncode = b.nbr_code + (size_t)img * MAXN_TERSOFF * b.n;
     const int ne = b.nbr_cnt[base + t];
     int bb[3];
     unpack_bin(b.slot_bin[base + t], bb[0], bb[1], bb[2]);
-    const T4 oi = off[t], oil = offl[t];
+    const T4 oi = off[t];
+    const float4 oil = offl[t];
     int cnt = 0;
     for (int e = 0; e < ne; ++e) {
         const int q = nslot[(size_t)e * b.n + t];
@@ -138,7 +145,7 @@ __device__ inline int list_vectors64(const BandDev &b, int img, int t, const Img
             c[k] = dd[0] * sc.bv[k] + dd[1] * sc.bv[3 + k] + dd[2] * sc.bv[6 + k] +
                    tt[0] * sc.dh[k] + tt[1] * sc.dh[3 + k] + tt[2] * sc.dh[6 + k];
         double r[3];
-        pair_vec64<T>(oi, oil, off[q], offl[q], c, r);
+        pair_vec64(oi, oil, off[q], offl[q], c, r);
         const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
         if (r2 < rc * rc && r2 > 0.0) {
             rx[cnt] = r[0];

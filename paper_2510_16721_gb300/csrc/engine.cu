@@ -991,8 +991,8 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
     d.atom_slot = (int *)dalloc(b, na * sizeof(int));
     d.atom_off = dalloc(b, na * 4 * b->ts);
     d.slot_off = dalloc(b, na * 4 * b->ts);
-    d.atom_off_lo = dalloc(b, na * 4 * b->ts);
-    d.slot_off_lo = dalloc(b, na * 4 * b->ts);
+    d.atom_off_lo = (float4 *)dalloc(b, na * sizeof(float4));
+    d.slot_off_lo = (float4 *)dalloc(b, na * sizeof(float4));
     if (skin > 0.0) {
         d.ref_X = dalloc(b, vec);  // the row layout of X (padding rows stay zero)
         d.atom_wrap = (int *)dalloc(b, na * 3 * sizeof(int));

@@ -140,11 +140,12 @@ template <typename T>
 struct LJGeom {
     T bv[9], dh[9], D[9];
     T rc2, sig2, c24, e4, ephi;   // rc^2, sigma^2, 24 eps / sigma^2, 4 eps, phi(rc)
-    T screen;                     // list screen: rl^2 with a 1e-5 relative margin
+    float screen;                 // list screen: rl^2 with a margin (screen_r2)
     int nb[3], m[3];
 };
 template <typename T>
-__device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandParams &bp) {
+__device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandParams &bp,
+                                bool fp64_band = false) {
     if (threadIdx.x == 0) {
         const LJParams p = *(const LJParams *)bp.pot;
         g.rc2 = (T)(p.rc * p.rc);
@@ -153,7 +154,7 @@ __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandPa
         g.e4 = (T)(4.0 * p.eps);
         g.ephi = (T)p.ephi_c;
         // the list-reuse test leaves the same 1e-5 relative margin
-        g.screen = (T)(bp.rl * bp.rl) * (T)1.00001;
+        g.screen = fp64_band ? screen_r2<double>(bp.rl, sc) : screen_r2<float>(bp.rl, sc);
     }
     if (threadIdx.x < 9) {
         g.bv[threadIdx.x] = (T)sc.bv[threadIdx.x];
@@ -233,24 +234,25 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 8 : 4) k_lj(const Tile 
 // as [entry][atom].  Entries inside rc at the build come first and those of
 // the skin shell after them, so that the force kernel's warps mostly agree
 // on which entries have a pair term.  Images that keep their cell list keep
-// their list too.
+// their list too.  The walk runs in FP32 in both precisions: FP64 bands
+// screen on their rounded offsets (entries are tested again in FP64 by the
+// force kernel).
 template <typename T>
-__device__ inline void lj_list_atom(BandDev &b, const Tile &tl, const LJGeom<T> &g, int t) {
-    using T4 = typename Vec4<T>::type;
+__device__ inline void lj_list_atom(BandDev &b, const Tile &tl, const LJGeom<float> &g, int t) {
     const int n = b.n, cap = b.lj_cap;
     const size_t base = (size_t)tl.img * n;
-    const T4 *off = (const T4 *)b.slot_off + base;
+    const float4 *off = screen_off<T>(b, base);
     const int *start = b.bin_start + (size_t)tl.img * (b.nbins_cap + 1);
     uint32_t *L = (uint32_t *)b.nbr_slot + (size_t)tl.img * cap * n + t;
-    const T rc2 = g.rc2, screen = g.screen;
+    const float rc2 = g.rc2, screen = g.screen;
     // the atom itself: slot t at zero offset and wrap
     const uint32_t self =
         lj_entry(t, 2 * g.m[0] + LJ_AXIS * 2 * g.m[1], 2 * g.m[2]);
     int nin = 0, nsh = 0;
-    const T4 oi = off[t];
-    lj_walk<T>(off, start, oi, b.slot_bin[base + t], g.bv, g.dh, g.nb, g.m,
-               [&](int q, T ux, T uy, T uz, int i01, int i2) {
-                   const T r2 = ux * ux + uy * uy + uz * uz;
+    const float4 oi = off[t];
+    lj_walk<float>(off, start, oi, b.slot_bin[base + t], g.bv, g.dh, g.nb, g.m,
+               [&](int q, float ux, float uy, float uz, int i01, int i2) {
+                   const float r2 = ux * ux + uy * uy + uz * uz;
                    if (!(r2 < screen)) return;
                    const uint32_t e = lj_entry(q, i01, i2);
                    if (e == self) return;
@@ -276,13 +278,13 @@ __device__ inline void lj_list_atom(BandDev &b, const Tile &tl, const LJGeom<T> 
 
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles, BandDev *bands) {
-    __shared__ LJGeom<T> g;
+    __shared__ LJGeom<float> g;
     for (int k = blockIdx.x; k < ntiles; k += gridDim.x) {
         const Tile tl = tiles[k];
         BandDev &b = bands[tl.band];
         const ImgScalars &sc = b.sc[tl.img];
         if (b.lj_cap == 0 || !sc.rebuild) continue;  // uniform over the block
-        lj_stage(g, sc, *b.bp);
+        lj_stage<float>(g, sc, *b.bp, sizeof(T) == 8);
         __syncthreads();
         const int t = tl.t * TILE + threadIdx.x;
         if (t < b.n) lj_list_atom<T>(b, tl, g, t);

@@ -52,9 +52,10 @@ constexpr size_t O_BSTART = O_BCOUNT + al(NA_MAX_BINS * sizeof(int));
 constexpr size_t O_BTSUM = O_BSTART + al((NA_MAX_BINS + 1) * sizeof(int));
 constexpr size_t O_INTS = O_BTSUM + al(NA_TSUM * sizeof(int));      // 6 int arrays
 constexpr size_t INT_ARR = al((size_t)NA_MAX_ATOMS * sizeof(int));
-constexpr size_t O_OFFS = O_INTS + 6 * INT_ARR;                       // 4 double4 arrays
+constexpr size_t O_OFFS = O_INTS + 6 * INT_ARR;                       // 2 double4 arrays
 constexpr size_t OFF_ARR = al((size_t)NA_MAX_ATOMS * 4 * sizeof(double));
-constexpr size_t O_PART = O_OFFS + 4 * OFF_ARR;
+constexpr size_t OFFL_ARR = al((size_t)NA_MAX_ATOMS * sizeof(float4));  // 2 float4 arrays
+constexpr size_t O_PART = O_OFFS + 2 * OFF_ARR + 2 * OFFL_ARR;
 constexpr size_t SCRATCH_BYTES = O_PART + al((size_t)NA_TILES * NPART * sizeof(double));
 
 // ~8.5 MB for 32,768 atoms
@@ -192,8 +193,8 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     dv.atom_slot = (int *)(base + O_INTS + 5 * INT_ARR);
     dv.atom_off = base + O_OFFS + 0 * OFF_ARR;
     dv.slot_off = base + O_OFFS + 1 * OFF_ARR;
-    dv.atom_off_lo = base + O_OFFS + 2 * OFF_ARR;
-    dv.slot_off_lo = base + O_OFFS + 3 * OFF_ARR;
+    dv.atom_off_lo = (float4 *)(base + O_OFFS + 2 * OFF_ARR);
+    dv.slot_off_lo = (float4 *)(base + O_OFFS + 2 * OFF_ARR + OFFL_ARR);
     dv.atom_part = (double *)(base + O_PART);
 
     BandParams bp;
