@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev 
     if (!sc.rebuild) {
         // keep the bins of the build: thread = slot, offset from the centre
         // of the slot's bin at the current position (unwrapped as at the build)
-        const int t = tl.t * TILE + threadIdx.x;
+        const int t = tile_atom(b, tl);
         if (t >= b.n) return;
         const size_t st = (size_t)tl.img * b.n + t;
         const int i = b.slot_atom[st];
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev 
         b.slot_off_lo[st] = lo;
         return;
     }
-    int i = tl.t * TILE + threadIdx.x;
+    const int i = tile_atom(b, tl);
     if (i >= b.n) return;
     const T *Xi = (const T *)b.X + ((size_t)tl.img * b.rows + i) * 3;
     int bi[3], wrap[3];
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(TILE) k_bin_scatter(const Tile *tiles, int nti
         const Tile tl = tiles[k];
         BandDev &b = bands[tl.band];
         if (!b.sc[tl.img].rebuild) continue;
-        const int i = tl.t * TILE + threadIdx.x;
+        const int i = tile_atom(b, tl);
         if (i >= b.n) continue;
         const size_t ai = (size_t)tl.img * b.n + i;
         const int *start = b.bin_start + (size_t)tl.img * (b.nbins_cap + 1);

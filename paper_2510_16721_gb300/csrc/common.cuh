@@ -9,7 +9,8 @@
 // ImgScalars[ncap]; per-band constants and FIRE state in BandParams.
 //
 // Kernels are launched over tile tables: each tile is (band, image, t) and
-// covers atoms [t*TILE, (t+1)*TILE) (atom tiles, one thread per atom) or
+// covers atoms [t*tile, (t+1)*tile) (atom tiles: one thread per atom, tile =
+// TILE, or several lanes per atom in the force kernels of small bands) or
 // rows [t*RTILE, (t+1)*RTILE) (row tiles of the band-vector kernels, RPT
 // rows per thread) of that image, so any mix of bands of different sizes
 // runs in one launch.  Partial sums of a tile land in a
@@ -207,6 +208,7 @@ __host__ __device__ inline void unpack_bin(int p, int &b0, int &b1, int &b2) {
 struct BandDev {
     int n, rows, ncap, nbins_cap;
     int atpi, rtpi;      // atom tiles / row tiles per image
+    int tile;            // atoms per atom tile (TILE / lanes per atom)
     void *X, *F, *Fneb, *v;
     ImgScalars *sc;
     BandParams *bp;
@@ -252,6 +254,29 @@ struct ImgRef {
     int band, img;
 };
 
+// The atom (slot) of this thread in a thread-per-atom kernel; n (none) for
+// the threads past the tile's atoms.
+__device__ inline int tile_atom(const BandDev &b, const Tile &tl) {
+    return (int)threadIdx.x < b.tile ? tl.t * b.tile + (int)threadIdx.x : b.n;
+}
+
+// Lanes that share one atom in the LJ force kernels of a band, by the atoms
+// of its moving images: a power of two up to 32 that brings the band to
+// `want` threads.  The band's own sizes decide (not its company in a batch:
+// the order of its sums must not depend on it).
+inline int lanes_per_atom(long long atoms, long long want, int least = 1) {
+    int l = least;
+    while (l < 32 && atoms * l < want) l *= 2;
+    return l;
+}
+// FP64: an SM's four FP64 pipes take one warp instruction per ~64 cycles
+// each: one busy warp per pipe (152 SMs x 4 x 32 lanes) fills them, at least
+// two even out the SMs' shares.
+constexpr long long LJ_LANES_FP64 = 152 * 4 * 32 * 2;
+// FP32, cell walk: latency of the chained bin and offset loads; eight warps
+// per scheduler hide it
+constexpr long long LJ_LANES_FP32 = 152 * 4 * 32 * 8;
+
 struct LJParams {
     double eps, sigma, rc, ephi_c;   // ephi_c = phi(rc) if shifted, else 0
 };
@@ -288,6 +313,29 @@ __device__ inline double rcp64(double x) {
     r = r * (2.0 - x * r);
     r = r * (2.0 - x * r);
     return r;
+}
+// The same bits for a normal x in FP32's range, with the conversions made of
+// integer operations (a conversion to or from FP64 holds the FP64 pipe like
+// any FP64 instruction; integer operations issue at full rate).
+__device__ inline double f2d(float f) {  // (double)f for normal f or +-0
+    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+    const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(m << 29));
+}
+__device__ inline float d2f_pos(double x) {  // a positive x truncated to FP32
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
+}
+// Reciprocal of a positive x from an FP32 seed (error e ~ 2^-22) and one
+// third-order step r (1 + e + e^2): ~1 ulp in three FP64 instructions.
+__device__ inline double rcp64_pos(double x) {
+    const double r = f2d(__fdividef(1.0f, d2f_pos(x)));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+// a < b for non-negative a, b, by their bits
+__device__ inline bool less_pos(double a, double b) {
+    return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
 }
 __device__ inline double rsqrt64(double x) {
     double y = (double)rsqrtf((float)x);
@@ -868,9 +916,13 @@ void launch_shard_fire(BandDev *band, double P, double FF, double VV, double fma
 template <typename T>
 void launch_fire_update(const Tile *tiles, int ntiles, const ImgRef *imgs, int nimg,
                         BandDev *bands, cudaStream_t s);
+// FP64 energies for reporting: per-tile sums (LJ bands / many-body bands),
+// then the images' totals
 template <typename T>
-void launch_energy64(const Tile *tiles, int ntiles, const ImgRef *imgs, int nimg, BandDev *bands,
-                     cudaStream_t s);
+void launch_energy64_lj(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
+template <typename T>
+void launch_energy64(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
+void launch_energy_finalize(const ImgRef *imgs, int nimg, BandDev *bands, cudaStream_t s);
 template <typename T>
 void launch_cartesian(const ImgRef *imgs, int count, int max_n, BandDev *bands, cudaStream_t s);
 template <typename T>

@@ -8,15 +8,12 @@
 // the energy -- and only the energy -- in FP64 from the cell list of the
 // configuration being reported: pair vectors from the two-term offsets (exact
 // positions), bin displacements and wrap corrections in FP64, then the
-// Lennard-Jones, Tersoff or NEP-style energy of Sec. II.B's per-atom split
-// summed over atoms in FP64.  Used by cfneb_get_path and cfneb_evaluate, never inside a
+// Tersoff or NEP-style energy of Sec. II.B's per-atom split (Lennard-Jones:
+// k_lj_energy64, beside its force kernels) summed over atoms in FP64.  Used by cfneb_get_path and cfneb_evaluate, never inside a
 // relaxation step.
 //
 // FP64 arithmetic is scarce on this GPU, so it is spent on the terms only:
-// LJ candidates from the cell-list stencil are screened with the leading
-// (working-precision) parts first, with a relative margin far above their
-// rounding, and only the survivors are formed and tested in FP64; Tersoff
-// walks the atom's neighbour list (rebuilt with the cell list) instead of
+// the atom's neighbour list (rebuilt with the cell list) is walked instead of
 // the stencil.
 #include "common.cuh"
 
@@ -34,57 +31,6 @@ __device__ inline void pair_vec64(const double4_32a &oi, const float4 &, const d
     r[0] = oj.x - oi.x + c[0];
     r[1] = oj.y - oi.y + c[1];
     r[2] = oj.z - oi.z + c[2];
-}
-
-// Walk the stencil of slot t and call f(r[3]) for every neighbour entry
-// within rc (periodic images included, the atom itself excluded).
-template <typename T, typename Fn>
-__device__ inline void for_neighbours64(const BandDev &b, int img, int t, const ImgScalars &sc,
-                                        double rc2, Fn f) {
-    using T4 = typename Vec4<T>::type;
-    const size_t base = (size_t)img * b.n;
-    const T4 *off = (const T4 *)b.slot_off + base;
-    const float4 *offl = b.slot_off_lo + base;
-    const int *start = b.bin_start + (size_t)img * (b.nbins_cap + 1);
-    const int nb0 = sc.nb[0], nb1 = sc.nb[1], nb2 = sc.nb[2];
-    int b0, b1, b2;
-    unpack_bin(b.slot_bin[base + t], b0, b1, b2);
-    const T4 oi = off[t];
-    const float4 oil = offl[t];
-    // leading-part screen: its error (~1e-6 relative in FP32) is far inside
-    // the 1e-3 margin; the FP64 test below decides
-    const T screen2 = (T)(rc2 * 1.001) + (T)1e-6;
-    for (int d0 = -sc.m[0]; d0 <= sc.m[0]; ++d0) {
-        int w0 = b0 + d0, t0 = 0;
-        while (w0 < 0) { w0 += nb0; --t0; }
-        while (w0 >= nb0) { w0 -= nb0; ++t0; }
-        for (int d1 = -sc.m[1]; d1 <= sc.m[1]; ++d1) {
-            int w1 = b1 + d1, t1 = 0;
-            while (w1 < 0) { w1 += nb1; --t1; }
-            while (w1 >= nb1) { w1 -= nb1; ++t1; }
-            for (int d2 = -sc.m[2]; d2 <= sc.m[2]; ++d2) {
-                int w2 = b2 + d2, t2 = 0;
-                while (w2 < 0) { w2 += nb2; --t2; }
-                while (w2 >= nb2) { w2 -= nb2; ++t2; }
-                const int w = (w0 * nb1 + w1) * nb2 + w2;
-                double c[3];
-                for (int k = 0; k < 3; ++k)
-                    c[k] = d0 * sc.bv[k] + d1 * sc.bv[3 + k] + d2 * sc.bv[6 + k] +
-                           t0 * sc.dh[k] + t1 * sc.dh[3 + k] + t2 * sc.dh[6 + k];
-                const T cx = (T)c[0] - oi.x, cy = (T)c[1] - oi.y, cz = (T)c[2] - oi.z;
-                const int q1 = start[w + 1];
-                for (int q = start[w]; q < q1; ++q) {
-                    const T4 oj = off[q];
-                    const T ux = oj.x + cx, uy = oj.y + cy, uz = oj.z + cz;
-                    if (!(ux * ux + uy * uy + uz * uz < screen2)) continue;
-                    double r[3];
-                    pair_vec64(oi, oil, oj, offl[q], c, r);
-                    const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-                    if (r2 < rc2 && r2 > 0.0) f(r, r2);
-                }
-            }
-        }
-    }
 }
 
 // sin a on [0, pi/2] in FP64 by its Taylor series to the a^25 term in
@@ -164,17 +110,10 @@ __global__ void __launch_bounds__(TILE) k_energy64(const Tile *tiles, BandDev *b
     BandDev &b = bands[tl.band];
     const ImgScalars &sc = b.sc[tl.img];
     const BandParams *bp = b.bp;
-    const int t = tl.t * TILE + threadIdx.x;
+    const int t = tile_atom(b, tl);
     double U = 0.0;
     if (t < b.n) {
-        if (bp->kind == 0) {
-            const LJParams p = *(const LJParams *)bp->pot;
-            const double s2 = p.sigma * p.sigma;
-            for_neighbours64<T>(b, tl.img, t, sc, p.rc * p.rc, [&](const double *r, double r2) {
-                const double sr6 = s2 * s2 * s2 / (r2 * r2 * r2);
-                U += 0.5 * (4.0 * p.eps * (sr6 * sr6 - sr6) - p.ephi_c);
-            });
-        } else if (bp->kind == 1) {
+        if (bp->kind == KIND_TERSOFF) {
             const TersoffParams p = *(const TersoffParams *)bp->pot;
             const double rc = p.R + p.D;
             double rx[MAXN_TERSOFF], ry[MAXN_TERSOFF], rz[MAXN_TERSOFF], rd[MAXN_TERSOFF];
@@ -266,15 +205,15 @@ __global__ void k_energy_finalize(const ImgRef *imgs, BandDev *bands) {
 }
 
 template <typename T>
-void launch_energy64(const Tile *tiles, int ntiles, const ImgRef *imgs, int nimg, BandDev *bands,
-                     cudaStream_t s) {
-    if (ntiles <= 0 || nimg <= 0) return;
+void launch_energy64(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
+    if (ntiles <= 0) return;
     k_energy64<T><<<ntiles, TILE, 0, s>>>(tiles, bands);
+}
+void launch_energy_finalize(const ImgRef *imgs, int nimg, BandDev *bands, cudaStream_t s) {
+    if (nimg <= 0) return;
     k_energy_finalize<<<nimg, RED_THREADS, 0, s>>>(imgs, bands);
 }
-template void launch_energy64<float>(const Tile *, int, const ImgRef *, int, BandDev *,
-                                     cudaStream_t);
-template void launch_energy64<double>(const Tile *, int, const ImgRef *, int, BandDev *,
-                                      cudaStream_t);
+template void launch_energy64<float>(const Tile *, int, BandDev *, cudaStream_t);
+template void launch_energy64<double>(const Tile *, int, BandDev *, cudaStream_t);
 
 }  // namespace cfneb

@@ -404,7 +404,11 @@ void enqueue_eval_set(const LaunchSet &ls, Launcher &L, bool forces = true) {
         enqueue_rebuild<T>(ls, L);
     }
     if (!forces) {
-        launch_energy64<T>(ls.atiles, ls.n_atiles, ls.imgs, ls.nimg, d, s);
+        launch_energy64_lj<T>(ls.atiles_lj, ls.n_lj, d, s);
+        launch_energy64_lj<T>(ls.atiles_ljc, ls.n_ljc, d, s);
+        launch_energy64<T>(ls.atiles_ters, ls.n_ters, d, s);
+        launch_energy64<T>(ls.atiles_nep, ls.n_nep, d, s);
+        launch_energy_finalize(ls.imgs, ls.nimg, d, s);
         return;
     }
     if (ls.n_lj) {
@@ -967,7 +971,17 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
     const int row_refine = 1;
     int nb0 = bins_for(A->cell, cap_w) * row_refine, nb1 = bins_for(B->cell, cap_w) * row_refine;
     d.nbins_cap = (int)std::min<long long>((long long)(1.5 * std::max(nb0, nb1)) + 64, 1LL << 26);
-    d.atpi = (n + TILE - 1) / TILE;
+    {
+        const long long atoms = (long long)n * std::max(1, N - 2);
+        const bool cells = pot->kind == CFNEB_LJ && !(skin > 0.0 && n <= LJ_LIST_MAX_ATOMS);
+        int lanes = 1;
+        // FP64 cell walk: at least two lanes (a thread's kept candidates)
+        if (pot->kind == CFNEB_LJ && b->ts == 8)
+            lanes = lanes_per_atom(atoms, LJ_LANES_FP64, cells ? 2 : 1);
+        else if (cells) lanes = lanes_per_atom(atoms, LJ_LANES_FP32);
+        d.tile = TILE / lanes;
+    }
+    d.atpi = (n + d.tile - 1) / d.tile;
     d.rtpi = (rows + RTILE - 1) / RTILE;
     const size_t nc = (size_t)b->ncap;
     const size_t vec = nc * rows * 3 * b->ts;

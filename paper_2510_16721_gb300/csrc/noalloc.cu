@@ -33,7 +33,11 @@ constexpr int NA_MAX_ATOMS = CFNEB_NOALLOC_MAX_ATOMS;
 constexpr int NA_MAX_BINS = 32768;
 constexpr int NA_IMAGES = 2;   // the set-up kernel writes two identical images
 constexpr int NA_ROWS = NA_MAX_ATOMS + 3;
-constexpr int NA_TILES = (NA_MAX_ATOMS + TILE - 1) / TILE;
+// tiles of TILE / lanes atoms: 2 NA_MAX_ATOMS / TILE with two lanes per atom
+// (the least), and with more (fewer than LJ_LANES_FP64 / (lanes / 2) atoms) at
+// most 2 LJ_LANES_FP64 / TILE
+constexpr int NA_TILES = (int)(2 * LJ_LANES_FP64 / TILE) + 2;
+static_assert(NA_TILES * TILE >= 2 * NA_MAX_ATOMS, "two lanes per atom");
 constexpr int NA_TSUM = (NA_MAX_BINS + 1023) / 1024 + 1;
 
 constexpr size_t al(size_t x) { return (x + 255) / 256 * 256; }
@@ -173,7 +177,8 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     dv.rows = n + 3;
     dv.ncap = NA_IMAGES;
     dv.nbins_cap = NA_MAX_BINS;
-    dv.atpi = (n + TILE - 1) / TILE;
+    dv.tile = TILE / lanes_per_atom(n, LJ_LANES_FP64, 2);
+    dv.atpi = (n + dv.tile - 1) / dv.tile;
     dv.rtpi = (n + 3 + RTILE - 1) / RTILE;
     dv.X = base + O_X;
     dv.F = base + O_F;
