@@ -149,7 +149,7 @@ struct BandParams {
     double rl;           // list cutoff rc + skin (0 in records made before skins: rc)
     double bin_w;        // target bin width
     double ftol;         // convergence tolerance (< 0: never converged)
-    double pot[12];      // LJ: eps, sigma, rc, phi(rc) or 0; Tersoff: A, B,
+    double pot[12];      // LJ: LJParams; Tersoff: A, B,
                          // lambda1, lambda2, beta, n, c, d, h, R, D
     int filter, variant, climb, n;
     int N;               // current image count
@@ -260,25 +260,55 @@ __device__ inline int tile_atom(const BandDev &b, const Tile &tl) {
     return (int)threadIdx.x < b.tile ? tl.t * b.tile + (int)threadIdx.x : b.n;
 }
 
-// Lanes that share one atom in the LJ force kernels of a band, by the atoms
-// of its moving images: a power of two up to 32 that brings the band to
-// `want` threads.  The band's own sizes decide (not its company in a batch:
-// the order of its sums must not depend on it).
-inline int lanes_per_atom(long long atoms, long long want, int least = 1) {
-    int l = least;
+// Lanes that share one atom in the LJ force kernels of a band.  The band's own
+// sizes decide (not its company in a batch: the order of its sums must not
+// depend on it).
+//
+// FP64: an SM's FP64 pipe takes a warp instruction every ~16 cycles, whichever
+// of its warps it comes from.  A block of TILE threads costs its share of the
+// atoms' pair terms, `instr` FP64 instructions per atom, plus ~80 per thread
+// for staging and reductions, and the chip takes as long as its fullest SM,
+// whose k blocks keep the pipe k / (k + 0.8) busy (measured at 2 and 4).  Few
+// lanes leave SMs idle, unevenly loaded or short of warps, many pay the
+// overhead (lists of 14,575 atoms: 2 lanes 128 us, 4 lanes 117 us, 8 lanes
+// 108 us).  152: GB300's SMs, also where fewer are visible.
+inline int fp64_lanes(long long n, long long images, double instr, int least = 1) {
+    int best = least;
+    double cost = 1e300;
+    for (int l = least; l <= 32; l *= 2) {
+        const long long tile = TILE / l, blocks = (n + tile - 1) / tile * images;
+        const double c = ((double)((blocks + 151) / 152) + 0.8) * (instr / l + 80.0);
+        if (c < cost) {
+            cost = c;
+            best = l;
+        }
+    }
+    return best;
+}
+inline int lanes_per_atom(long long atoms, long long want) {
+    int l = 1;
     while (l < 32 && atoms * l < want) l *= 2;
     return l;
 }
-// FP64: an SM's four FP64 pipes take one warp instruction per ~64 cycles
-// each: one busy warp per pipe (152 SMs x 4 x 32 lanes) fills them, at least
-// two even out the SMs' shares.
-constexpr long long LJ_LANES_FP64 = 152 * 4 * 32 * 2;
+// FP64 instructions of an atom's LJ pair terms at the cell's mean density
+inline double lj_fp64_instr(double n, double volume, double rc) {
+    return 36.0 * n / volume * 4.18879020478639 * rc * rc * rc;
+}
 // FP32, cell walk: latency of the chained bin and offset loads; eight warps
 // per scheduler hide it
 constexpr long long LJ_LANES_FP32 = 152 * 4 * 32 * 8;
 
 struct LJParams {
     double eps, sigma, rc, ephi_c;   // ephi_c = phi(rc) if shifted, else 0
+    // derived on the host (an FP64 divide per block is a chain of ~20 FP64
+    // instructions on one thread): sigma^2, 24 eps / sigma^2, 4 eps, rc^2
+    double sig2, c24, e4, rc2;
+    __host__ void derive() {
+        sig2 = sigma * sigma;
+        c24 = 24.0 * eps / (sigma * sigma);
+        e4 = 4.0 * eps;
+        rc2 = rc * rc;
+    }
 };
 
 

@@ -902,10 +902,9 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
         double eps = pot->eps, sig = pot->sigma;
         rc = pot->rc;
         double sr6 = std::pow(sig / rc, 6.0);
-        P.pot[0] = eps;
-        P.pot[1] = sig;
-        P.pot[2] = rc;
-        P.pot[3] = pot->shift_energy ? 4.0 * eps * (sr6 * sr6 - sr6) : 0.0;
+        LJParams lp{eps, sig, rc, pot->shift_energy ? 4.0 * eps * (sr6 * sr6 - sr6) : 0.0};
+        lp.derive();
+        std::memcpy(P.pot, &lp, sizeof(lp));
     } else if (pot->kind == CFNEB_NEP) {
         rc = pot->nep_rc;
         P.pot[0] = rc;
@@ -977,7 +976,8 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
         int lanes = 1;
         // FP64 cell walk: at least two lanes (a thread's kept candidates)
         if (pot->kind == CFNEB_LJ && b->ts == 8)
-            lanes = lanes_per_atom(atoms, LJ_LANES_FP64, cells ? 2 : 1);
+            lanes = fp64_lanes(n, std::max(1, N - 2),
+                               lj_fp64_instr(n, std::fabs(det3(A->cell)), rc), cells ? 2 : 1);
         else if (cells) lanes = lanes_per_atom(atoms, LJ_LANES_FP32);
         d.tile = TILE / lanes;
     }

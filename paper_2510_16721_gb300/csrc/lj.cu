@@ -163,17 +163,16 @@ __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandPa
                                 bool fp64_band, bool list) {
     if (threadIdx.x == 0) {
         const LJParams p = *(const LJParams *)bp.pot;
-        g.rc2 = (T)(p.rc * p.rc);
-        g.sig2 = (T)(p.sigma * p.sigma);
-        g.c24 = (T)(24.0 * p.eps / (p.sigma * p.sigma));
-        g.e4 = (T)(4.0 * p.eps);
+        g.rc2 = (T)p.rc2;
+        g.sig2 = (T)p.sig2;
+        g.c24 = (T)p.c24;
+        g.e4 = (T)p.e4;
         g.ephi = (T)p.ephi_c;
-        // the list-reuse test leaves the same 1e-5 relative margin
         // lists cover rl; a walk that evaluates its candidates is cut at rc
         // (the test in T decides: the margin only has to cover the screen's
         // FP32 rounding)
         if (list) g.screen = fp64_band ? screen_r2<double>(bp.rl, sc) : screen_r2<float>(bp.rl, sc);
-        else g.screen = fp64_band ? screen_r2<double>(p.rc, sc) : (float)(p.rc * p.rc) * 1.001f;
+        else g.screen = fp64_band ? screen_r2<double>(p.rc, sc) : (float)p.rc2 * 1.001f;
     }
     if (threadIdx.x < 9) {
         g.bv[threadIdx.x] = (T)sc.bv[threadIdx.x];
@@ -598,9 +597,10 @@ __global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles,
 // MINB: resident blocks per SM the register allocation is held to (the
 // autotuner picks it with the bin width: more blocks hide more gather
 // latency, fewer leave more registers for the look-ahead)
-template <typename T, int MINB>
+template <int MINB>
 __global__ void __launch_bounds__(TILE, MINB) k_lj_nbr(const Tile *tiles, BandDev *bands) {
-    using T4 = typename Vec4<T>::type;
+    using T = float;
+    using T4 = float4;
     Tile tl = tiles[blockIdx.x];
     BandDev &b = bands[tl.band];
     if (b.lj_cap == 0) return;  // uniform over the block: the direct path runs
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_lj_nbr(const Tile *tiles, BandDe
     __shared__ LJGeom<T> g;
     __shared__ T4 s_c01[LJ_AXIS * LJ_AXIS];
     __shared__ T4 s_c2[32];
-    lj_stage(g, sc, *b.bp, sizeof(T) == 8, true);
+    lj_stage(g, sc, *b.bp, false, true);
     __syncthreads();
     {
         const int L0 = 2 * (2 * g.m[0] + 1), L1 = 2 * (2 * g.m[1] + 1), L2 = 2 * (2 * g.m[2] + 1);
@@ -675,6 +675,85 @@ __global__ void __launch_bounds__(TILE, MINB) k_lj_nbr(const Tile *tiles, BandDe
     lj_finish(A, g, b, tl, t, t < n);
 }
 
+// The FP64 list path: bound by the FP64 pipe (~64 cycles per warp instruction),
+// and in bands of few atoms by the chain of one thread's entries (31 atoms, 110
+// entries each: 129 us with one thread per atom, four warps busy; 11 us with 32
+// lanes.  2,915 atoms x 5 images: 146 us, now 108 us of which the FP64 pipe's
+// share is 65 us).  An atom's entries are dealt to its lanes (BandDev::tile), every entry is screened in
+// FP32 on the rounded offsets first, and only entries inside the screen (78 of
+// 110; the shell entries stand last in a list, so a warp skips most of them
+// together) reach FP64.
+struct LJDispF {  // LJDisp rounded, for the screen
+    float4 c01[LJ_C01], a[2][32], c2[32];
+};
+__global__ void __launch_bounds__(TILE, 4) k_lj_nbr64(const Tile *tiles, BandDev *bands) {
+    using T4 = typename Vec4<double>::type;
+    Tile tl = tiles[blockIdx.x];
+    BandDev &b = bands[tl.band];
+    if (b.lj_cap == 0) return;  // uniform over the block: the direct path runs
+    const ImgScalars &sc = b.sc[tl.img];
+    __shared__ LJGeom<double> g;
+    __shared__ LJDisp D;
+    __shared__ LJDispF Df;
+    lj_stage(g, sc, *b.bp, true, false);
+    __syncthreads();
+    lj_disp_stage(D, g);
+    __syncthreads();
+    const bool table = D.l0 * D.l1 <= LJ_C01;
+    for (int k = threadIdx.x; k < LJ_C01 + 96; k += TILE) {
+        const double *v = k < 64 ? D.a[k >> 5][k & 31] : k < 96 ? D.c2[k & 31] : D.c01 + 3 * (k - 96);
+        if (k >= 96 && (!table || k - 96 >= D.l0 * D.l1)) break;
+        const float4 f = make_float4((float)v[0], (float)v[1], (float)v[2], 0.0f);
+        if (k < 64) Df.a[k >> 5][k & 31] = f;
+        else if (k < 96) Df.c2[k & 31] = f;
+        else Df.c01[k - 96] = f;
+    }
+    __syncthreads();
+    const int n = b.n, cap = b.lj_cap, lanes = TILE / b.tile, lane = threadIdx.x % lanes;
+    const int t = tl.t * b.tile + (int)threadIdx.x / lanes;
+    const size_t base = (size_t)tl.img * n;
+    const T4 *off = (const T4 *)b.slot_off + base;
+    const float4 *offf = b.slot_off_lo + base;
+    const double rc2 = g.rc2, sig2 = g.sig2;
+    const float screen = g.screen;
+    const int l0 = D.l0;
+    LJAcc<double> A;
+    if (t < n) {
+        const uint32_t *L = (const uint32_t *)b.nbr_slot + (size_t)tl.img * cap * n + t;
+        const int cnt = b.nbr_cnt[base + t];
+        const T4 oi = off[t];
+        const float4 of = offf[t];
+        uint32_t e = lane < cnt ? L[(size_t)lane * n] : 0u;
+        for (int k = lane; k < cnt; k += lanes) {
+            const uint32_t c = e;
+            if (k + lanes < cnt) e = L[(size_t)(k + lanes) * n];
+            const int q = (int)(c & 0x1FFFFu), i01 = (int)((c >> 17) & 1023u), i2 = (int)(c >> 27);
+            const int i1 = i01 / LJ_AXIS, i0 = i01 - LJ_AXIS * i1;
+            const float4 oq = offf[q], f2 = Df.c2[i2];
+            float4 f;
+            if (table) {
+                f = Df.c01[i0 + l0 * i1];
+            } else {
+                const float4 fa = Df.a[0][i0], fb = Df.a[1][i1];
+                f = make_float4(fa.x + fb.x, fa.y + fb.y, fa.z + fb.z, 0.0f);
+            }
+            const float ux = (oq.x - of.x) + (f.x + f2.x), uy = (oq.y - of.y) + (f.y + f2.y),
+                        uz = (oq.z - of.z) + (f.z + f2.z);
+            if (!(ux * ux + uy * uy + uz * uz < screen)) continue;
+            const T4 oj = off[q];
+            double x = oj.x - oi.x, y = oj.y - oi.y, z = oj.z - oi.z;
+            lj_disp(D, (uint32_t)(i0 | (i1 << 5) | (i2 << 10)), x, y, z);
+            const double r2 = x * x + y * y + z * z;
+            // r2 == 0: a padding entry (the atom itself)
+            if (lj_inside(r2, rc2)) A.pair(x, y, z, r2, sig2);
+        }
+    }
+    A.fx = lane_group_sum(A.fx, lanes);
+    A.fy = lane_group_sum(A.fy, lanes);
+    A.fz = lane_group_sum(A.fz, lanes);
+    lj_finish(A, g, b, tl, t, t < n && lane == 0);
+}
+
 template <typename T>
 void launch_lj(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
@@ -692,14 +771,14 @@ template <typename T>
 void launch_lj_nbr(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s, int minb) {
     if (ntiles <= 0) return;
     if (sizeof(T) == 8) {
-        k_lj_nbr<T, 4><<<ntiles, TILE, 0, s>>>(tiles, bands);
+        k_lj_nbr64<<<ntiles, TILE, 0, s>>>(tiles, bands);
         return;
     }
     switch (minb) {
-        case 5: k_lj_nbr<T, 5><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
-        case 6: k_lj_nbr<T, 6><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
-        case 8: k_lj_nbr<T, 8><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
-        default: k_lj_nbr<T, 7><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
+        case 5: k_lj_nbr<5><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
+        case 6: k_lj_nbr<6><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
+        case 8: k_lj_nbr<8><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
+        default: k_lj_nbr<7><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
     }
 }
 template <typename T>

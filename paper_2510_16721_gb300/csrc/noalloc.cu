@@ -33,11 +33,9 @@ constexpr int NA_MAX_ATOMS = CFNEB_NOALLOC_MAX_ATOMS;
 constexpr int NA_MAX_BINS = 32768;
 constexpr int NA_IMAGES = 2;   // the set-up kernel writes two identical images
 constexpr int NA_ROWS = NA_MAX_ATOMS + 3;
-// tiles of TILE / lanes atoms: 2 NA_MAX_ATOMS / TILE with two lanes per atom
-// (the least), and with more (fewer than LJ_LANES_FP64 / (lanes / 2) atoms) at
-// most 2 LJ_LANES_FP64 / TILE
-constexpr int NA_TILES = (int)(2 * LJ_LANES_FP64 / TILE) + 2;
-static_assert(NA_TILES * TILE >= 2 * NA_MAX_ATOMS, "two lanes per atom");
+// tiles of 128 / lanes atoms, most at 32 lanes (4 atoms)
+constexpr int NA_TILES = NA_MAX_ATOMS / 4;
+static_assert(TILE == 128, "four atoms per tile at 32 lanes");
 constexpr int NA_TSUM = (NA_MAX_BINS + 1023) / 1024 + 1;
 
 constexpr size_t al(size_t x) { return (x + 255) / 256 * 256; }
@@ -62,7 +60,7 @@ constexpr size_t OFFL_ARR = al((size_t)NA_MAX_ATOMS * sizeof(float4));  // 2 flo
 constexpr size_t O_PART = O_OFFS + 2 * OFF_ARR + 2 * OFFL_ARR;
 constexpr size_t SCRATCH_BYTES = O_PART + al((size_t)NA_TILES * NPART * sizeof(double));
 
-// ~8.5 MB for 32,768 atoms
+// ~8.3 MB for 32,768 atoms
 __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
 
 struct H1 {
@@ -177,7 +175,7 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     dv.rows = n + 3;
     dv.ncap = NA_IMAGES;
     dv.nbins_cap = NA_MAX_BINS;
-    dv.tile = TILE / lanes_per_atom(n, LJ_LANES_FP64, 2);
+    dv.tile = TILE / fp64_lanes(n, 1, lj_fp64_instr(n, std::fabs(det3(cell)), rc), 2);
     dv.atpi = (n + dv.tile - 1) / dv.tile;
     dv.rtpi = (n + 3 + RTILE - 1) / RTILE;
     dv.X = base + O_X;
@@ -219,10 +217,9 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     bp.kind = CFNEB_LJ;
     bp.ci = -1;
     const double sr6 = std::pow(sigma / rc, 6.0);
-    bp.pot[0] = eps;
-    bp.pot[1] = sigma;
-    bp.pot[2] = rc;
-    bp.pot[3] = shift_energy ? 4.0 * eps * (sr6 * sr6 - sr6) : 0.0;
+    LJParams lp{eps, sigma, rc, shift_energy ? 4.0 * eps * (sr6 * sr6 - sr6) : 0.0};
+    lp.derive();
+    memcpy(bp.pot, &lp, sizeof(lp));
     H1 h1;
     for (int k = 0; k < 9; ++k) h1.h[k] = cell[k];
 

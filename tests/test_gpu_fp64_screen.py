@@ -48,3 +48,21 @@ def test_fp64_lists_screened_in_fp32(g, oracle_mod, pot, bin_scale, skin):
     for i in range(1, N - 1):
         assert _rel(st["F"][i], ob.F[i]) <= 1e-9, i
         assert _rel(st["X"][i], ob.X[i]) <= 1e-9, i
+
+
+@pytest.mark.parametrize("reps", [(2, 2, 2), (3, 4, 5), (6, 6, 7), (11, 9, 10)])
+def test_fp64_lj_lists_with_lanes(g, oracle_mod, reps):
+    """FP64 LJ bands with neighbour lists give an atom 32 to 4 lanes by their
+    size (31, 239, 1007 and 3959 atoms, each with a ragged last tile): one
+    step from displaced positions against the oracle."""
+    R0, h0, R1, h1 = ci.lj_vacancy_hop(ci.LJ_A, reps)
+    h1s = ci.strained_cell(h1, 3, 0.01)
+    kw = dict(k=1.0, dt=0.01, cell_filter=True, noise=ci.interior_noise(4, 4, len(R0), 0.02))
+    gb = gpu_band(g, R0, h0, ci.affine(R1, h1, h1s), h1s, 4, g.lj_potential(), **kw)
+    ob = oracle_band(oracle_mod, oracle_mod.LJ(), R0, h0, ci.affine(R1, h1, h1s), h1s, 4, **kw)
+    gb.step(1)
+    ob.step(1)
+    st = gb.get_state()
+    for i in (1, 2):
+        assert _rel(st["F"][i], ob.F[i]) <= 1e-10, i
+        assert _rel(st["virials"][i], ob.info[i]["V"]) <= 1e-10, i
