@@ -344,9 +344,9 @@ __device__ inline double rcp64(double x) {
     r = r * (2.0 - x * r);
     return r;
 }
-// The same bits for a normal x in FP32's range, with the conversions made of
-// integer operations (a conversion to or from FP64 holds the FP64 pipe like
-// any FP64 instruction; integer operations issue at full rate).
+// Conversions made of integer operations (a conversion to or from FP64 holds
+// the FP64 pipe like any FP64 instruction; integer operations issue at full
+// rate), for normal values of FP32's range.
 __device__ inline double f2d(float f) {  // (double)f for normal f or +-0
     const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
     const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
@@ -356,12 +356,47 @@ __device__ inline float d2f_pos(double x) {  // a positive x truncated to FP32
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
 }
+// x lies in FP32's normal range (and is positive), with room for a square
+__device__ inline bool in_f32_range(double x) {
+    return (unsigned)__double2hiint(x) - 0x38100000u < 0x47E00000u - 0x38100000u;
+}
 // Reciprocal of a positive x from an FP32 seed (error e ~ 2^-22) and one
-// third-order step r (1 + e + e^2): ~1 ulp in three FP64 instructions.
+// third-order step r (1 + e + e^2): ~1 ulp in three FP64 instructions; outside
+// FP32's range a divide.
 __device__ inline double rcp64_pos(double x) {
+    if (!in_f32_range(x)) return 1.0 / x;
     const double r = f2d(__fdividef(1.0f, d2f_pos(x)));
     const double e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);
+}
+// sqrt(x) and 1 / sqrt(x) of a positive x: an FP32 seed and two coupled
+// Newton steps (~1 ulp, nine FP64 instructions)
+__device__ inline void sqrt_rcp64(double x, double &g, double &ig) {
+    if (!in_f32_range(x)) {
+        g = sqrt(x);
+        ig = 1.0 / g;
+        return;
+    }
+    const double y = f2d(rsqrtf(d2f_pos(x)));
+    double h = 0.5 * y;
+    g = x * y;
+    double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    ig = 2.0 * fma(h, r, h);
+}
+// sin a on [0, pi/2] in FP64 by its Taylor series to the a^25 term in
+// nested form (truncation below 2e-23 at pi/2); the coefficients
+// 1 / ((2k)(2k + 1)) are compile-time constants (an FP64 divide is a long
+// dependent sequence on this GPU)
+__device__ inline double sin_quarter64(double a) {
+    const double a2 = a * a;
+    double p = 1.0;
+#pragma unroll
+    for (int k = 12; k >= 1; --k) p = 1.0 - a2 * (1.0 / (double)((2 * k) * (2 * k + 1))) * p;
+    return a * p;
 }
 // a < b for non-negative a, b, by their bits
 __device__ inline bool less_pos(double a, double b) {

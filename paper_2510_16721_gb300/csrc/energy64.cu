@@ -33,18 +33,6 @@ __device__ inline void pair_vec64(const double4_32a &oi, const float4 &, const d
     r[2] = oj.z - oi.z + c[2];
 }
 
-// sin a on [0, pi/2] in FP64 by its Taylor series to the a^25 term in
-// nested form (truncation below 2e-23 at pi/2); the coefficients
-// 1 / ((2k)(2k + 1)) are compile-time constants (an FP64 divide is a long
-// dependent sequence on this GPU)
-__device__ inline double sin_quarter64(double a) {
-    const double a2 = a * a;
-    double p = 1.0;
-#pragma unroll
-    for (int k = 12; k >= 1; --k) p = 1.0 - a2 * (1.0 / (double)((2 * k) * (2 * k + 1))) * p;
-    return a * p;
-}
-
 // b = (1 + (beta zeta)^n)^(-1/2n) with m2n = -1/2n: x = (beta zeta)^n from
 // log and exp; for x < 1e-3 (carbon: x ~ 1e-5) b = exp(m2n log1p(x)) by
 // their series (log1p to x^5: 2e-13 relative at the bound, exp to y^6);

@@ -979,6 +979,9 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
             lanes = fp64_lanes(n, std::max(1, N - 2),
                                lj_fp64_instr(n, std::fabs(det3(A->cell)), rc), cells ? 2 : 1);
         else if (cells) lanes = lanes_per_atom(atoms, LJ_LANES_FP32);
+        // FP64 many-body kernels take four lanes per atom: one pass per block
+        // (32 atoms) where the band's blocks would leave SMs idle, else four
+        if (pot->kind != CFNEB_LJ && b->ts == 8 && atoms < 152 * 2 * TILE) lanes = 4;
         d.tile = TILE / lanes;
     }
     d.atpi = (n + d.tile - 1) / d.tile;

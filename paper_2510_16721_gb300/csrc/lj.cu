@@ -98,8 +98,9 @@ __device__ inline uint32_t lj_entry(int q, int i01, int i2) {
 // so it is one contiguous range of atoms (one pair of bin-start loads
 // instead of one per bin) and each atom's displacement comes from its own
 // innermost bin index, stored in the offset's fourth lane.  Rows that wrap
-// are walked bin by bin.
-template <typename Visit>
+// are walked bin by bin.  AHEAD: the next candidate is loaded under the
+// current one's work (worth its registers where few warps are resident).
+template <bool AHEAD, typename Visit>
 __device__ inline void lj_row(const float4 *off, const int *start, const float4 &oi, int b0, int b1,
                               int b2, int d0, int d1, const float *s_bv, const float *s_dh,
                               const int *s_nb, const int *s_m, Visit &&visit) {
@@ -120,10 +121,11 @@ __device__ inline void lj_row(const float4 *off, const int *start, const float4 
     const float cz = (d0 * s_bv[2] + d1 * s_bv[5]) + (t0 * s_dh[2] + t1 * s_dh[5]);
     if (row_ok) {
         const int q0 = start[rowbase + b2 - m2], q1 = start[rowbase + b2 + m2 + 1];
-        float4 next = q0 < q1 ? off[q0] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 next;
+        if (AHEAD && q0 < q1) next = off[q0];
         for (int q = q0; q < q1; ++q) {
-            const float4 oj = next;
-            if (q + 1 < q1) next = off[q + 1];  // under this candidate's arithmetic
+            const float4 oj = AHEAD ? next : off[q];
+            if (AHEAD && q + 1 < q1) next = off[q + 1];
             const float d2 = oj.w - (float)b2;
             const float ex = cx + d2 * s_bv[6], ey = cy + d2 * s_bv[7], ez = cz + d2 * s_bv[8];
             // no wrap along the row: t2 = 0, and |d2| <= m2 < nb2
@@ -148,6 +150,23 @@ __device__ inline void lj_row(const float4 *off, const int *start, const float4 
         }
     }
 }
+
+// A lane's rows of the stencil: lane, lane + lanes, ... of the (2 m0 + 1)(2 m1
+// + 1) rows, as (d0, d1) stepped without a division per row.
+struct LJRows {
+    int d0, d1, m0, m1;
+    __device__ LJRows(const int *m, int lane) : d0(-m[0]), d1(-m[1]), m0(m[0]), m1(m[1]) {
+        step(lane);
+    }
+    __device__ bool more() const { return d0 <= m0; }
+    __device__ void step(int k) {
+        d1 += k;
+        while (d1 > m1) {
+            d1 -= 2 * m1 + 1;
+            ++d0;
+        }
+    }
+};
 
 // Per-block staging of an image's bin geometry and the LJ constants in T
 template <typename T>
@@ -298,32 +317,32 @@ __device__ inline void lj_walk_keep(const BandDev &b, const Tile &tl, const LJGe
     const uint32_t zero = (uint32_t)(2 * g.m[0] | (2 * g.m[1] << 5) | (2 * g.m[2] << 10));
     uint32_t *row = kp.word + tid * LJ_KEEP_STRIDE;
     int kept = 0;
-    const int r1 = 2 * g.m[1] + 1, rows = (2 * g.m[0] + 1) * r1;
-    for (int r0 = 0; r0 < rows; r0 += lanes) {  // uniform over the block
-        const int r = r0 + lane;
-        if (active && r < rows)
-            lj_row(off, start, oi, b0, b1, b2, r / r1 - g.m[0], r % r1 - g.m[1], g.bvf, g.dhf,
-                   g.nb, g.m, [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
-                       if (!(ux * ux + uy * uy + uz * uz < g.screen)) return;
-                       if (HALF && q < t) return;
-                       const uint32_t code = (uint32_t)(i0 | (i1 << 5) | (i2 << 10));
-                       if (q == t && (code == zero || (HALF && lj_back(code, g.m, g.nb))))
-                           return;
-                       if (kept == cap) {  // a very dense row: this thread alone
-                           for (int k = 0; k < kept; ++k) {
-                               if (wide) term((int)row[2 * k], row[2 * k + 1], tid);
-                               else term((int)(row[k] & 0x1FFFFu), row[k] >> 17, tid);
-                           }
-                           kept = 0;
-                       }
-                       if (wide) {
-                           row[2 * kept] = (uint32_t)q;
-                           row[2 * kept + 1] = code;
-                       } else {
-                           row[kept] = (uint32_t)q | (code << 17);
-                       }
-                       ++kept;
-                   });
+    LJRows r(g.m, lane);
+    const int rows = (2 * g.m[0] + 1) * (2 * g.m[1] + 1);
+    for (int r0 = 0; r0 < rows; r0 += lanes, r.step(lanes)) {  // uniform over the block
+        if (active && r.more())
+            lj_row<true>(
+                off, start, oi, b0, b1, b2, r.d0, r.d1, g.bvf, g.dhf, g.nb, g.m,
+                [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
+                    if (!(ux * ux + uy * uy + uz * uz < g.screen)) return;
+                    if (HALF && q < t) return;
+                    const uint32_t code = (uint32_t)(i0 | (i1 << 5) | (i2 << 10));
+                    if (q == t && (code == zero || (HALF && lj_back(code, g.m, g.nb)))) return;
+                    if (kept == cap) {  // a very dense row: this thread alone
+                        for (int k = 0; k < kept; ++k) {
+                            if (wide) term((int)row[2 * k], row[2 * k + 1], tid);
+                            else term((int)(row[k] & 0x1FFFFu), row[k] >> 17, tid);
+                        }
+                        kept = 0;
+                    }
+                    if (wide) {
+                        row[2 * kept] = (uint32_t)q;
+                        row[2 * kept + 1] = code;
+                    } else {
+                        row[kept] = (uint32_t)q | (code << 17);
+                    }
+                    ++kept;
+                });
         if (__any_sync(0xffffffffu, kept > cap - room)) lj_share(kp, group, wide, kept, term);
     }
     lj_share(kp, group, wide, kept, term);
@@ -376,7 +395,7 @@ __device__ inline void lj_disp(const LJDisp &D, uint32_t code, double &x, double
 
 template <typename T> __global__ void k_lj(const Tile *tiles, BandDev *bands);
 template <>
-__global__ void __launch_bounds__(TILE, 7) k_lj<float>(const Tile *tiles, BandDev *bands) {
+__global__ void __launch_bounds__(TILE, 8) k_lj<float>(const Tile *tiles, BandDev *bands) {
     Tile tl = tiles[blockIdx.x];
     BandDev &b = bands[tl.band];
     if (b.lj_cap > 0) return;  // uniform over the block: the list path runs
@@ -395,14 +414,13 @@ __global__ void __launch_bounds__(TILE, 7) k_lj<float>(const Tile *tiles, BandDe
         int b0, b1, b2;
         unpack_bin(b.slot_bin[base + t], b0, b1, b2);
         const float4 oi = off[t];
-        const int r1 = 2 * g.m[1] + 1, rows = (2 * g.m[0] + 1) * r1;
-        for (int r = lane; r < rows; r += lanes)
-            lj_row(off, start, oi, b0, b1, b2, r / r1 - g.m[0], r % r1 - g.m[1], g.bvf, g.dhf,
-                   g.nb, g.m, [&](int, float ux, float uy, float uz, int, int, int) {
-                       const float r2 = ux * ux + uy * uy + uz * uz;
-                       // r2 == 0 only for the atom itself at zero shift
-                       if (lj_inside(r2, rc2)) A.pair(ux, uy, uz, r2, sig2);
-                   });
+        for (LJRows r(g.m, lane); r.more(); r.step(lanes))
+            lj_row<false>(off, start, oi, b0, b1, b2, r.d0, r.d1, g.bvf, g.dhf, g.nb, g.m,
+                          [&](int, float ux, float uy, float uz, int, int, int) {
+                              const float r2 = ux * ux + uy * uy + uz * uz;
+                              // r2 == 0 only for the atom itself at zero shift
+                              if (lj_inside(r2, rc2)) A.pair(ux, uy, uz, r2, sig2);
+                          });
     }
     A.fx = lane_group_sum(A.fx, lanes);
     A.fy = lane_group_sum(A.fy, lanes);
@@ -543,16 +561,17 @@ __device__ inline void lj_list_atom(BandDev &b, const Tile &tl, const LJGeom<flo
     unpack_bin(b.slot_bin[base + t], b0, b1, b2);
     for (int d0 = -g.m[0]; d0 <= g.m[0]; ++d0)
         for (int d1 = -g.m[1]; d1 <= g.m[1]; ++d1)
-            lj_row(off, start, oi, b0, b1, b2, d0, d1, g.bvf, g.dhf, g.nb, g.m,
-                   [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
-                       const float r2 = ux * ux + uy * uy + uz * uz;
-                       if (!(r2 < screen)) return;
-                       const uint32_t e = lj_entry(q, i0 + LJ_AXIS * i1, i2);
-                       if (e == self) return;
-                       if (nin + nsh < cap) L[(size_t)(r2 < rc2 ? nin : cap - 1 - nsh) * n] = e;
-                       if (r2 < rc2) ++nin;
-                       else ++nsh;
-                   });
+            lj_row<false>(off, start, oi, b0, b1, b2, d0, d1, g.bvf, g.dhf, g.nb, g.m,
+                          [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
+                              const float r2 = ux * ux + uy * uy + uz * uz;
+                              if (!(r2 < screen)) return;
+                              const uint32_t e = lj_entry(q, i0 + LJ_AXIS * i1, i2);
+                              if (e == self) return;
+                              if (nin + nsh < cap)
+                                  L[(size_t)(r2 < rc2 ? nin : cap - 1 - nsh) * n] = e;
+                              if (r2 < rc2) ++nin;
+                              else ++nsh;
+                          });
     const int total = nin + nsh;
     if (total > cap) {
         // not every slot of [0, cap) holds an entry: none is read

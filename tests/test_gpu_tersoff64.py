@@ -1,0 +1,60 @@
+"""FP64 Tersoff site terms: four lanes per atom in small bands, one thread per
+atom in large ones, each with atoms of at most four list entries and with more
+(compressed and disordered carbon, a graphite sheet, ragged last tiles), in
+single points against the oracle at 1e-10, and the two forms against each
+other across the size where the rule switches."""
+import numpy as np
+import pytest
+
+import cfneb_inputs as ci
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2510_16721_gb300 as g
+    g.build()
+    return g
+
+
+def _carbon(kind, reps, drop, seed):
+    Rg, hg, Rd, hd = ci.tersoff_endpoint_cells()
+    R, h = ci.tile(Rg, hg, reps) if kind == "graphite" else ci.tile(Rd, hd, reps)
+    rng = np.random.default_rng(seed)
+    if kind == "dense":  # 7% shorter bonds: second neighbours enter the shell
+        R, h = 0.86 * R, 0.86 * h
+    R = R + rng.normal(0.0, 0.12 if kind == "disordered" else 0.03, R.shape)
+    keep = np.sort(rng.permutation(len(R))[:len(R) - drop])
+    return R[keep], h
+
+
+@pytest.mark.parametrize("kind", ["graphite", "diamond", "dense", "disordered"])
+@pytest.mark.parametrize("reps,drop", [((1, 1, 1), 0), ((2, 1, 2), 1), ((3, 2, 2), 0),
+                                       ((4, 3, 2), 5)])
+def test_small_points(g, oracle_mod, kind, reps, drop):
+    R, h = _carbon(kind, reps, drop, 3)
+    e, Fo, Vo = oracle_mod.Tersoff().evaluate(R, h)
+    E, F, V = g.evaluate([(R, h)], g.tersoff_potential(), g.FP64)
+    s = max(1.0, np.max(np.abs(Fo)))
+    assert abs(E[0] - e.sum()) <= 1e-10 * max(1.0, np.abs(e).sum())
+    assert np.max(np.abs(F[0] - Fo)) <= 1e-10 * s
+    assert np.max(np.abs(V[0] - Vo)) <= 1e-10 * max(1.0, np.max(np.abs(Vo)))
+
+
+@pytest.mark.parametrize("kind", ["graphite", "dense", "disordered"])
+def test_both_forms_agree(g, kind):
+    """The same disordered cell once (lanes) and tiled past the rule's line
+    (one thread per atom): per-atom forces agree and the totals scale."""
+    R, h = _carbon(kind, (8, 6, 5), 3, 5)
+    Rt, ht = ci.tile(R, h, (3, 3, 3))
+    assert len(R) < 152 * 2 * 128 <= len(Rt)
+    (E1, F1, V1), (E2, F2, V2) = (g.evaluate([s], g.tersoff_potential(), g.FP64)
+                                  for s in ((R, h), (Rt, ht)))
+    s = max(1.0, np.max(np.abs(F1[0])))
+    assert np.max(np.abs(F2[0].reshape(27, -1, 3) - F1[0])) <= 1e-10 * s
+    assert abs(E2[0] - 27 * E1[0]) <= 1e-10 * abs(E2[0])
+    assert np.max(np.abs(V2[0] - 27 * V1[0])) <= 1e-9 * max(1.0, np.max(np.abs(V2[0])))
