@@ -296,8 +296,9 @@ int cfneb_destroy_band(cfneb_band *band);
 /* Single-point evaluation of `count` structures (any cells, any sizes):
  * energies[count], forces[sum n_i x 3] (Cartesian, structures back to
  * back), virials[count x 9].  Forces and virials come from the kernels of a
- * relaxation step in the requested precision; energies from the FP64
- * energy pass.  Output pointers may be NULL.  Synchronises. */
+ * relaxation step in the requested precision; energies are FP64 totals (mixed
+ * precision: of an FP64 energy pass).  Output pointers may be NULL.
+ * Synchronises. */
 int cfneb_evaluate(const cfneb_structure *structures, int32_t count,
                    const cfneb_potential *potential, int32_t precision, void *cuda_stream,
                    double *energies, double *forces, double *virials);

@@ -714,15 +714,17 @@ __global__ void k_midpoint(BandDev *band, int img) {
 // interior atom rows.  Everything in FP64, stored as T.
 template <typename T>
 __global__ void k_setup(const double *R0, const double *R1, const double *noise, int N,
-                        BandDev *band, const double *h1) {
+                        BandDev *band, Mat3 H1) {
     BandDev &b = *band;
     const BandParams *bp = b.bp;
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = b.n;
+    const double *h1 = H1.m;
+    __shared__ double h1inv[9];
+    if (threadIdx.x == 0) inv3(h1, h1inv);
+    __syncthreads();
     if (row > n) return;
     const size_t stride = (size_t)b.rows * 3;
-    double h1inv[9];
-    inv3(h1, h1inv);
     if (row < n) {
         double s0[3], s1[3], a0[3], a1[3];
         for (int a = 0; a < 3; ++a) {
@@ -777,6 +779,72 @@ __global__ void k_setup(const double *R0, const double *R1, const double *noise,
     }
 }
 
+// Single points (see launch_points_load).  Lattice and padding rows of X are
+// zero: c (B - I) with B = I.
+template <typename T>
+__global__ void __launch_bounds__(TILE) k_points_load(const Tile *tiles, BandDev *bands) {
+    const Tile tl = tiles[blockIdx.x];
+    const BandDev &b = bands[tl.band];
+    T *X = (T *)b.X;
+    const int first = tl.t * b.tile * 3, end = min((tl.t + 1) * b.tile, b.n) * 3;
+    for (int e = first + threadIdx.x; e < end; e += TILE) X[e] = (T)b.cart[e];
+    if (tl.t == 0)
+        for (int e = b.n * 3 + threadIdx.x; e < b.rows * 3; e += TILE) X[e] = (T)0;
+}
+template <typename T>
+__global__ void __launch_bounds__(TILE) k_points_store(const Tile *tiles, BandDev *bands) {
+    const Tile tl = tiles[blockIdx.x];
+    const BandDev &b = bands[tl.band];
+    const T *F = (const T *)b.F;
+    const int first = tl.t * b.tile * 3, end = min((tl.t + 1) * b.tile, b.n) * 3;
+    for (int e = first + threadIdx.x; e < end; e += TILE) b.cart[e] = (double)F[e];
+}
+
+// State exchange on the device: the band's padded T rows against [N][n + 3][3]
+// doubles in the scratch array (converted by one thread per value: host loops
+// over 98,304-atom bands took as long as tens of steps).  blockIdx.y = image.
+template <typename T>
+__global__ void k_state_load(BandDev *band, int n, double c) {
+    BandDev &b = *band;
+    const size_t img = blockIdx.y;
+    const int per = (n + 3) * 3, e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= b.rows * 3) return;
+    double v = 0.0;
+    if (e < per) {
+        v = b.cart[img * per + e];
+        const int l = e - 3 * n;
+        if (l >= 0 && l % 4 == 0) v -= c;
+    }
+    ((T *)b.X)[img * (size_t)b.rows * 3 + e] = (T)v;
+}
+template <typename T>
+__global__ void k_state_store(BandDev *band, int which, int N, int n, double c) {
+    BandDev &b = *band;
+    const size_t img = blockIdx.y;
+    const int per = (n + 3) * 3, e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= per) return;
+    const void *src = which == 0 ? b.X : which == 1 ? b.F : b.Fneb;
+    double v = (double)((const T *)src)[img * (size_t)b.rows * 3 + e];
+    const int l = e - 3 * n;
+    if (which == 0 && l >= 0 && l % 4 == 0) v += c;
+    if (which == 2 && (img == 0 || (int)img == N - 1)) v = 0.0;
+    b.cart[img * per + e] = v;
+}
+__global__ void k_fire_reset(BandDev *band) {
+    BandParams *p = band->bp;
+    p->dt = p->dt0;
+    p->alpha = 0.1;
+    p->npos = 0;
+    p->fresh = 1;
+    p->stale = 1;
+}
+__global__ void k_set_control(BandDev *band, double ftol, long long move_limit) {
+    BandParams *p = band->bp;
+    p->ftol = ftol;
+    p->converged = 0;
+    p->move_limit = move_limit;
+}
+
 // per band: moves, converged, status, fmax, climbing image, N (batch polling)
 __global__ void k_gather_status(BandDev *bands, int nb, double *out) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -800,8 +868,30 @@ void launch_gather_status(BandDev *bands, int nb, double *out, cudaStream_t s) {
 
 template <typename T>
 void launch_setup(const double *R0, const double *R1, const double *noise, int n, int N,
-                  BandDev *band, cudaStream_t s, const double *h1) {
+                  BandDev *band, cudaStream_t s, const Mat3 &h1) {
     k_setup<T><<<(n + 1 + 127) / 128, 128, 0, s>>>(R0, R1, noise, N, band, h1);
+}
+
+template <typename T>
+void launch_points_load(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
+    if (ntiles > 0) k_points_load<T><<<ntiles, TILE, 0, s>>>(tiles, bands);
+}
+template <typename T>
+void launch_points_store(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
+    if (ntiles > 0) k_points_store<T><<<ntiles, TILE, 0, s>>>(tiles, bands);
+}
+template <typename T>
+void launch_state_load(BandDev *band, int N, int n, double c, cudaStream_t s) {
+    const int rows = (n + 3 + 3) / 4 * 4;
+    k_state_load<T><<<dim3((rows * 3 + 255) / 256, N), 256, 0, s>>>(band, n, c);
+}
+template <typename T>
+void launch_state_store(BandDev *band, int which, int N, int n, double c, cudaStream_t s) {
+    k_state_store<T><<<dim3(((n + 3) * 3 + 255) / 256, N), 256, 0, s>>>(band, which, N, n, c);
+}
+void launch_fire_reset(BandDev *band, cudaStream_t s) { k_fire_reset<<<1, 1, 0, s>>>(band); }
+void launch_set_control(BandDev *band, double ftol, long long move_limit, cudaStream_t s) {
+    k_set_control<<<1, 1, 0, s>>>(band, ftol, move_limit);
 }
 
 template <typename T>
@@ -857,7 +947,11 @@ void launch_midpoint(BandDev *band, int img, int rows, cudaStream_t s) {
                                         cudaStream_t);                                    \
     template void launch_midpoint<T>(BandDev *, int, int, cudaStream_t);                  \
     template void launch_setup<T>(const double *, const double *, const double *, int, int, \
-                                  BandDev *, cudaStream_t, const double *);
+                                  BandDev *, cudaStream_t, const Mat3 &);               \
+    template void launch_points_load<T>(const Tile *, int, BandDev *, cudaStream_t);      \
+    template void launch_points_store<T>(const Tile *, int, BandDev *, cudaStream_t);     \
+    template void launch_state_load<T>(BandDev *, int, int, double, cudaStream_t);        \
+    template void launch_state_store<T>(BandDev *, int, int, int, double, cudaStream_t);
 CFNEB_INST(float)
 CFNEB_INST(double)
 #undef CFNEB_INST

@@ -523,11 +523,12 @@ __global__ void k_bin_order(const ImgRef *imgs, BandDev *bands) {
     }
 }
 
-// Cartesian positions R = R~ D (FP64) of the listed images, for output.
+// Cartesian positions R = R~ D (FP64) of a band's images (blockIdx.y), for
+// output.
 template <typename T>
-__global__ void k_cartesian(const ImgRef *imgs, BandDev *bands) {
-    ImgRef r = imgs[blockIdx.y];
-    BandDev &b = bands[r.band];
+__global__ void k_cartesian(BandDev *band) {
+    const ImgRef r = {0, (int)blockIdx.y};
+    BandDev &b = *band;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= b.n) return;
     const ImgScalars &sc = b.sc[r.img];
@@ -570,10 +571,10 @@ void launch_bin_order(const ImgRef *imgs, int count, int max_bins, BandDev *band
     k_bin_order<T><<<grid, 128, 0, s>>>(imgs, bands);
 }
 template <typename T>
-void launch_cartesian(const ImgRef *imgs, int count, int max_n, BandDev *bands, cudaStream_t s) {
-    if (count <= 0 || max_n <= 0) return;
-    dim3 grid((max_n + 127) / 128, count);
-    k_cartesian<T><<<grid, 128, 0, s>>>(imgs, bands);
+void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {
+    if (N <= 0 || n <= 0) return;
+    dim3 grid((n + 127) / 128, N);
+    k_cartesian<T><<<grid, 128, 0, s>>>(band);
 }
 
 #define CFNEB_INST(T)                                                                     \
@@ -581,7 +582,7 @@ void launch_cartesian(const ImgRef *imgs, int count, int max_n, BandDev *bands, 
     template void launch_bin_assign<T>(const Tile *, int, BandDev *, cudaStream_t,       \
                                        cudaGraphConditionalHandle, int);                 \
     template void launch_bin_order<T>(const ImgRef *, int, int, BandDev *, cudaStream_t); \
-    template void launch_cartesian<T>(const ImgRef *, int, int, BandDev *, cudaStream_t);
+    template void launch_cartesian<T>(int, int, BandDev *, cudaStream_t);
 CFNEB_INST(float)
 CFNEB_INST(double)
 #undef CFNEB_INST

@@ -242,7 +242,8 @@ struct BandDev {
     // partial sums
     double *atom_part;   // [ncap][atpi][NPART]
     double *row_part;    // [ncap][rtpi][NPART]
-    // Cartesian output scratch [ncap][n][3] doubles (get_path)
+    // double scratch [ncap][n + 3][3]: Cartesian positions (get_path), state
+    // exchange, set-up inputs
     double *cart;
 };
 
@@ -989,12 +990,32 @@ template <typename T>
 void launch_energy64(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
 void launch_energy_finalize(const ImgRef *imgs, int nimg, BandDev *bands, cudaStream_t s);
 template <typename T>
-void launch_cartesian(const ImgRef *imgs, int count, int max_n, BandDev *bands, cudaStream_t s);
+void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s);
 template <typename T>
 void launch_midpoint(BandDev *band, int img, int rows, cudaStream_t s);
 void launch_gather_status(BandDev *bands, int nb, double *out, cudaStream_t s);
+struct Mat3 {
+    double m[9];
+};
 template <typename T>
 void launch_setup(const double *R0, const double *R1, const double *noise, int n, int N,
-                  BandDev *band, cudaStream_t s, const double *h1);
+                  BandDev *band, cudaStream_t s, const Mat3 &h1);
+// Single points: image 0 of every tile's band from the Cartesian positions in
+// BandDev::cart (R~ = R: the reference cell is the structure's own), and its
+// forces back into them
+template <typename T>
+void launch_points_load(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
+template <typename T>
+void launch_points_store(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
+// Vectors [N][n + 3][3] of doubles in BandDev::cart to and from the band's
+// padded rows (which: 0 X, 1 F, 2 f_NEB; X with the lattice rows c B of the C
+// ABI, f_NEB with zero end images)
+template <typename T>
+void launch_state_load(BandDev *band, int N, int n, double c, cudaStream_t s);
+template <typename T>
+void launch_state_store(BandDev *band, int which, int N, int n, double c, cudaStream_t s);
+// FIRE restart and stale lists; tolerance and move budget
+void launch_fire_reset(BandDev *band, cudaStream_t s);
+void launch_set_control(BandDev *band, double ftol, long long move_limit, cudaStream_t s);
 
 }  // namespace cfneb

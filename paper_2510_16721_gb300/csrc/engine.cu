@@ -129,7 +129,7 @@ struct cfneb_band {
     double h0[9]{}, c = 1.0;
     BandDev dv{};                // host copy holding device pointers
     BandDev *d_self = nullptr;   // device copy (array of one)
-    std::vector<void *> allocs;
+    void *slab = nullptr;        // the one allocation behind dv and the tables
     size_t bytes = 0;
     long long last_change = 0;
     long long last_check = -1;
@@ -152,6 +152,8 @@ struct cfneb_band {
     int *d_band_ids = nullptr;
     Tile *d_scratch_tiles = nullptr;   // tables for ad-hoc image sets
     ImgRef *d_scratch_imgs = nullptr;
+    std::vector<Tile> up_tiles;  // sources of the scratch tables' last upload
+    std::vector<ImgRef> up_imgs;
     int n_atiles = 0, n_rtiles = 0, n_imgs = 0;
     // graphs: one step, and GRAPH_STEPS steps
     cudaGraphExec_t gexec = nullptr, gexec_n = nullptr;
@@ -170,16 +172,32 @@ struct cfneb_band {
 
 namespace {
 
-void *dalloc(cfneb_band *b, size_t bytes) {
+// One device allocation carved into arrays (256-byte aligned): a band's ~35
+// arrays used to cost a cudaMalloc and a cudaFree each.
+struct Arena {
+    std::vector<std::pair<char *, size_t>> want;  // address of the pointer, offset
+    size_t total = 0, bytes = 0;                  // with and without alignment
+    template <typename P> void add(P **p, size_t n) {
+        want.push_back({(char *)p, total});
+        n = std::max<size_t>(n, 16);
+        total += (n + 255) / 256 * 256;
+        bytes += n;
+    }
+    void place(void *base) const {
+        for (const auto &w : want) {
+            void *q = (char *)base + w.second;
+            std::memcpy(w.first, &q, sizeof(q));
+        }
+    }
+};
+
+void *device_alloc(size_t bytes) {
     void *p = nullptr;
-    if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMalloc(&p, bytes);
+    const cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
         g_last_error = std::string("cudaMalloc: ") + cudaGetErrorString(e);
         throw CudaFail{e};
     }
-    b->allocs.push_back(p);
-    b->bytes += bytes;
     return p;
 }
 
@@ -187,8 +205,8 @@ void free_band(cfneb_band *b) {
     if (!b) return;
     if (b->s) cudaStreamSynchronize(b->s);
     if (b->own_s) b->s = b->own_s;
-    for (void *p : b->allocs) cudaFree(p);
-    b->allocs.clear();
+    if (b->slab) cudaFree(b->slab);
+    b->slab = nullptr;
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->gexec_n) cudaGraphExecDestroy(b->gexec_n);
     for (auto e : b->prof_ev) cudaEventDestroy(e);
@@ -532,6 +550,11 @@ int launches_per_step(const cfneb_band *b) {
 // times to (ms, n)
 template <typename F>
 void profiled(cudaStream_t s, std::vector<cudaEvent_t> &ev, double *ms, long long *n, F enq) {
+    while (ev.size() < 2 * 64) {  // made when profiling first needs them
+        cudaEvent_t e = nullptr;
+        CK(cudaEventCreate(&e));
+        ev.push_back(e);
+    }
     Launcher L;
     L.prof = true;
     L.ev = &ev;
@@ -610,10 +633,13 @@ void steps(cfneb_band *b, int n) {
     launch_steps(b->gexec, b->gexec_n, b->s, n, enq);
 }
 
-// evaluate an arbitrary list of images of the band (endpoints, new images)
-void eval_images(cfneb_band *b, const std::vector<int> &imgs) {
-    std::vector<ImgRef> im;
-    std::vector<Tile> at;
+// launch tables of an arbitrary list of images of the band, into the scratch
+// tables (every caller waits for the stream before the next upload)
+int upload_images(cfneb_band *b, const std::vector<int> &imgs) {
+    std::vector<ImgRef> &im = b->up_imgs;
+    std::vector<Tile> &at = b->up_tiles;
+    im.clear();
+    at.clear();
     for (int i : imgs) {
         im.push_back({0, i});
         for (int t = 0; t < b->dv.atpi; ++t) at.push_back({0, i, t, 0});
@@ -622,40 +648,42 @@ void eval_images(cfneb_band *b, const std::vector<int> &imgs) {
                        cudaMemcpyHostToDevice, b->s));
     CK(cudaMemcpyAsync(b->d_scratch_tiles, at.data(), at.size() * sizeof(Tile),
                        cudaMemcpyHostToDevice, b->s));
-    Launcher L;
-    if (b->precision == CFNEB_MIXED)
-        enqueue_eval<float>(b, L, b->d_scratch_imgs, (int)im.size(), b->d_scratch_tiles,
-                            (int)at.size());
-    else
-        enqueue_eval<double>(b, L, b->d_scratch_imgs, (int)im.size(), b->d_scratch_tiles,
-                             (int)at.size());
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(b->s));
+    return (int)at.size();
 }
 
-// FP64 energies (ImgScalars::E64) of the images' current coordinates:
-// map-back, cell list and the FP64 energy kernel, no forces
-void refine_energies(cfneb_band *b, const std::vector<int> &imgs) {
-    std::vector<ImgRef> im;
-    std::vector<Tile> at;
-    for (int i : imgs) {
-        im.push_back({0, i});
-        for (int t = 0; t < b->dv.atpi; ++t) at.push_back({0, i, t, 0});
-    }
-    if (im.empty()) return;
-    CK(cudaMemcpyAsync(b->d_scratch_imgs, im.data(), im.size() * sizeof(ImgRef),
-                       cudaMemcpyHostToDevice, b->s));
-    CK(cudaMemcpyAsync(b->d_scratch_tiles, at.data(), at.size() * sizeof(Tile),
-                       cudaMemcpyHostToDevice, b->s));
+// evaluate a list of images of the band (endpoints)
+void eval_images(cfneb_band *b, const std::vector<int> &imgs) {
+    const int nt = upload_images(b, imgs);
     Launcher L;
     if (b->precision == CFNEB_MIXED)
-        enqueue_eval<float>(b, L, b->d_scratch_imgs, (int)im.size(), b->d_scratch_tiles,
-                            (int)at.size(), false);
+        enqueue_eval<float>(b, L, b->d_scratch_imgs, (int)imgs.size(), b->d_scratch_tiles, nt);
     else
-        enqueue_eval<double>(b, L, b->d_scratch_imgs, (int)im.size(), b->d_scratch_tiles,
-                             (int)at.size(), false);
+        enqueue_eval<double>(b, L, b->d_scratch_imgs, (int)imgs.size(), b->d_scratch_tiles, nt);
     CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(b->s));
+}
+
+// FP64 energies (ImgScalars::E64) of the current coordinates: map-back, cell
+// list and the FP64 energy kernel, no forces.  The interior images keep their
+// lists while those still hold (what moves them leaves the displacements the
+// decision needs); the end images, which a caller may have replaced, are
+// evaluated from new ones.
+void refine_interior(cfneb_band *b) {
+    if (b->N < 3) return;
+    const LaunchSet ls = band_step_set(b);
+    Launcher L;
+    if (b->precision == CFNEB_MIXED) enqueue_eval_set<float>(ls, L, false);
+    else enqueue_eval_set<double>(ls, L, false);
+    CK(cudaGetLastError());
+}
+void refine_ends(cfneb_band *b) {
+    upload_images(b, {0, b->N - 1});
+    Launcher L;
+    if (b->precision == CFNEB_MIXED)
+        enqueue_eval<float>(b, L, b->d_scratch_imgs, 2, b->d_scratch_tiles, 2 * b->dv.atpi, false);
+    else
+        enqueue_eval<double>(b, L, b->d_scratch_imgs, 2, b->d_scratch_tiles, 2 * b->dv.atpi,
+                             false);
+    CK(cudaGetLastError());
 }
 
 void read_params(cfneb_band *b) {
@@ -678,18 +706,12 @@ void lattice_rows_public(const cfneb_band *b, double *x, double sign) {
     for (int e = 0; e < 9; e += 4) x[(size_t)b->n * 3 + e] += sign * b->c;
 }
 
-// write FIRE reset values into the device params and zero velocities
+// FIRE reset values, zero velocities, every list rebuilt (images were
+// inserted, removed or moved)
 void fire_reset(cfneb_band *b) {
-    read_params(b);
-    BandParams *p = b->h_bp;
-    p->dt = p->dt0;
-    p->alpha = 0.1;
-    p->npos = 0;
-    p->fresh = 1;
-    p->stale = 1;  // images were inserted, removed or moved: rebuild every list
-    CK(cudaMemcpyAsync(b->dv.bp, p, sizeof(BandParams), cudaMemcpyHostToDevice, b->s));
+    launch_fire_reset(b->d_self, b->s);
+    CK(cudaGetLastError());
     CK(cudaMemsetAsync(b->dv.v, 0, (size_t)b->ncap * b->dv.rows * 3 * b->ts, b->s));
-    CK(cudaStreamSynchronize(b->s));
 }
 
 void set_N(cfneb_band *b, int N) {
@@ -813,13 +835,9 @@ void refine(cfneb_band *b) {
 }
 
 void set_control(cfneb_band *b, double ftol, long long move_limit) {
-    read_params(b);
+    launch_set_control(b->d_self, ftol, move_limit, b->s);
+    CK(cudaGetLastError());
     b->move_limit = move_limit;
-    b->h_bp->ftol = ftol;
-    b->h_bp->converged = 0;
-    b->h_bp->move_limit = move_limit;
-    CK(cudaMemcpyAsync(b->dv.bp, b->h_bp, sizeof(BandParams), cudaMemcpyHostToDevice, b->s));
-    CK(cudaStreamSynchronize(b->s));
     b->ftol = ftol;
 }
 
@@ -859,44 +877,29 @@ void run_steps(cfneb_band *b, long long n_eval, bool stop_on_converged, int *sta
     }
 }
 
-cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
-                   const cfneb_potential *pot, const cfneb_cell_filter *cf,
-                   const cfneb_options *opt, void *stream, int *err) {
-    *err = CFNEB_OK;
-    cfneb_band *b = new cfneb_band();
-    b->user = (cudaStream_t)stream;
-    b->n = A->n_atoms;
-    b->N = N;
-    b->opt = *opt;
-    if (b->opt.n_max < N) b->opt.n_max = N;
-    if (b->opt.n_min < 3) b->opt.n_min = 3;
-    b->ncap = b->opt.n_max;
-    b->precision = opt->precision;
-    b->ts = (opt->precision == CFNEB_MIXED) ? 4 : 8;
-    b->kind = pot->kind;
-    b->filt = cf ? *cf : cfneb_cell_filter{1, CFNEB_ROTFREE_B, 0.0, 0.0};
-    std::memcpy(b->h0, A->cell, sizeof(b->h0));
-    // lattice scale: the caller's c, or J = Omega0^(1/3) n^(1/6) (the scale
-    // of the generalized solid-state NEB: it keeps the lattice rows'
-    // stiffness per unit of X independent of n), or n_atoms
-    if (b->filt.cell_factor > 0)
-        b->c = b->filt.cell_factor;
-    else if (b->filt.cell_factor == CFNEB_CELL_FACTOR_J)
-        b->c = std::cbrt(std::fabs(det3(A->cell))) * std::pow((double)b->n, 1.0 / 6.0);
-    else
-        b->c = (double)b->n;
-    CK(cudaStreamCreateWithFlags(&b->s, cudaStreamNonBlocking));
-    CK(cudaStreamCreateWithFlags(&b->s_body, cudaStreamNonBlocking));
-    b->fork.create();
-    CK(cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming));
-    CK(cudaMallocHost((void **)&b->h_bp, sizeof(BandParams)));
-    b->prof_ev.resize(2 * 64);
-    for (auto &e : b->prof_ev) CK(cudaEventCreate(&e));
+// the argument checks of a potential; *rc = its cutoff
+int check_potential(const cfneb_potential *pot, double *rc) {
+    if (pot->kind != CFNEB_LJ && pot->kind != CFNEB_TERSOFF && pot->kind != CFNEB_NEP)
+        return CFNEB_ERR_INVALID_ARG;
+    if (pot->kind == CFNEB_NEP) {
+        if (!pot->nep_weights || !(pot->nep_rc > 0.0) || !std::isfinite(pot->nep_rc))
+            return CFNEB_ERR_INVALID_ARG;
+        for (int k = 0; k < NEP_NW; ++k)
+            if (!std::isfinite(pot->nep_weights[k])) return CFNEB_ERR_INVALID_ARG;
+    }
+    if (pot->kind == CFNEB_LJ && (pot->rc <= 0 || pot->sigma <= 0 || pot->eps <= 0))
+        return CFNEB_ERR_INVALID_ARG;
+    *rc = pot->kind == CFNEB_NEP ? pot->nep_rc : pot->rc;
+    if (pot->kind == CFNEB_TERSOFF) {
+        const bool dflt = std::all_of(pot->tersoff, pot->tersoff + 11,
+                                      [](double v) { return v == 0.0; });
+        *rc = dflt ? kTersoff1988C[9] + kTersoff1988C[10] : pot->tersoff[9] + pot->tersoff[10];
+    }
+    return CFNEB_OK;
+}
 
-    // potential
-    BandParams &P = *b->h_bp;
-    std::memset(&P, 0, sizeof(P));
+// the potential's constants in the band parameters; returns its cutoff
+double fill_potential(const cfneb_potential *pot, BandParams &P) {
     double rc;
     if (pot->kind == CFNEB_LJ) {
         double eps = pot->eps, sig = pot->sigma;
@@ -930,6 +933,314 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
         P.tpf.load(tp);
         P.tpd.load(tp);
     }
+    return rc;
+}
+
+// Device to caller's (pageable) memory.  A fresh array's pages are touched
+// first: a copy into pages that nobody has written yet faults them in one by
+// one from the device (26 MB: 24 ms, against ~1 ms once touched).
+void to_host(void *dst, const void *src, size_t bytes, cudaStream_t s) {
+    for (size_t i = 0; i < bytes; i += 4096) ((volatile char *)dst)[i] = 0;
+    if (bytes) ((volatile char *)dst)[bytes - 1] = 0;
+    CK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
+}
+
+// no NaN or Inf among n doubles (exponent bits, four at a time)
+bool all_finite(const double *x, size_t n) {
+    const uint64_t E = 0x7ff0000000000000ull;
+    uint64_t bad[4] = {0, 0, 0, 0}, w[4];
+    size_t i = 0;
+    for (; i + 4 <= n; i += 4) {
+        std::memcpy(w, x + i, sizeof(w));
+        for (int k = 0; k < 4; ++k) bad[k] |= (uint64_t)((w[k] & E) == E);
+    }
+    for (; i < n; ++i)
+        if (!std::isfinite(x[i])) return false;
+    return !(bad[0] | bad[1] | bad[2] | bad[3]);
+}
+
+// NEP weights in FP64 and FP32 at w (device)
+void upload_nep(const cfneb_potential *pot, double *w, BandDev &d, cudaStream_t s) {
+    float hf[NEP_NW];
+    for (int k = 0; k < NEP_NW; ++k) hf[k] = (float)pot->nep_weights[k];
+    float *wf = (float *)(w + NEP_NW);
+    CK(cudaMemcpyAsync(w, pot->nep_weights, NEP_NW * sizeof(double), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(wf, hf, NEP_NW * sizeof(float), cudaMemcpyHostToDevice, s));
+    CK(cudaStreamSynchronize(s));  // hf is a stack array
+    d.nep_w = w;
+    d.nep_wf = wf;
+}
+
+// atoms per atom tile (see common.cuh: lanes per atom)
+int atom_tile(const cfneb_potential *pot, int precision, long long n, long long images,
+              double volume, double rc, bool cells) {
+    const long long atoms = n * images;
+    int lanes = 1;
+    // FP64 cell walk: at least two lanes (a thread's kept candidates)
+    if (pot->kind == CFNEB_LJ && precision == CFNEB_FP64)
+        lanes = fp64_lanes(n, images, lj_fp64_instr((double)n, volume, rc), cells ? 2 : 1);
+    else if (cells) lanes = lanes_per_atom(atoms, LJ_LANES_FP32);
+    // FP64 many-body kernels take four lanes per atom (32 atoms per block)
+    // where the band's blocks would leave SMs idle, else one
+    if (pot->kind != CFNEB_LJ && precision == CFNEB_FP64 && atoms < 152 * 2 * TILE) lanes = 4;
+    return TILE / lanes;
+}
+
+std::tuple<int, int, int, int> tune_class(const cfneb_potential *pot, int precision, int n,
+                                          double volume, double rc) {
+    const double dens = (double)n / volume * rc * rc * rc;
+    return std::make_tuple(pot->kind, precision, (int)std::floor(std::log2((double)std::max(1, n))),
+                           (int)std::floor(2.0 * std::log2(std::max(dens, 1e-3))));
+}
+
+// ---- single points -----------------------------------------------------------
+//
+// A structure is one image whose reference cell is its own (D = I, forces are
+// Cartesian), evaluated from a fresh cell list without a skin.  A group of
+// structures is laid out as one set of bands in one allocation and goes
+// through each kernel of an evaluation in one launch, on the caller's stream.
+// (It used to be a three-image band each: both end images evaluated, then
+// another cell list for the energies, ~37 allocations; three carbon cells of 8
+// to 480 atoms 3.1 ms, a 98,304-atom one 3.4 ms.)  The FP64 energies come from
+// the same cell list; an FP64 evaluation's own energy is one already.
+
+constexpr long long POINT_GROUP_ATOMS = 1LL << 18;
+
+// every reason to refuse a structure (all CFNEB_ERR_INVALID_ARG)
+int check_point(const cfneb_structure &S, const cfneb_potential *pot, int precision) {
+    if (!S.positions || S.n_atoms <= 0) return CFNEB_ERR_INVALID_ARG;
+    if (S.types)
+        for (int i = 1; i < S.n_atoms; ++i)
+            if (S.types[i] != S.types[0]) return CFNEB_ERR_INVALID_ARG;
+    double rc = 0.0;
+    const int st = check_potential(pot, &rc);
+    if (st != CFNEB_OK) return st;
+    if (!(std::fabs(det3(S.cell)) > 0)) return CFNEB_ERR_INVALID_ARG;
+    if (!all_finite(S.cell, 9) || !all_finite(S.positions, 3 * (size_t)S.n_atoms))
+        return CFNEB_ERR_INVALID_ARG;
+    if (precision != CFNEB_FP64 && precision != CFNEB_MIXED) return CFNEB_ERR_INVALID_ARG;
+    if (!(0.0 <= rc) || !stencil_reaches(S.cell, rc)) return CFNEB_ERR_INVALID_ARG;
+    return CFNEB_OK;
+}
+
+struct DeviceBlock {  // frees its memory with the scope
+    void *p = nullptr;
+    ~DeviceBlock() {
+        if (p) cudaFree(p);
+    }
+};
+
+template <typename T>
+void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *pot,
+                   cudaStream_t s, double *energies, double *forces, double *virials,
+                   int *status) {
+    const bool lj = pot->kind == CFNEB_LJ;
+    const int precision = sizeof(T) == 4 ? CFNEB_MIXED : CFNEB_FP64;
+    std::vector<BandDev> dv(count);
+    std::vector<BandParams> bp(count);
+    std::vector<Tile> tiles;
+    std::vector<ImgRef> imgs;
+    size_t atoms = 0, big = 0;
+    int max_bins = 0, minb = 0;
+    for (int k = 0; k < count; ++k) {
+        BandDev &d = dv[k];
+        BandParams &P = bp[k];
+        std::memset(&d, 0, sizeof(d));
+        std::memset(&P, 0, sizeof(P));
+        const double rc = fill_potential(pot, P), vol = std::fabs(det3(S[k].cell));
+        const int n = S[k].n_atoms;
+        d.n = P.n = n;
+        d.rows = (n + 3 + 3) / 4 * 4;
+        d.ncap = P.N = 1;
+        const auto key = tune_class(pot, precision, n, vol, rc);
+        const int nb = bins_for(S[k].cell, rc * kTuneScales[0]);
+        d.nbins_cap = (int)std::min<long long>((long long)(1.5 * nb) + 64, 1LL << 26);
+        d.tsum_cap = (d.nbins_cap + 1023) / 1024 + 1;
+        d.tile = atom_tile(pot, precision, n, 1, vol, rc, lj);
+        d.atpi = (n + d.tile - 1) / d.tile;
+        d.rtpi = (d.rows + RTILE - 1) / RTILE;
+        std::memcpy(P.h0, S[k].cell, sizeof(P.h0));
+        inv3(P.h0, P.h0inv);
+        P.c = (double)n;
+        P.rc = P.rl = rc;
+        P.bin_w = rc * tuned_scale(key);
+        P.row_refine = 1;
+        P.ftol = -1.0;
+        P.stale = 1;
+        P.filter = 1;
+        P.variant = CFNEB_ROTFREE_B;
+        P.kind = pot->kind;
+        P.ci = -1;
+        max_bins = std::max(max_bins, d.nbins_cap);
+        if ((size_t)n >= big) {  // the force kernel variant of the largest one
+            big = (size_t)n;
+            minb = tuned_minb(key);
+        }
+        imgs.push_back({k, 0});
+        for (int t = 0; t < d.atpi; ++t) tiles.push_back({k, 0, t, 0});
+        atoms += (size_t)n;
+    }
+    Arena ar;
+    ImgScalars *sc = nullptr;
+    BandDev *d_bands = nullptr;
+    BandParams *d_bp = nullptr;
+    Tile *d_tiles = nullptr;
+    ImgRef *d_imgs = nullptr;
+    double *cart = nullptr, *nep_w = nullptr;
+    ar.add(&sc, count * sizeof(ImgScalars));
+    for (BandDev &d : dv) ar.add(&d.bin_count, d.nbins_cap * sizeof(int));
+    const size_t zeroed = ar.total;
+    ar.add(&d_bands, count * sizeof(BandDev));
+    ar.add(&d_bp, count * sizeof(BandParams));
+    ar.add(&d_tiles, tiles.size() * sizeof(Tile));
+    ar.add(&d_imgs, imgs.size() * sizeof(ImgRef));
+    ar.add(&cart, atoms * 3 * sizeof(double));
+    if (pot->kind == CFNEB_NEP) ar.add(&nep_w, NEP_NW * (sizeof(double) + sizeof(float)));
+    for (BandDev &d : dv) {
+        const size_t na = (size_t)d.n, vec = (size_t)d.rows * 3 * sizeof(T);
+        ar.add(&d.X, vec);
+        ar.add(&d.F, vec);
+        ar.add(&d.bin_start, (d.nbins_cap + 1) * sizeof(int));
+        ar.add(&d.bin_tsum, d.tsum_cap * sizeof(int));
+        for (int **p : {&d.atom_bin, &d.atom_rank, &d.slot_unsorted, &d.slot_atom, &d.slot_bin,
+                        &d.atom_slot})
+            ar.add(p, na * sizeof(int));
+        ar.add(&d.atom_off, na * 4 * sizeof(T));
+        ar.add(&d.slot_off, na * 4 * sizeof(T));
+        ar.add(&d.atom_off_lo, na * sizeof(float4));
+        ar.add(&d.slot_off_lo, na * sizeof(float4));
+        if (!lj) {
+            ar.add(&d.nbr_cnt, na * sizeof(int));
+            ar.add(&d.nbr_slot, na * MAXN_TERSOFF * sizeof(int));
+            ar.add(&d.nbr_code, na * MAXN_TERSOFF * sizeof(int));
+            ar.add(&d.nbr_rev, na * MAXN_TERSOFF);
+            ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * sizeof(T));
+        }
+        ar.add(&d.atom_part, (size_t)d.atpi * NPART * sizeof(double));
+    }
+    DeviceBlock mem;
+    mem.p = device_alloc(ar.total);
+    ar.place(mem.p);
+    CK(cudaMemsetAsync(mem.p, 0, zeroed, s));
+    size_t off = 0;
+    for (int k = 0; k < count; ++k) {
+        dv[k].sc = sc + k;
+        dv[k].bp = d_bp + k;
+        dv[k].cart = cart + 3 * off;
+        CK(cudaMemcpyAsync(dv[k].cart, S[k].positions, (size_t)dv[k].n * 3 * sizeof(double),
+                           cudaMemcpyHostToDevice, s));
+        off += (size_t)dv[k].n;
+    }
+    if (nep_w) {
+        upload_nep(pot, nep_w, dv[0], s);
+        for (BandDev &d : dv) {
+            d.nep_w = dv[0].nep_w;
+            d.nep_wf = dv[0].nep_wf;
+        }
+    }
+    // descriptors and tables: adjacent in the block, one copy
+    std::vector<char> meta((char *)cart - (char *)d_bands);
+    std::memcpy(meta.data(), dv.data(), count * sizeof(BandDev));
+    std::memcpy(meta.data() + ((char *)d_bp - (char *)d_bands), bp.data(),
+                count * sizeof(BandParams));
+    std::memcpy(meta.data() + ((char *)d_tiles - (char *)d_bands), tiles.data(),
+                tiles.size() * sizeof(Tile));
+    std::memcpy(meta.data() + ((char *)d_imgs - (char *)d_bands), imgs.data(),
+                imgs.size() * sizeof(ImgRef));
+    CK(cudaMemcpyAsync(d_bands, meta.data(), meta.size(), cudaMemcpyHostToDevice, s));
+
+    LaunchSet ls;
+    ls.d_bands = d_bands;
+    ls.s = s;
+    ls.imgs = d_imgs;
+    ls.nimg = count;
+    ls.atiles = d_tiles;
+    ls.n_atiles = (int)tiles.size();
+    (lj ? ls.atiles_ljc : pot->kind == CFNEB_NEP ? ls.atiles_nep : ls.atiles_ters) = d_tiles;
+    (lj ? ls.n_ljc : pot->kind == CFNEB_NEP ? ls.n_nep : ls.n_ters) = (int)tiles.size();
+    ls.max_bins = max_bins;
+    ls.force_rebuild = 1;
+    if (minb > 0 && pot->kind == CFNEB_TERSOFF) ls.ters_minb = minb;
+    launch_points_load<T>(d_tiles, ls.n_atiles, d_bands, s);
+    Launcher L;
+    enqueue_eval_set<T>(ls, L);
+    if (sizeof(T) == 4) {
+        if (lj) launch_energy64_lj<T>(d_tiles, ls.n_atiles, d_bands, s);
+        else launch_energy64<T>(d_tiles, ls.n_atiles, d_bands, s);
+        launch_energy_finalize(d_imgs, count, d_bands, s);
+    }
+    if (forces) launch_points_store<T>(d_tiles, ls.n_atiles, d_bands, s);
+    CK(cudaGetLastError());
+    std::vector<ImgScalars> hs(count);
+    CK(cudaMemcpyAsync(hs.data(), sc, count * sizeof(ImgScalars), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(bp.data(), d_bp, count * sizeof(BandParams), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    // results up to the first structure whose kernels raised a status
+    *status = CFNEB_OK;
+    size_t good = 0;
+    for (int k = 0; k < count; ++k) {
+        *status = status_from_bits(bp[k].status);
+        if (*status != CFNEB_OK) break;
+        if (energies) energies[k] = sizeof(T) == 4 ? hs[k].E64 : hs[k].E;
+        if (virials) std::memcpy(virials + 9 * (size_t)k, hs[k].V, 9 * sizeof(double));
+        good += (size_t)dv[k].n;
+    }
+    if (forces && good) {
+        to_host(forces, cart, good * 3 * sizeof(double), s);
+        CK(cudaStreamSynchronize(s));
+    }
+}
+
+int eval_points(const cfneb_structure *S, int count, const cfneb_potential *pot, int precision,
+                cudaStream_t s, double *energies, double *forces, double *virials) {
+    int status = CFNEB_OK;
+    try {
+        if (precision == CFNEB_MIXED)
+            eval_points_t<float>(S, count, pot, s, energies, forces, virials, &status);
+        else
+            eval_points_t<double>(S, count, pot, s, energies, forces, virials, &status);
+    } catch (CudaFail &f) {
+        return f.e == cudaErrorMemoryAllocation ? CFNEB_ERR_OUT_OF_MEMORY : CFNEB_ERR_CUDA;
+    }
+    return status;
+}
+
+cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
+                   const cfneb_potential *pot, const cfneb_cell_filter *cf,
+                   const cfneb_options *opt, void *stream, int *err) {
+    *err = CFNEB_OK;
+    cfneb_band *b = new cfneb_band();
+    b->user = (cudaStream_t)stream;
+    b->n = A->n_atoms;
+    b->N = N;
+    b->opt = *opt;
+    if (b->opt.n_max < N) b->opt.n_max = N;
+    if (b->opt.n_min < 3) b->opt.n_min = 3;
+    b->ncap = b->opt.n_max;
+    b->precision = opt->precision;
+    b->ts = (opt->precision == CFNEB_MIXED) ? 4 : 8;
+    b->kind = pot->kind;
+    b->filt = cf ? *cf : cfneb_cell_filter{1, CFNEB_ROTFREE_B, 0.0, 0.0};
+    std::memcpy(b->h0, A->cell, sizeof(b->h0));
+    // lattice scale: the caller's c, or J = Omega0^(1/3) n^(1/6) (the scale
+    // of the generalized solid-state NEB: it keeps the lattice rows'
+    // stiffness per unit of X independent of n), or n_atoms
+    if (b->filt.cell_factor > 0)
+        b->c = b->filt.cell_factor;
+    else if (b->filt.cell_factor == CFNEB_CELL_FACTOR_J)
+        b->c = std::cbrt(std::fabs(det3(A->cell))) * std::pow((double)b->n, 1.0 / 6.0);
+    else
+        b->c = (double)b->n;
+    CK(cudaStreamCreateWithFlags(&b->s, cudaStreamNonBlocking));
+    CK(cudaStreamCreateWithFlags(&b->s_body, cudaStreamNonBlocking));
+    b->fork.create();
+    CK(cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming));
+    CK(cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming));
+    CK(cudaMallocHost((void **)&b->h_bp, sizeof(BandParams)));
+
+    BandParams &P = *b->h_bp;
+    std::memset(&P, 0, sizeof(P));
+    const double rc = fill_potential(pot, P);
     // neighbour-list skin: the caller's, or 0.15 A for Tersoff (carbon's
     // second neighbours, 2.46-2.52 A, stay outside R + D + skin, so the lists
     // keep their 3-4 entries) and 0.12 rc for LJ (0.3 sigma at rc = 2.5
@@ -945,10 +1256,7 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
         return b;
     }
     // bin width: the caller's, the cached autotuned one for this class, or rc
-    const double dens = (double)b->n / std::fabs(det3(A->cell)) * rc * rc * rc;
-    b->tune_key = std::make_tuple(pot->kind, opt->precision,
-                                  (int)std::floor(std::log2((double)std::max(1, b->n))),
-                                  (int)std::floor(2.0 * std::log2(std::max(dens, 1e-3))));
+    b->tune_key = tune_class(pot, opt->precision, b->n, std::fabs(det3(A->cell)), rc);
     double bscale = opt->bin_scale > 0 ? opt->bin_scale : tuned_scale(b->tune_key);
     b->minb = tuned_minb(b->tune_key);
     double bin_w = rl * bscale;
@@ -970,100 +1278,75 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
     const int row_refine = 1;
     int nb0 = bins_for(A->cell, cap_w) * row_refine, nb1 = bins_for(B->cell, cap_w) * row_refine;
     d.nbins_cap = (int)std::min<long long>((long long)(1.5 * std::max(nb0, nb1)) + 64, 1LL << 26);
-    {
-        const long long atoms = (long long)n * std::max(1, N - 2);
-        const bool cells = pot->kind == CFNEB_LJ && !(skin > 0.0 && n <= LJ_LIST_MAX_ATOMS);
-        int lanes = 1;
-        // FP64 cell walk: at least two lanes (a thread's kept candidates)
-        if (pot->kind == CFNEB_LJ && b->ts == 8)
-            lanes = fp64_lanes(n, std::max(1, N - 2),
-                               lj_fp64_instr(n, std::fabs(det3(A->cell)), rc), cells ? 2 : 1);
-        else if (cells) lanes = lanes_per_atom(atoms, LJ_LANES_FP32);
-        // FP64 many-body kernels take four lanes per atom: one pass per block
-        // (32 atoms) where the band's blocks would leave SMs idle, else four
-        if (pot->kind != CFNEB_LJ && b->ts == 8 && atoms < 152 * 2 * TILE) lanes = 4;
-        d.tile = TILE / lanes;
-    }
+    d.tile = atom_tile(pot, opt->precision, n, std::max(1, N - 2), std::fabs(det3(A->cell)), rc,
+                       pot->kind == CFNEB_LJ && !(skin > 0.0 && n <= LJ_LIST_MAX_ATOMS));
     d.atpi = (n + d.tile - 1) / d.tile;
     d.rtpi = (rows + RTILE - 1) / RTILE;
     const size_t nc = (size_t)b->ncap;
     const size_t vec = nc * rows * 3 * b->ts;
-    d.X = dalloc(b, vec);
-    d.F = dalloc(b, vec);
-    d.Fneb = dalloc(b, vec);
-    d.v = dalloc(b, vec);
-    for (void *p : {d.X, d.F, d.Fneb, d.v}) CK(cudaMemsetAsync(p, 0, vec, b->s));
-    d.sc = (ImgScalars *)dalloc(b, nc * sizeof(ImgScalars));
-    d.bp = (BandParams *)dalloc(b, sizeof(BandParams));
-    d.bin_count = (int *)dalloc(b, nc * d.nbins_cap * sizeof(int));
-    d.bin_start = (int *)dalloc(b, nc * (d.nbins_cap + 1) * sizeof(int));
-    d.tsum_cap = (d.nbins_cap + 1023) / 1024 + 1;
-    d.bin_tsum = (int *)dalloc(b, nc * d.tsum_cap * sizeof(int));
     const size_t na = nc * n;
-    d.atom_bin = (int *)dalloc(b, na * sizeof(int));
-    d.atom_rank = (int *)dalloc(b, na * sizeof(int));
-    d.slot_unsorted = (int *)dalloc(b, na * sizeof(int));
-    d.slot_atom = (int *)dalloc(b, na * sizeof(int));
-    d.slot_bin = (int *)dalloc(b, na * sizeof(int));
-    d.atom_slot = (int *)dalloc(b, na * sizeof(int));
-    d.atom_off = dalloc(b, na * 4 * b->ts);
-    d.slot_off = dalloc(b, na * 4 * b->ts);
-    d.atom_off_lo = (float4 *)dalloc(b, na * sizeof(float4));
-    d.slot_off_lo = (float4 *)dalloc(b, na * sizeof(float4));
-    if (skin > 0.0) {
-        d.ref_X = dalloc(b, vec);  // the row layout of X (padding rows stay zero)
-        d.atom_wrap = (int *)dalloc(b, na * 3 * sizeof(int));
-        d.skin_part = (float *)dalloc(b, nc * d.atpi * sizeof(float));
-    }
+    d.tsum_cap = (d.nbins_cap + 1023) / 1024 + 1;
     d.lj_cap = 0;
-    if (pot->kind == CFNEB_LJ && skin > 0.0 && n <= LJ_LIST_MAX_ATOMS) {
+    const bool lj_list = pot->kind == CFNEB_LJ && skin > 0.0 && n <= LJ_LIST_MAX_ATOMS;
+    const bool many = pot->kind == CFNEB_TERSOFF || pot->kind == CFNEB_NEP;
+    if (lj_list) {
         // list capacity: 1.5 x the entries within rl at the denser endpoint's
         // mean density, plus 32 (the path never gets much denser than its
         // ends; an overflow is reported as CFNEB_ERR_NBR_OVERFLOW)
         const double vmin = std::min(std::fabs(det3(A->cell)), std::fabs(det3(B->cell)));
         const double expect = n / vmin * 4.0 / 3.0 * 3.14159265358979323846 * rl * rl * rl;
         d.lj_cap = (int)std::min<double>(std::ceil((1.5 * expect + 32.0) / 8.0) * 8.0, 4096.0);
-        d.nbr_cnt = (int *)dalloc(b, na * sizeof(int));
-        d.nbr_slot = (int *)dalloc(b, na * d.lj_cap * sizeof(int));
-        CK(cudaMemsetAsync(d.nbr_cnt, 0, na * sizeof(int), b->s));
     }
-    if (pot->kind == CFNEB_NEP) {
-        double *w = (double *)dalloc(b, NEP_NW * (sizeof(double) + sizeof(float)));
-        float *wf = (float *)(w + NEP_NW);
-        float hf[NEP_NW];
-        for (int k = 0; k < NEP_NW; ++k) hf[k] = (float)pot->nep_weights[k];
-        CK(cudaMemcpyAsync(w, pot->nep_weights, NEP_NW * sizeof(double), cudaMemcpyHostToDevice, b->s));
-        CK(cudaMemcpyAsync(wf, hf, NEP_NW * sizeof(float), cudaMemcpyHostToDevice, b->s));
-        CK(cudaStreamSynchronize(b->s));  // hf is a stack array
-        d.nep_w = w;
-        d.nep_wf = wf;
+    Arena ar;
+    // arrays that start at zero first: one clear
+    ar.add(&d.X, vec);
+    ar.add(&d.F, vec);
+    ar.add(&d.Fneb, vec);
+    ar.add(&d.v, vec);
+    if (skin > 0.0) ar.add(&d.ref_X, vec);  // the row layout of X (padding rows stay zero)
+    ar.add(&d.sc, nc * sizeof(ImgScalars));
+    ar.add(&d.bin_count, nc * d.nbins_cap * sizeof(int));
+    if (lj_list) ar.add(&d.nbr_cnt, na * sizeof(int));
+    ar.add(&b->d_band_ids, sizeof(int));
+    const size_t zeroed = ar.total;
+    ar.add(&d.bp, sizeof(BandParams));
+    ar.add(&d.bin_start, nc * (d.nbins_cap + 1) * sizeof(int));
+    ar.add(&d.bin_tsum, nc * d.tsum_cap * sizeof(int));
+    for (int **p : {&d.atom_bin, &d.atom_rank, &d.slot_unsorted, &d.slot_atom, &d.slot_bin,
+                    &d.atom_slot})
+        ar.add(p, na * sizeof(int));
+    ar.add(&d.atom_off, na * 4 * b->ts);
+    ar.add(&d.slot_off, na * 4 * b->ts);
+    ar.add(&d.atom_off_lo, na * sizeof(float4));
+    ar.add(&d.slot_off_lo, na * sizeof(float4));
+    if (skin > 0.0) {
+        ar.add(&d.atom_wrap, na * 3 * sizeof(int));
+        ar.add(&d.skin_part, nc * d.atpi * sizeof(float));
     }
-    if (pot->kind == CFNEB_TERSOFF || pot->kind == CFNEB_NEP) {
-        d.nbr_cnt = (int *)dalloc(b, na * sizeof(int));
-        d.nbr_slot = (int *)dalloc(b, na * MAXN_TERSOFF * sizeof(int));
-        d.nbr_code = (int *)dalloc(b, na * MAXN_TERSOFF * sizeof(int));
-        d.nbr_rev = (unsigned char *)dalloc(b, na * MAXN_TERSOFF);
-        d.nbr_P = dalloc(b, na * 4 * MAXN_TERSOFF * b->ts);
+    if (lj_list) ar.add(&d.nbr_slot, na * d.lj_cap * sizeof(int));
+    double *nep_w = nullptr;
+    if (pot->kind == CFNEB_NEP) ar.add(&nep_w, NEP_NW * (sizeof(double) + sizeof(float)));
+    if (many) {
+        ar.add(&d.nbr_cnt, na * sizeof(int));
+        ar.add(&d.nbr_slot, na * MAXN_TERSOFF * sizeof(int));
+        ar.add(&d.nbr_code, na * MAXN_TERSOFF * sizeof(int));
+        ar.add(&d.nbr_rev, na * MAXN_TERSOFF);
+        ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * b->ts);
     }
-    d.atom_part = (double *)dalloc(b, nc * d.atpi * NPART * sizeof(double));
-    d.row_part = (double *)dalloc(b, nc * d.rtpi * NPART * sizeof(double));
-    d.cart = (double *)dalloc(b, na * 3 * sizeof(double));
-    b->d_self = (BandDev *)dalloc(b, sizeof(BandDev));
-    b->d_atiles = (Tile *)dalloc(b, nc * d.atpi * sizeof(Tile));
-    b->d_rtiles = (Tile *)dalloc(b, nc * d.rtpi * sizeof(Tile));
-    b->d_imgs = (ImgRef *)dalloc(b, nc * sizeof(ImgRef));
-    b->d_band_ids = (int *)dalloc(b, sizeof(int));
-    b->d_scratch_tiles =
-        (Tile *)dalloc(b, nc * std::max(d.atpi, d.rtpi) * sizeof(Tile));
-    b->d_scratch_imgs = (ImgRef *)dalloc(b, nc * sizeof(ImgRef));
-    CK(cudaMemsetAsync(d.bin_count, 0, nc * d.nbins_cap * sizeof(int), b->s));
-    CK(cudaMemsetAsync(d.v, 0, vec, b->s));
-    if (d.ref_X) CK(cudaMemsetAsync(d.ref_X, 0, vec, b->s));
-    CK(cudaMemsetAsync(d.Fneb, 0, vec, b->s));
-    CK(cudaMemsetAsync(d.F, 0, vec, b->s));
-    CK(cudaMemsetAsync(d.sc, 0, nc * sizeof(ImgScalars), b->s));
-    int zero = 0;
-    CK(cudaMemcpyAsync(b->d_band_ids, &zero, sizeof(int), cudaMemcpyHostToDevice, b->s));
+    ar.add(&d.atom_part, nc * d.atpi * NPART * sizeof(double));
+    ar.add(&d.row_part, nc * d.rtpi * NPART * sizeof(double));
+    ar.add(&d.cart, nc * (n + 3) * 3 * sizeof(double));
+    ar.add(&b->d_self, sizeof(BandDev));
+    ar.add(&b->d_atiles, nc * d.atpi * sizeof(Tile));
+    ar.add(&b->d_rtiles, nc * d.rtpi * sizeof(Tile));
+    ar.add(&b->d_imgs, nc * sizeof(ImgRef));
+    ar.add(&b->d_scratch_tiles, nc * std::max(d.atpi, d.rtpi) * sizeof(Tile));
+    ar.add(&b->d_scratch_imgs, nc * sizeof(ImgRef));
+    b->slab = device_alloc(ar.total);
+    b->bytes = ar.bytes;
+    ar.place(b->slab);
+    CK(cudaMemsetAsync(b->slab, 0, zeroed, b->s));
+    if (nep_w) upload_nep(pot, nep_w, d, b->s);
     CK(cudaMemcpyAsync(b->d_self, &d, sizeof(BandDev), cudaMemcpyHostToDevice, b->s));
 
     // band parameters
@@ -1097,30 +1380,24 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
     CK(cudaMemcpyAsync(d.bp, &P, sizeof(BandParams), cudaMemcpyHostToDevice, b->s));
 
     // endpoints and interpolation on the device
-    double *dR = nullptr;
-    size_t rbytes = (size_t)n * 3 * sizeof(double);
-    size_t nbytes = opt->interior_noise ? (size_t)(N - 2) * n * 3 * sizeof(double) : 0;
-    CK(cudaMalloc(&dR, 2 * rbytes + nbytes + 9 * sizeof(double)));
-    double *dR1 = dR + (size_t)n * 3;
-    double *dnoise = opt->interior_noise ? dR1 + (size_t)n * 3 : nullptr;
-    double *dh1 = dR1 + (size_t)n * 3 + (opt->interior_noise ? (size_t)(N - 2) * n * 3 : 0);
-    try {
-        CK(cudaMemcpyAsync(dR, A->positions, rbytes, cudaMemcpyHostToDevice, b->s));
-        CK(cudaMemcpyAsync(dR1, B->positions, rbytes, cudaMemcpyHostToDevice, b->s));
-        if (dnoise)
-            CK(cudaMemcpyAsync(dnoise, opt->interior_noise, nbytes, cudaMemcpyHostToDevice, b->s));
-        CK(cudaMemcpyAsync(dh1, B->cell, 9 * sizeof(double), cudaMemcpyHostToDevice, b->s));
-        if (b->precision == CFNEB_MIXED)
-            launch_setup<float>(dR, dR1, dnoise, n, N, b->d_self, b->s, dh1);
-        else
-            launch_setup<double>(dR, dR1, dnoise, n, N, b->d_self, b->s, dh1);
-        CK(cudaGetLastError());
-        CK(cudaStreamSynchronize(b->s));
-    } catch (...) {
-        cudaFree(dR);
-        throw;
+    // (the scratch array holds the two endpoints and the interior images'
+    // displacements: N x n rows)
+    const size_t rbytes = (size_t)n * 3 * sizeof(double);
+    double *dR1 = d.cart + (size_t)n * 3, *dnoise = nullptr;
+    CK(cudaMemcpyAsync(d.cart, A->positions, rbytes, cudaMemcpyHostToDevice, b->s));
+    CK(cudaMemcpyAsync(dR1, B->positions, rbytes, cudaMemcpyHostToDevice, b->s));
+    if (opt->interior_noise) {
+        dnoise = dR1 + (size_t)n * 3;
+        CK(cudaMemcpyAsync(dnoise, opt->interior_noise, (N - 2) * rbytes, cudaMemcpyHostToDevice,
+                           b->s));
     }
-    CK(cudaFree(dR));
+    Mat3 h1;
+    std::memcpy(h1.m, B->cell, sizeof(h1.m));
+    if (b->precision == CFNEB_MIXED)
+        launch_setup<float>(d.cart, dR1, dnoise, n, N, b->d_self, b->s, h1);
+    else
+        launch_setup<double>(d.cart, dR1, dnoise, n, N, b->d_self, b->s, h1);
+    CK(cudaGetLastError());
     build_tables(b);
     eval_images(b, {0, N - 1});
     read_params(b);
@@ -1629,13 +1906,10 @@ int cfneb_default_options(cfneb_options *o) {
     return CFNEB_OK;
 }
 
-namespace {
-// cfneb_create_band with the argument checks; need_path: refuse coincident
-// endpoints (single-point evaluations build a band of one structure)
-int create_band_checked(const cfneb_structure *initial, const cfneb_structure *final_,
-                        int32_t n_images, const cfneb_potential *potential,
-                        const cfneb_cell_filter *cell_filter, const cfneb_options *options,
-                        void *cuda_stream, cfneb_band **out, bool need_path) {
+int cfneb_create_band(const cfneb_structure *initial, const cfneb_structure *final_,
+                      int32_t n_images, const cfneb_potential *potential,
+                      const cfneb_cell_filter *cell_filter, const cfneb_options *options,
+                      void *cuda_stream, cfneb_band **out) {
     if (!initial || !final_ || !potential || !out || n_images < 3) return CFNEB_ERR_INVALID_ARG;
     *out = nullptr;
     if (!initial->positions || !final_->positions || initial->n_atoms <= 0)
@@ -1648,19 +1922,9 @@ int create_band_checked(const cfneb_structure *initial, const cfneb_structure *f
     if (initial->types)
         for (int i = 1; i < initial->n_atoms; ++i)
             if (initial->types[i] != initial->types[0]) return CFNEB_ERR_INVALID_ARG;
-    if (potential->kind != CFNEB_LJ && potential->kind != CFNEB_TERSOFF &&
-        potential->kind != CFNEB_NEP)
-        return CFNEB_ERR_INVALID_ARG;
-    if (potential->kind == CFNEB_NEP) {
-        if (!potential->nep_weights || !(potential->nep_rc > 0.0) ||
-            !std::isfinite(potential->nep_rc))
-            return CFNEB_ERR_INVALID_ARG;
-        for (int k = 0; k < NEP_NW; ++k)
-            if (!std::isfinite(potential->nep_weights[k])) return CFNEB_ERR_INVALID_ARG;
-    }
-    if (potential->kind == CFNEB_LJ &&
-        (potential->rc <= 0 || potential->sigma <= 0 || potential->eps <= 0))
-        return CFNEB_ERR_INVALID_ARG;
+    double rcut = 0.0;
+    const int pst = check_potential(potential, &rcut);
+    if (pst != CFNEB_OK) return pst;
     if (!(std::fabs(det3(initial->cell)) > 0) || !(std::fabs(det3(final_->cell)) > 0))
         return CFNEB_ERR_INVALID_ARG;
     // finite coordinates and cells only (a non-finite coordinate would reach
@@ -1668,13 +1932,12 @@ int create_band_checked(const cfneb_structure *initial, const cfneb_structure *f
     for (const cfneb_structure *S : {initial, final_}) {
         for (int k = 0; k < 9; ++k)
             if (!std::isfinite(S->cell[k])) return CFNEB_ERR_INVALID_ARG;
-        for (long long k = 0; k < 3LL * S->n_atoms; ++k)
-            if (!std::isfinite(S->positions[k])) return CFNEB_ERR_INVALID_ARG;
+        if (!all_finite(S->positions, 3 * (size_t)S->n_atoms)) return CFNEB_ERR_INVALID_ARG;
     }
     // coincident endpoints (every atom on the same periodic site, the same
     // cell where the filter is on) leave no path: every tangent of the
     // band would vanish (Sec. II.A's projection is undefined)
-    if (need_path) {
+    {
         const bool filter = cell_filter && cell_filter->enabled;
         bool same_cell = true;
         for (int k = 0; k < 9 && filter; ++k)
@@ -1706,17 +1969,8 @@ int create_band_checked(const cfneb_structure *initial, const cfneb_structure *f
     if (opt.dt <= 0 || opt.maxstep <= 0) return CFNEB_ERR_INVALID_ARG;
     if (opt.k_ref <= 0) opt.k_ref = 10;
     if (opt.bin_scale != 0 && opt.bin_scale < 0.25) return CFNEB_ERR_INVALID_ARG;
-    {
-        // a skin (< 0: the default) of at most the potential's cutoff
-        double rcut = potential->kind == CFNEB_NEP ? potential->nep_rc : potential->rc;
-        if (potential->kind == CFNEB_TERSOFF) {
-            const bool dflt = std::all_of(potential->tersoff, potential->tersoff + 11,
-                                          [](double v) { return v == 0.0; });
-            rcut = dflt ? kTersoff1988C[9] + kTersoff1988C[10]
-                        : potential->tersoff[9] + potential->tersoff[10];
-        }
-        if (!(opt.skin < 0.0 || opt.skin <= rcut)) return CFNEB_ERR_INVALID_ARG;
-    }
+    // a skin (< 0: the default) of at most the potential's cutoff
+    if (!(opt.skin < 0.0 || opt.skin <= rcut)) return CFNEB_ERR_INVALID_ARG;
     if (cell_filter && cell_filter->variant != CFNEB_ROTFREE_B &&
         cell_filter->variant != CFNEB_DEFGRAD_D)
         return CFNEB_ERR_INVALID_ARG;
@@ -1735,16 +1989,6 @@ int create_band_checked(const cfneb_structure *initial, const cfneb_structure *f
     }
     *out = b;
     return CFNEB_OK;
-}
-
-}  // namespace
-
-int cfneb_create_band(const cfneb_structure *initial, const cfneb_structure *final_,
-                      int32_t n_images, const cfneb_potential *potential,
-                      const cfneb_cell_filter *cell_filter, const cfneb_options *options,
-                      void *cuda_stream, cfneb_band **out) {
-    return create_band_checked(initial, final_, n_images, potential, cell_filter, options,
-                               cuda_stream, out, true);
 }
 
 int cfneb_step(cfneb_band *b, int32_t n_steps) {
@@ -1822,23 +2066,26 @@ int cfneb_get_path(const cfneb_band *cb, int32_t *n_images, double *positions, d
             // FP64 energies of the current images (map-back, cell list, energy),
             // then Cartesian positions R = R~ D from the same map-back; the
             // endpoints never move, so theirs are computed once
-            std::vector<int> imgs;
-            if (!b->ends_e64) imgs = {0, b->N - 1};
-            for (int i = 1; i < b->N - 1; ++i) imgs.push_back(i);
-            refine_energies(b, imgs);
+            if (!b->ends_e64) refine_ends(b);
             b->ends_e64 = true;
-            if (b->precision == CFNEB_MIXED)
-                launch_cartesian<float>(b->d_scratch_imgs, b->N, b->n, b->d_self, b->s);
-            else
-                launch_cartesian<double>(b->d_scratch_imgs, b->N, b->n, b->d_self, b->s);
+            refine_interior(b);
+            if (positions) {
+                if (b->precision == CFNEB_MIXED)
+                    launch_cartesian<float>(b->N, b->n, b->d_self, b->s);
+                else
+                    launch_cartesian<double>(b->N, b->n, b->d_self, b->s);
+            }
             CK(cudaGetLastError());
+        } else if (!fmax) {  // the image count alone
+            read_params(b);
+            leave(b);
+            return status_from_bits(b->h_bp->status);
         }
         std::vector<ImgScalars> sc(b->N);
         CK(cudaMemcpyAsync(sc.data(), b->dv.sc, b->N * sizeof(ImgScalars),
                            cudaMemcpyDeviceToHost, b->s));
         if (positions)
-            CK(cudaMemcpyAsync(positions, b->dv.cart, (size_t)b->N * b->n * 3 * sizeof(double),
-                               cudaMemcpyDeviceToHost, b->s));
+            to_host(positions, b->dv.cart, (size_t)b->N * b->n * 3 * sizeof(double), b->s);
         read_params(b);
         for (int i = 0; i < b->N; ++i) {
             if (cells) std::memcpy(cells + 9 * i, sc[i].h, 9 * sizeof(double));
@@ -1858,27 +2105,14 @@ int cfneb_get_state(const cfneb_band *cb, double *X, double *F, double *Fneb, do
     if (!b) return CFNEB_ERR_INVALID_ARG;
     try {
         enter(b);
-        // per image n + 3 rows out of the padded row stride
-        const size_t per = (size_t)(b->n + 3) * 3, stride = (size_t)b->dv.rows * 3;
-        const size_t cnt = (size_t)b->N * stride;
-        std::vector<char> tmp(cnt * b->ts);
-        auto fetch = [&](void *src, double *dst) {
-            if (!dst) return;
-            CK(cudaMemcpyAsync(tmp.data(), src, cnt * b->ts, cudaMemcpyDeviceToHost, b->s));
-            CK(cudaStreamSynchronize(b->s));
-            for (int im = 0; im < b->N; ++im)
-                for (size_t i = 0; i < per; ++i)
-                    dst[im * per + i] = b->ts == 4 ? ((const float *)tmp.data())[im * stride + i]
-                                                   : ((const double *)tmp.data())[im * stride + i];
-        };
-        fetch(b->dv.X, X);
-        if (X)
-            for (int im = 0; im < b->N; ++im) lattice_rows_public(b, X + im * per, 1.0);
-        fetch(b->dv.F, F);
-        fetch(b->dv.Fneb, Fneb);
-        if (Fneb) {  // endpoints carry no NEB force
-            std::memset(Fneb, 0, per * sizeof(double));
-            std::memset(Fneb + (size_t)(b->N - 1) * per, 0, per * sizeof(double));
+        // converted on the device, then one copy into the caller's array
+        double *dst[3] = {X, F, Fneb};
+        for (int which = 0; which < 3; ++which) {
+            if (!dst[which]) continue;
+            if (b->ts == 4) launch_state_store<float>(b->d_self, which, b->N, b->n, b->c, b->s);
+            else launch_state_store<double>(b->d_self, which, b->N, b->n, b->c, b->s);
+            CK(cudaGetLastError());
+            to_host(dst[which], b->dv.cart, (size_t)b->N * (b->n + 3) * 3 * sizeof(double), b->s);
         }
         std::vector<ImgScalars> sc(b->N);
         CK(cudaMemcpyAsync(sc.data(), b->dv.sc, b->N * sizeof(ImgScalars),
@@ -1902,29 +2136,14 @@ int cfneb_get_state(const cfneb_band *cb, double *X, double *F, double *Fneb, do
 
 int cfneb_set_state(cfneb_band *b, const double *X) {
     if (!b || !X) return CFNEB_ERR_INVALID_ARG;
-    const size_t per = (size_t)(b->n + 3) * 3, stride = (size_t)b->dv.rows * 3;
-    for (size_t i = 0; i < (size_t)b->N * per; ++i)
-        if (!std::isfinite(X[i])) return CFNEB_ERR_INVALID_ARG;
+    const size_t count = (size_t)b->N * (b->n + 3) * 3;
+    if (!all_finite(X, count)) return CFNEB_ERR_INVALID_ARG;
     try {
         enter(b);
-        // n + 3 rows per image into the padded row stride (padding stays 0)
-        const size_t cnt = (size_t)b->N * stride;
-        std::vector<double> pad(cnt, 0.0);
-        for (int im = 0; im < b->N; ++im) {
-            std::memcpy(pad.data() + im * stride, X + im * per, per * sizeof(double));
-            lattice_rows_public(b, pad.data() + im * stride, -1.0);
-        }
-        if (b->ts == 4) {
-            std::vector<float> tmp(cnt);
-            for (size_t i = 0; i < cnt; ++i) tmp[i] = (float)pad[i];
-            CK(cudaMemcpyAsync(b->dv.X, tmp.data(), cnt * sizeof(float), cudaMemcpyHostToDevice,
-                               b->s));
-            CK(cudaStreamSynchronize(b->s));
-        } else {
-            CK(cudaMemcpyAsync(b->dv.X, pad.data(), cnt * sizeof(double), cudaMemcpyHostToDevice,
-                               b->s));
-            CK(cudaStreamSynchronize(b->s));
-        }
+        CK(cudaMemcpyAsync(b->dv.cart, X, count * sizeof(double), cudaMemcpyHostToDevice, b->s));
+        if (b->ts == 4) launch_state_load<float>(b->d_self, b->N, b->n, b->c, b->s);
+        else launch_state_load<double>(b->d_self, b->N, b->n, b->c, b->s);
+        CK(cudaGetLastError());
         fire_reset(b);
         eval_images(b, {0, b->N - 1});  // the endpoints' energies and forces
         b->ends_e64 = false;            // their FP64 energies are re-taken when reported
@@ -2122,44 +2341,37 @@ int cfneb_evaluate(const cfneb_structure *structures, int32_t count,
                    const cfneb_potential *potential, int32_t precision, void *cuda_stream,
                    double *energies, double *forces, double *virials) {
     if (!structures || count <= 0 || !potential) return CFNEB_ERR_INVALID_ARG;
-    size_t off = 0;
-    for (int k = 0; k < count; ++k) {
-        const cfneb_structure &S = structures[k];
-        // each structure is the middle image of a three-image band whose
-        // reference cell is its own cell (D = I, forces are Cartesian)
-        cfneb_options opt;
-        cfneb_default_options(&opt);
-        opt.precision = precision;
-        opt.skin = 0.0;  // one evaluation: nothing to reuse
-        cfneb_cell_filter cf{1, CFNEB_ROTFREE_B, 0.0, 0.0};
-        cfneb_band *b = nullptr;
-        int st = create_band_checked(&S, &S, 3, potential, &cf, &opt, cuda_stream, &b, false);
-        if (st != CFNEB_OK) return st;
-        try {
-            enter(b);
-            // the endpoints were evaluated at creation: image 0 is S; its
-            // reported energy is the FP64 one
-            refine_energies(b, {0});
-            std::vector<ImgScalars> sc(1);
-            CK(cudaMemcpyAsync(sc.data(), b->dv.sc, sizeof(ImgScalars), cudaMemcpyDeviceToHost,
-                               b->s));
-            std::vector<char> tmp((size_t)b->dv.rows * 3 * b->ts);
-            CK(cudaMemcpyAsync(tmp.data(), b->dv.F, tmp.size(), cudaMemcpyDeviceToHost, b->s));
-            CK(cudaStreamSynchronize(b->s));
-            if (energies) energies[k] = sc[0].E64;
-            if (virials) std::memcpy(virials + 9 * k, sc[0].V, 9 * sizeof(double));
-            if (forces) {
-                for (int i = 0; i < S.n_atoms * 3; ++i)
-                    forces[off + i] = b->ts == 4 ? ((const float *)tmp.data())[i]
-                                                 : ((const double *)tmp.data())[i];
-            }
-            leave(b);
-        } catch (CudaFail &) {
-            cfneb_destroy_band(b);
-            return CFNEB_ERR_CUDA;
+    // groups of structures share one allocation and one launch per kernel, as
+    // far as that stays small next to the device's memory; a structure that
+    // is refused ends the call after those before it
+    size_t atoms = 0;  // of the structures done
+    int k = 0;
+    while (k < count) {
+        int e = k, st = CFNEB_OK;
+        long long n = 0;
+        while (e < count && (st = check_point(structures[e], potential, precision)) == CFNEB_OK) {
+            if (e > k && n + structures[e].n_atoms > POINT_GROUP_ATOMS) break;
+            n += structures[e++].n_atoms;
         }
-        off += (size_t)S.n_atoms * 3;
-        cfneb_destroy_band(b);
+        const int refused = st;
+        int done = 0;
+        if (e > k) {
+            double *E = energies ? energies + k : nullptr;
+            double *F = forces ? forces + 3 * atoms : nullptr;
+            double *V = virials ? virials + 9 * (size_t)k : nullptr;
+            st = eval_points(structures + k, e - k, potential, precision,
+                             (cudaStream_t)cuda_stream, E, F, V);
+            if (st == CFNEB_ERR_OUT_OF_MEMORY && e - k > 1) {  // one at a time
+                e = k + 1;
+                st = eval_points(structures + k, 1, potential, precision,
+                                 (cudaStream_t)cuda_stream, E, F, V);
+                done = 1;
+            }
+            if (st != CFNEB_OK) return st;
+        }
+        for (int i = k; i < e; ++i) atoms += (size_t)structures[i].n_atoms;
+        k = e;
+        if (!done && refused != CFNEB_OK) return refused;
     }
     return CFNEB_OK;
 }
@@ -2184,8 +2396,6 @@ int cfneb_batch_create(int32_t precision, uint64_t budget_bytes, void *cuda_stre
         bt->fork.create();
         CK(cudaEventCreateWithFlags(&bt->ev_in, cudaEventDisableTiming));
         CK(cudaEventCreateWithFlags(&bt->ev_out, cudaEventDisableTiming));
-        bt->prof_ev.resize(2 * 64);
-        for (auto &e : bt->prof_ev) CK(cudaEventCreate(&e));
     } catch (CudaFail &) {
         batch_free(bt);
         return CFNEB_ERR_CUDA;

@@ -5,7 +5,7 @@
 // start-up) leave nothing for a library to take, and long-running services
 // must not allocate once they are serving (an allocation can fail or stall
 // at any time).  This entry point runs the library's existing FP64
-// evaluation kernels (set-up, map-back, cell list, LJ forces, per-image
+// evaluation kernels (load, map-back, cell list, LJ forces, per-image
 // finalize) on scratch memory that lives in one file-scope __device__
 // array, and copies the results into the caller's device buffers.  The
 // caller passes inputs and outputs; nothing is allocated or freed, here or
@@ -31,7 +31,7 @@ namespace {
 
 constexpr int NA_MAX_ATOMS = CFNEB_NOALLOC_MAX_ATOMS;
 constexpr int NA_MAX_BINS = 32768;
-constexpr int NA_IMAGES = 2;   // the set-up kernel writes two identical images
+constexpr int NA_IMAGES = 1;
 constexpr int NA_ROWS = NA_MAX_ATOMS + 3;
 // tiles of 128 / lanes atoms, most at 32 lanes (4 atoms)
 constexpr int NA_TILES = NA_MAX_ATOMS / 4;
@@ -44,8 +44,7 @@ constexpr size_t al(size_t x) { return (x + 255) / 256 * 256; }
 constexpr size_t O_BAND = 0;
 constexpr size_t O_PARAMS = O_BAND + al(sizeof(BandDev));
 constexpr size_t O_SC = O_PARAMS + al(sizeof(BandParams));
-constexpr size_t O_H1 = O_SC + al(NA_IMAGES * sizeof(ImgScalars));
-constexpr size_t O_TILES = O_H1 + al(9 * sizeof(double));
+constexpr size_t O_TILES = O_SC + al(NA_IMAGES * sizeof(ImgScalars));
 constexpr size_t O_IMG = O_TILES + al(NA_TILES * sizeof(Tile));
 constexpr size_t O_X = O_IMG + al(sizeof(ImgRef));
 constexpr size_t O_F = O_X + al((size_t)NA_IMAGES * NA_ROWS * 3 * sizeof(double));
@@ -63,20 +62,14 @@ constexpr size_t SCRATCH_BYTES = O_PART + al((size_t)NA_TILES * NPART * sizeof(d
 // ~8.3 MB for 32,768 atoms
 __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
 
-struct H1 {
-    double h[9];
-};
-
 // Writes the launch descriptors into the scratch array (arguments arrive by
 // value, so no host-to-device copy is needed) and clears the bin counts.
-__global__ void k_noalloc_init(BandDev dv, BandParams bp, H1 cell, int ntiles) {
+__global__ void k_noalloc_init(BandDev dv, BandParams bp, int ntiles) {
     unsigned char *base = g_noalloc_scratch;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     if (tid == 0) {
         *(BandDev *)(base + O_BAND) = dv;
         *(BandParams *)(base + O_PARAMS) = bp;
-        double *h1 = (double *)(base + O_H1);
-        for (int k = 0; k < 9; ++k) h1[k] = cell.h[k];
         ImgRef r;
         r.band = 0;
         r.img = 0;
@@ -199,6 +192,7 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     dv.atom_off_lo = (float4 *)(base + O_OFFS + 2 * OFF_ARR);
     dv.slot_off_lo = (float4 *)(base + O_OFFS + 2 * OFF_ARR + OFFL_ARR);
     dv.atom_part = (double *)(base + O_PART);
+    dv.cart = const_cast<double *>(d_positions);  // read by the load kernel only
 
     BandParams bp;
     memset(&bp, 0, sizeof(bp));
@@ -220,15 +214,12 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     LJParams lp{eps, sigma, rc, shift_energy ? 4.0 * eps * (sr6 * sr6 - sr6) : 0.0};
     lp.derive();
     memcpy(bp.pot, &lp, sizeof(lp));
-    H1 h1;
-    for (int k = 0; k < 9; ++k) h1.h[k] = cell[k];
 
     BandDev *d_band = (BandDev *)(base + O_BAND);
     const Tile *d_tiles = (const Tile *)(base + O_TILES);
     const ImgRef *d_img = (const ImgRef *)(base + O_IMG);
-    const double *d_h1 = (const double *)(base + O_H1);
-    k_noalloc_init<<<32, 256, 0, s>>>(dv, bp, h1, dv.atpi);
-    launch_setup<double>(d_positions, d_positions, nullptr, n, NA_IMAGES, d_band, s, d_h1);
+    k_noalloc_init<<<32, 256, 0, s>>>(dv, bp, dv.atpi);
+    launch_points_load<double>(d_tiles, dv.atpi, d_band, s);
     launch_mapback<double>(d_img, 1, d_band, 1, s);  // forced: the scratch record is reused
     launch_bin_assign<double>(d_tiles, dv.atpi, d_band, s);
     launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 0);
