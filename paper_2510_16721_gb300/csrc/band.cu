@@ -265,10 +265,10 @@ __device__ inline void image_coef(BandDev &b, int i, int ci, const double *d, do
 // tile into the tile's partial record; with FUSE, the last tile of an image
 // sums the image's records (fixed order) into its dots, and the last image
 // of a band computes the band's NEB coefficients and FIRE sums.
-// Each thread of a row tile owns 4 consecutive rows: 12 values, loaded and
-// stored with 16-byte vector accesses (the row stride of an image is a
-// multiple of 4 rows, so every thread's first value is 16-byte aligned).
-__device__ inline void ld12(const float *p, float (&v)[12]) {
+// The values of a thread's rows: FP32 12 values with 16-byte vector accesses
+// (the row stride of an image is a multiple of 4 rows, so every thread's first
+// value is 16-byte aligned), FP64 one row.
+__device__ inline void ld_rows(const float *p, float (&v)[12]) {
     const float4 *q = reinterpret_cast<const float4 *>(p);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -276,23 +276,18 @@ __device__ inline void ld12(const float *p, float (&v)[12]) {
         v[4 * k] = a.x; v[4 * k + 1] = a.y; v[4 * k + 2] = a.z; v[4 * k + 3] = a.w;
     }
 }
-__device__ inline void ld12(const double *p, double (&v)[12]) {
-    const double2 *q = reinterpret_cast<const double2 *>(p);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const double2 a = q[k];
-        v[2 * k] = a.x; v[2 * k + 1] = a.y;
-    }
-}
-__device__ inline void st12(float *p, const float (&v)[12]) {
+__device__ inline void st_rows(float *p, const float (&v)[12]) {
     float4 *q = reinterpret_cast<float4 *>(p);
 #pragma unroll
     for (int k = 0; k < 3; ++k) q[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
 }
-__device__ inline void st12(double *p, const double (&v)[12]) {
-    double2 *q = reinterpret_cast<double2 *>(p);
+__device__ inline void ld_rows(const double *p, double (&v)[3]) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) q[k] = make_double2(v[2 * k], v[2 * k + 1]);
+    for (int k = 0; k < 3; ++k) v[k] = p[k];
+}
+__device__ inline void st_rows(double *p, const double (&v)[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) p[k] = v[k];
 }
 
 template <typename T, bool FUSE>
@@ -300,16 +295,17 @@ __global__ void __launch_bounds__(RTHREADS, sizeof(T) == 4 ? 4 : 2) k_band_dots(
     Tile tl = tiles[blockIdx.x];
     BandDev &b = bands[tl.band];
     Acc<T> acc[10];
+    constexpr int RPT = rows_per_thread(sizeof(T));
     const size_t stride = (size_t)b.rows * 3;
-    const int r0 = tl.t * RTILE + RPT * (int)threadIdx.x;  // first of this thread's rows
+    const int r0 = tl.t * row_tile(sizeof(T)) + RPT * (int)threadIdx.x;  // first of this thread's rows
     if (r0 < b.rows) {
         const size_t o0 = tl.img * stride + (size_t)r0 * 3;
-        T a[12], xp[12], xm[12], f[12], v[12];
-        ld12((const T *)b.X + o0, a);
-        ld12((const T *)b.X + o0 + stride, xp);
-        ld12((const T *)b.X + o0 - stride, xm);
-        ld12((const T *)b.F + o0, f);
-        ld12((const T *)b.v + o0, v);
+        T a[3 * RPT], xp[3 * RPT], xm[3 * RPT], f[3 * RPT], v[3 * RPT];
+        ld_rows((const T *)b.X + o0, a);
+        ld_rows((const T *)b.X + o0 + stride, xp);
+        ld_rows((const T *)b.X + o0 - stride, xm);
+        ld_rows((const T *)b.F + o0, f);
+        ld_rows((const T *)b.v + o0, v);
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
             T r[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -434,6 +430,10 @@ __device__ inline void atomic_max_nonneg(unsigned long long *bits, double v) {
     atomicMax(bits, (unsigned long long)__double_as_longlong(v));
 }
 
+template <typename T> struct UIntOf;
+template <> struct UIntOf<float> { using type = unsigned int; };
+template <> struct UIntOf<double> { using type = unsigned long long; };
+
 // Pass 2: f_NEB rows (written for the state read-back and the move) and the
 // largest row norm; the last tile of the band runs the convergence test and
 // the FIRE decision on the sums of pass 1.
@@ -446,19 +446,20 @@ __global__ void __launch_bounds__(RTHREADS, 4) k_neb_force(const Tile *tiles, Ba
     if (threadIdx.x < 2) s_coef[threadIdx.x] = (T)b.sc[tl.img].coef[threadIdx.x];
     __syncthreads();
     const T ca = s_coef[0], cb = s_coef[1];
+    constexpr int RPT = rows_per_thread(sizeof(T));
     const size_t stride = (size_t)b.rows * 3;
-    const int r0 = tl.t * RTILE + RPT * (int)threadIdx.x;
+    const int r0 = tl.t * row_tile(sizeof(T)) + RPT * (int)threadIdx.x;
     T mx = 0;
     if (r0 < b.rows) {
         const size_t o0 = tl.img * stride + (size_t)r0 * 3;
-        T a[12], xp[12], xm[12], gv[12];
-        ld12((const T *)b.X + o0, a);
-        ld12((const T *)b.X + o0 + stride, xp);
-        ld12((const T *)b.X + o0 - stride, xm);
-        ld12((const T *)b.F + o0, gv);
+        T a[3 * RPT], xp[3 * RPT], xm[3 * RPT], gv[3 * RPT];
+        ld_rows((const T *)b.X + o0, a);
+        ld_rows((const T *)b.X + o0 + stride, xp);
+        ld_rows((const T *)b.X + o0 - stride, xm);
+        ld_rows((const T *)b.F + o0, gv);
 #pragma unroll
-        for (int c = 0; c < 12; ++c) gv[c] = gv[c] + ca * (xp[c] - a[c]) + cb * (a[c] - xm[c]);
-        st12((T *)b.Fneb + o0, gv);
+        for (int c = 0; c < 3 * RPT; ++c) gv[c] = gv[c] + ca * (xp[c] - a[c]) + cb * (a[c] - xm[c]);
+        st_rows((T *)b.Fneb + o0, gv);
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
             const T ff = fma(gv[3 * q + 2], gv[3 * q + 2],
@@ -466,16 +467,19 @@ __global__ void __launch_bounds__(RTHREADS, 4) k_neb_force(const Tile *tiles, Ba
             mx = fmax(mx, ff);
         }
     }
-    // block max of the row norms (a max is exact in any precision)
-    __shared__ T smax[RTHREADS / 32];
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) smax[threadIdx.x >> 5] = mx;
+    // block max of the row norms, by the bits of the non-negative values (FP64
+    // comparisons would queue in the FP64 pipe)
+    using Bits = typename UIntOf<T>::type;
+    __shared__ Bits smax[RTHREADS / 32];
+    Bits mb = __builtin_bit_cast(Bits, mx);
+    for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+    if ((threadIdx.x & 31) == 0) smax[threadIdx.x >> 5] = mb;
     __syncthreads();
     BandParams *bp = b.bp;
     if (threadIdx.x == 0) {
-        T m = (T)0;
-        for (int q = 0; q < RTHREADS / 32; ++q) m = fmax(m, smax[q]);
-        atomic_max_nonneg(&bp->fmax2_bits, (double)m);
+        Bits m = 0;
+        for (int q = 0; q < RTHREADS / 32; ++q) m = max(m, smax[q]);
+        atomic_max_nonneg(&bp->fmax2_bits, (double)__builtin_bit_cast(T, m));
     }
     if (!last_arrival(&bp->done_b, (unsigned)((bp->N - 2) * b.rtpi))) return;
     // the band's FIRE sums over the interior images, in image order (the
@@ -595,7 +599,7 @@ __device__ inline void lattice_move_warp(const ImgRef r, BandDev *bands) {
     }
 }
 
-// Pass 3 on one row tile: the atom rows move, 4 rows a thread (lattice
+// Pass 3 on one row tile: the atom rows move, a thread its rows (lattice
 // rows: lattice_move_warp; padding rows stay zero), and with a skin the
 // tile records its largest displacement since the last list build.
 template <typename T>
@@ -618,7 +622,8 @@ __device__ inline void move_tile(const Tile tl, BandDev *bands) {
         return;
     }
     const T cv = s_k[0], cf = s_k[1], dt = s_k[2], ms = s_k[3];
-    const int r0 = tl.t * RTILE + RPT * (int)threadIdx.x;
+    constexpr int RPT = rows_per_thread(sizeof(T));
+    const int r0 = tl.t * row_tile(sizeof(T)) + RPT * (int)threadIdx.x;
     const int n = b.n;
     T d2 = 0;  // largest squared displacement of this thread's atom rows since the build
     if (r0 < n) {
@@ -626,17 +631,17 @@ __device__ inline void move_tile(const Tile tl, BandDev *bands) {
         // only atom rows move here (lattice rows: lattice_move_warp;
         // padding rows stay zero)
         const size_t o0 = (tl.img * (size_t)b.rows + (size_t)r0) * 3;
-        T x[12], v[12], fn[12], rf[12];
-        ld12((const T *)b.X + o0, x);
-        ld12((const T *)b.v + o0, v);
-        ld12((const T *)b.Fneb + o0, fn);
-        if (b.ref_X) ld12((const T *)b.ref_X + o0, rf);  // with the others: one round trip
+        T x[3 * RPT], v[3 * RPT], fn[3 * RPT], rf[3 * RPT];
+        ld_rows((const T *)b.X + o0, x);
+        ld_rows((const T *)b.v + o0, v);
+        ld_rows((const T *)b.Fneb + o0, fn);
+        if (b.ref_X) ld_rows((const T *)b.ref_X + o0, rf);  // with the others: one round trip
 #pragma unroll
         for (int q = 0; q < RPT; ++q)
             if (r0 + q < n) fire_row(x + 3 * q, v + 3 * q, fn + 3 * q, cv, cf, dt, ms);
         if (r0 + RPT <= n) {
-            st12((T *)b.v + o0, v);
-            st12((T *)b.X + o0, x);
+            st_rows((T *)b.v + o0, v);
+            st_rows((T *)b.X + o0, x);
         } else {  // the last atom rows of the image: row by row
 #pragma unroll
             for (int q = 0; q < RPT; ++q)
@@ -661,14 +666,15 @@ __device__ inline void move_tile(const Tile tl, BandDev *bands) {
     // the row tile's largest displacement for the next evaluation's list
     // decision (FP32, rounded up: the reuse test never sees one too small)
     if (b.ref_X) {
-        __shared__ T wmax[RTHREADS / 32];
-        for (int o = 16; o > 0; o >>= 1) d2 = fmax(d2, __shfl_xor_sync(0xffffffffu, d2, o));
-        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = d2;
+        __shared__ float wmax[RTHREADS / 32];
+        float df = to_float_ru(d2);
+        for (int o = 16; o > 0; o >>= 1) df = fmaxf(df, __shfl_xor_sync(0xffffffffu, df, o));
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = df;
         __syncthreads();
         if (threadIdx.x == 0) {
-            T m = wmax[0];
-            for (int q = 1; q < RTHREADS / 32; ++q) m = fmax(m, wmax[q]);
-            b.skin_part[(size_t)tl.img * b.atpi + tl.t] = __fsqrt_ru(to_float_ru(m));
+            float m = wmax[0];
+            for (int q = 1; q < RTHREADS / 32; ++q) m = fmaxf(m, wmax[q]);
+            b.skin_part[(size_t)tl.img * b.rtpi + tl.t] = __fsqrt_ru(m);
         }
     }
     __syncthreads();  // the shared scalars are reused by the block's next tile

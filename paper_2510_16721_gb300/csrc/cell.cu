@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(32) k_mapback(const ImgRef *imgs, int count, B
     double dmax = 0.0;
     if (b.skin_part) {
         // per row tile, left by the last move (k_fire_update)
-        const float *part = b.skin_part + (size_t)r.img * b.atpi;
+        const float *part = b.skin_part + (size_t)r.img * b.rtpi;
         float m = 0.0f;
 #pragma unroll 8
         for (int t = lane; t < b.rtpi; t += 32) m = fmaxf(m, part[t]);

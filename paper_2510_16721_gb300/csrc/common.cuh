@@ -11,7 +11,7 @@
 // Kernels are launched over tile tables: each tile is (band, image, t) and
 // covers atoms [t*tile, (t+1)*tile) (atom tiles: one thread per atom, tile =
 // TILE, or several lanes per atom in the force kernels of small bands) or
-// rows [t*RTILE, (t+1)*RTILE) (row tiles of the band-vector kernels, RPT
+// rows [t*rtile, (t+1)*rtile) (row tiles of the band-vector kernels, 4 or 1
 // rows per thread) of that image, so any mix of bands of different sizes
 // runs in one launch.  Partial sums of a tile land in a
 // fixed slot (image, t) of its band, and every reduction sums the slots of a
@@ -27,8 +27,13 @@ namespace cfneb {
 
 constexpr int TILE = 128;           // atoms per atom tile = threads per block
 constexpr int RTHREADS = 256;       // threads per block of the row-tile kernels
-constexpr int RPT = 4;              // consecutive rows per thread of the row-tile kernels
-constexpr int RTILE = RTHREADS * RPT;  // rows per row tile (band vector kernels)
+// Consecutive rows per thread of the row-tile kernels.  FP32: 4 (12 values, moved
+// with 16-byte accesses).  FP64: 1 -- a row costs ~36 FP64 instructions in the
+// dot pass, one per ~64 cycles and warp, and four of them in turn made that
+// chain the pass (31 rows: band_dots 13 us, fire_update 12 us).
+constexpr int rows_per_thread(size_t ts) { return ts == 4 ? 4 : 1; }
+// rows per row tile (band vector kernels)
+constexpr int row_tile(size_t ts) { return RTHREADS * rows_per_thread(ts); }
 constexpr int MAXN_TERSOFF = 16;    // Tersoff list capacity per atom (entries within rl)
 constexpr int NPART = 12;           // doubles per tile partial record
 constexpr int MAX_STENCIL = 7;      // |delta| <= 7 bins per axis
@@ -227,7 +232,7 @@ struct BandDev {
     // neighbour-list reuse: positions and periodic wraps at the last build
     void *ref_X;         // [ncap][rows][3] T: R~ at the build (the layout of X)
     int *atom_wrap;      // [ncap][n][3]: floor(s) at the build
-    float *skin_part;    // [ncap][atpi]: per-row-tile max displacement (rtpi used)
+    float *skin_part;    // [ncap][rtpi]: per-row-tile max displacement
     // per-slot neighbour lists: Tersoff (slot, code) pairs of MAXN_TERSOFF
     // entries, or LJ packed entries of lj_cap (0: the LJ kernel walks the
     // cell list directly)

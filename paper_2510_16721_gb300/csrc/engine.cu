@@ -1058,7 +1058,7 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
         d.tsum_cap = (d.nbins_cap + 1023) / 1024 + 1;
         d.tile = atom_tile(pot, precision, n, 1, vol, rc, lj);
         d.atpi = (n + d.tile - 1) / d.tile;
-        d.rtpi = (d.rows + RTILE - 1) / RTILE;
+        d.rtpi = (d.rows + row_tile(sizeof(T)) - 1) / row_tile(sizeof(T));
         std::memcpy(P.h0, S[k].cell, sizeof(P.h0));
         inv3(P.h0, P.h0inv);
         P.c = (double)n;
@@ -1281,7 +1281,7 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
     d.tile = atom_tile(pot, opt->precision, n, std::max(1, N - 2), std::fabs(det3(A->cell)), rc,
                        pot->kind == CFNEB_LJ && !(skin > 0.0 && n <= LJ_LIST_MAX_ATOMS));
     d.atpi = (n + d.tile - 1) / d.tile;
-    d.rtpi = (rows + RTILE - 1) / RTILE;
+    d.rtpi = (rows + row_tile(b->ts) - 1) / row_tile(b->ts);
     const size_t nc = (size_t)b->ncap;
     const size_t vec = nc * rows * 3 * b->ts;
     const size_t na = nc * n;
@@ -1321,7 +1321,7 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
     ar.add(&d.slot_off_lo, na * sizeof(float4));
     if (skin > 0.0) {
         ar.add(&d.atom_wrap, na * 3 * sizeof(int));
-        ar.add(&d.skin_part, nc * d.atpi * sizeof(float));
+        ar.add(&d.skin_part, nc * d.rtpi * sizeof(float));
     }
     if (lj_list) ar.add(&d.nbr_slot, na * d.lj_cap * sizeof(int));
     double *nep_w = nullptr;

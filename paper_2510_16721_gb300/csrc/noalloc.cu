@@ -170,7 +170,7 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     dv.nbins_cap = NA_MAX_BINS;
     dv.tile = TILE / fp64_lanes(n, 1, lj_fp64_instr(n, std::fabs(det3(cell)), rc), 2);
     dv.atpi = (n + dv.tile - 1) / dv.tile;
-    dv.rtpi = (n + 3 + RTILE - 1) / RTILE;
+    dv.rtpi = (n + 3 + row_tile(8) - 1) / row_tile(8);
     dv.X = base + O_X;
     dv.F = base + O_F;
     dv.Fneb = dv.F;  // not used by an evaluation
