@@ -491,35 +491,35 @@ __global__ void __launch_bounds__(TILE) k_bin_scatter(const Tile *tiles, int nti
     }
 }
 
-// Threads stride over the bins: order each bin's atoms by atom index and
-// write the sorted slot arrays.
+// Order each bin's atoms by atom index and write the sorted slot arrays: one
+// thread per atom, its rank among its bin's atoms counted from the unordered
+// slots.  (One thread per bin left the chip to a few threads with quadratic
+// loops: 19,380 atoms in 972 bins, 54 us.)
 template <typename T>
-__global__ void k_bin_order(const ImgRef *imgs, BandDev *bands) {
+__global__ void __launch_bounds__(TILE) k_bin_order(const Tile *tiles, int ntiles, BandDev *bands) {
     using T4 = typename Vec4<T>::type;
-    ImgRef r = imgs[blockIdx.y];
-    BandDev &b = bands[r.band];
-    if (!b.sc[r.img].rebuild) return;
-    const int nbins = b.sc[r.img].nbins;
-    const int *start = b.bin_start + (size_t)r.img * (b.nbins_cap + 1);
-    const size_t base = (size_t)r.img * b.n;
-    const int *un = b.slot_unsorted + base;
-    const int nb1 = b.sc[r.img].nb[1], nb2 = b.sc[r.img].nb[2];
-    for (int bin = blockIdx.x * blockDim.x + threadIdx.x; bin < nbins;
-         bin += gridDim.x * blockDim.x) {
+    for (int k = blockIdx.x; k < ntiles; k += gridDim.x) {
+        const Tile tl = tiles[k];
+        BandDev &b = bands[tl.band];
+        const ImgScalars &sc = b.sc[tl.img];
+        if (!sc.rebuild) continue;
+        const int i = tile_atom(b, tl);
+        if (i >= b.n) continue;
+        const size_t base = (size_t)tl.img * b.n;
+        const int *start = b.bin_start + (size_t)tl.img * (b.nbins_cap + 1);
+        const int *un = b.slot_unsorted + base;
+        const int nb1 = sc.nb[1], nb2 = sc.nb[2];
+        const int bin = b.atom_bin[base + i];
+        const T4 o = ((const T4 *)b.atom_off)[base + i];
+        const float4 ol = b.atom_off_lo[base + i];
         const int s0 = start[bin], s1 = start[bin + 1];
-        const int b0 = bin / (nb1 * nb2), b1 = (bin / nb2) % nb1;
-        const int pb = pack_bin(b0, b1, bin % nb2);
-        for (int p = s0; p < s1; ++p) {
-            const int idx = un[p];
-            int rk = 0;
-            for (int q = s0; q < s1; ++q) rk += (un[q] < idx);
-            const int dst = s0 + rk;
-            b.slot_atom[base + dst] = idx;
-            b.slot_bin[base + dst] = pb;
-            b.atom_slot[base + idx] = dst;
-            ((T4 *)b.slot_off)[base + dst] = ((const T4 *)b.atom_off)[base + idx];
-            b.slot_off_lo[base + dst] = b.atom_off_lo[base + idx];
-        }
+        int dst = s0;
+        for (int q = s0; q < s1; ++q) dst += un[q] < i;
+        b.slot_atom[base + dst] = i;
+        b.slot_bin[base + dst] = pack_bin(bin / (nb1 * nb2), (bin / nb2) % nb1, bin % nb2);
+        b.atom_slot[base + i] = dst;
+        ((T4 *)b.slot_off)[base + dst] = o;
+        b.slot_off_lo[base + dst] = ol;
     }
 }
 
@@ -564,11 +564,9 @@ void launch_bin_scatter(const Tile *tiles, int ntiles, BandDev *bands, cudaStrea
     k_bin_scatter<<<ntiles < gated_grid() ? ntiles : gated_grid(), TILE, 0, s>>>(tiles, ntiles, bands);
 }
 template <typename T>
-void launch_bin_order(const ImgRef *imgs, int count, int max_bins, BandDev *bands,
-                      cudaStream_t s) {
-    if (count <= 0 || max_bins <= 0) return;
-    dim3 grid(std::min((max_bins + 127) / 128, 128), count);
-    k_bin_order<T><<<grid, 128, 0, s>>>(imgs, bands);
+void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
+    if (ntiles <= 0) return;
+    k_bin_order<T><<<ntiles < gated_grid() ? ntiles : gated_grid(), TILE, 0, s>>>(tiles, ntiles, bands);
 }
 template <typename T>
 void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {
@@ -581,7 +579,7 @@ void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {
     template void launch_mapback<T>(const ImgRef *, int, BandDev *, int, cudaStream_t);  \
     template void launch_bin_assign<T>(const Tile *, int, BandDev *, cudaStream_t,       \
                                        cudaGraphConditionalHandle, int);                 \
-    template void launch_bin_order<T>(const ImgRef *, int, int, BandDev *, cudaStream_t); \
+    template void launch_bin_order<T>(const Tile *, int, BandDev *, cudaStream_t);        \
     template void launch_cartesian<T>(int, int, BandDev *, cudaStream_t);
 CFNEB_INST(float)
 CFNEB_INST(double)

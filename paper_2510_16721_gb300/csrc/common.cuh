@@ -948,8 +948,7 @@ void launch_bin_scan(const ImgRef *imgs, int count, int max_bins, BandDev *bands
                      cudaStream_t s, int part);
 void launch_bin_scatter(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
 template <typename T>
-void launch_bin_order(const ImgRef *imgs, int count, int max_bins, BandDev *bands,
-                      cudaStream_t s);
+void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
 template <typename T>
 void launch_lj(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
 template <typename T>

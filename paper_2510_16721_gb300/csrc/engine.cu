@@ -345,7 +345,7 @@ void enqueue_rebuild(const LaunchSet &ls, Launcher &L) {
     L.pre(K_BIN_TILESCAN); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 1); L.post(K_BIN_TILESCAN);
     L.pre(K_BIN_SCANFILL); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 2); L.post(K_BIN_SCANFILL);
     L.pre(K_BIN_SCATTER); launch_bin_scatter(ls.atiles, ls.n_atiles, d, s); L.post(K_BIN_SCATTER);
-    L.pre(K_BIN_ORDER); launch_bin_order<T>(ls.imgs, ls.nimg, ls.max_bins, d, s); L.post(K_BIN_ORDER);
+    L.pre(K_BIN_ORDER); launch_bin_order<T>(ls.atiles, ls.n_atiles, d, s); L.post(K_BIN_ORDER);
     // the neighbour lists index cell-list slots: they are rebuilt with every
     // cell list, also by an energy-only evaluation
     if (ls.n_lj) {

@@ -226,7 +226,7 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 1);
     launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 2);
     launch_bin_scatter(d_tiles, dv.atpi, d_band, s);
-    launch_bin_order<double>(d_img, 1, NA_MAX_BINS, d_band, s);
+    launch_bin_order<double>(d_tiles, dv.atpi, d_band, s);
     launch_lj<double>(d_tiles, dv.atpi, d_band, s);
     launch_image_finalize<double>(d_img, 1, d_band, s);
     if (cudaGetLastError() != cudaSuccess) return CFNEB_ERR_CUDA;
