@@ -29,30 +29,40 @@ __device__ inline bool lj_inside(double r2, double rc2) {
     return less_pos(r2, rc2) && __double_as_longlong(r2) != 0;
 }
 
-// Per-thread LJ accumulators: force on atom i and virial in units of c24 = 24
-// eps / sigma^2 (scaled once per atom, not per pair), energy sum, pair count
+// Per-thread LJ accumulators: force on atom i, energy sum, virial, pair count.
+// FP64 keeps force and virial in units of c24 = 24 eps / sigma^2 and scales
+// once per atom: two FP64 instructions less per pair.  FP32 scales each pair:
+// its steps feed relaxations that amplify a changed rounding, for no gain (the
+// list kernel waits on its gathers).
 template <typename T>
 struct LJAcc {
     T fx = 0, fy = 0, fz = 0, e = 0;
     T v00 = 0, v01 = 0, v02 = 0, v11 = 0, v12 = 0, v22 = 0;
     int cnt = 0;
     // pair vector (rx, ry, rz) with |r|^2 = r2
-    __device__ inline void pair(T rx, T ry, T rz, T r2, T sig2) {
+    __device__ inline void pair(T rx, T ry, T rz, T r2, T sig2, T c24) {
         const T sr2 = lj_sr2(sig2, r2);
-        const T sr6 = sr2 * sr2 * sr2, sr12 = sr6 * sr6;
-        // phi'(r)/r = 24 eps (sr6 - 2 sr12) / r^2
-        const T fr = fma((T)-2, sr12, sr6) * sr2;
+        const T sr6 = sr2 * sr2 * sr2;
+        // phi'(r)/r = 24 eps (sr6 - 2 sr6^2) / r^2
+        T fr;
+        if constexpr (sizeof(T) == 4) {
+            fr = c24 * sr2 * sr6 * ((T)1 - (T)2 * sr6);
+            e += sr6 * (sr6 - (T)1);
+        } else {
+            const T sr12 = sr6 * sr6;
+            fr = fma((T)-2, sr12, sr6) * sr2;
+            e += sr12 - sr6;
+        }
         const T frx = fr * rx, fry = fr * ry, frz = fr * rz;
         fx += frx;
         fy += fry;
         fz += frz;
-        e += sr12 - sr6;
-        v00 = fma(frx, rx, v00);
-        v01 = fma(frx, ry, v01);
-        v02 = fma(frx, rz, v02);
-        v11 = fma(fry, ry, v11);
-        v12 = fma(fry, rz, v12);
-        v22 = fma(frz, rz, v22);
+        v00 += frx * rx;
+        v01 += frx * ry;
+        v02 += frx * rz;
+        v11 += fry * ry;
+        v12 += fry * rz;
+        v22 += frz * rz;
         ++cnt;
     }
 };
@@ -211,8 +221,9 @@ __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandPa
 template <typename T>
 __device__ inline void lj_finish(const LJAcc<T> &A, const LJGeom<T> &g, BandDev &b,
                                  const Tile &tl, int t, bool active) {
+    const T scale = sizeof(T) == 4 ? (T)1 : g.c24;
     if (active) {
-        const T fx = g.c24 * A.fx, fy = g.c24 * A.fy, fz = g.c24 * A.fz;
+        const T fx = scale * A.fx, fy = scale * A.fy, fz = scale * A.fz;
         const T g0 = fx * g.D[0] + fy * g.D[1] + fz * g.D[2];
         const T g1 = fx * g.D[3] + fy * g.D[4] + fz * g.D[5];
         const T g2 = fx * g.D[6] + fy * g.D[7] + fz * g.D[8];
@@ -224,7 +235,7 @@ __device__ inline void lj_finish(const LJAcc<T> &A, const LJGeom<T> &g, BandDev 
     }
     // U_i = 1/2 sum_j [4 eps (sr12 - sr6) - phi(rc)];  V = -1/2 sum r (x) f,
     // written as the symmetric virial in row-major order
-    const T vs = (T)(-0.5) * g.c24;
+    const T vs = (T)(-0.5) * scale;
     T acc[12];
     acc[0] = (T)0.5 * (g.e4 * A.e - g.ephi * (T)A.cnt);
     acc[1] = vs * A.v00;
@@ -235,7 +246,9 @@ __device__ inline void lj_finish(const LJAcc<T> &A, const LJGeom<T> &g, BandDev 
     acc[9] = vs * A.v22;
     acc[10] = (T)A.cnt;
     acc[11] = (T)0;
-    block_sum_store_tr<12, T>(acc, b.atom_part + ((size_t)tl.img * b.atpi + tl.t) * NPART);
+    double *part = b.atom_part + ((size_t)tl.img * b.atpi + tl.t) * NPART;
+    if (sizeof(T) == 4) block_sum_store<12, T>(acc, part);
+    else block_sum_store_tr<12, T>(acc, part);  // 17 FP64 additions per warp instead of 60
 }
 
 // Sums v over the `lanes` (a power of two) adjacent lanes that share an atom.
@@ -408,7 +421,7 @@ __global__ void __launch_bounds__(TILE, 8) k_lj<float>(const Tile *tiles, BandDe
     const size_t base = (size_t)tl.img * n;
     const float4 *off = (const float4 *)b.slot_off + base;
     const int *start = b.bin_start + (size_t)tl.img * (b.nbins_cap + 1);
-    const float rc2 = g.rc2, sig2 = g.sig2;
+    const float rc2 = g.rc2, sig2 = g.sig2, c24 = g.c24;
     LJAcc<float> A;
     if (t < n) {
         int b0, b1, b2;
@@ -419,7 +432,7 @@ __global__ void __launch_bounds__(TILE, 8) k_lj<float>(const Tile *tiles, BandDe
                           [&](int, float ux, float uy, float uz, int, int, int) {
                               const float r2 = ux * ux + uy * uy + uz * uz;
                               // r2 == 0 only for the atom itself at zero shift
-                              if (lj_inside(r2, rc2)) A.pair(ux, uy, uz, r2, sig2);
+                              if (lj_inside(r2, rc2)) A.pair(ux, uy, uz, r2, sig2, c24);
                           });
     }
     A.fx = lane_group_sum(A.fx, lanes);
@@ -445,7 +458,7 @@ __global__ void __launch_bounds__(TILE) k_lj<double>(const Tile *tiles, BandDev 
     const int n = b.n, lanes = TILE / b.tile, lane = threadIdx.x % lanes;
     const int t = tl.t * b.tile + (int)threadIdx.x / lanes;
     const T4 *off = (const T4 *)b.slot_off + (size_t)tl.img * n;
-    const double rc2 = g.rc2, sig2 = g.sig2;
+    const double rc2 = g.rc2, sig2 = g.sig2, c24 = g.c24;
     T4 oi = {};
     if (t < n) oi = off[t];
     LJAcc<double> A;
@@ -455,7 +468,7 @@ __global__ void __launch_bounds__(TILE) k_lj<double>(const Tile *tiles, BandDev 
                                     double x = oj.x - oi.x, y = oj.y - oi.y, z = oj.z - oi.z;
                                     lj_disp(D, code, x, y, z);
                                     const double r2 = x * x + y * y + z * z;
-                                    if (lj_inside(r2, rc2)) A.pair(x, y, z, r2, sig2);
+                                    if (lj_inside(r2, rc2)) A.pair(x, y, z, r2, sig2, c24);
                                 });
     A.fx = lane_group_sum(A.fx, lanes);
     A.fy = lane_group_sum(A.fy, lanes);
@@ -659,7 +672,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_lj_nbr(const Tile *tiles, BandDe
     const int t = tile_atom(b, tl);
     const size_t base = (size_t)tl.img * n;
     const T4 *off = (const T4 *)b.slot_off + base;
-    const T rc2 = g.rc2, sig2 = g.sig2;
+    const T rc2 = g.rc2, sig2 = g.sig2, c24 = g.c24;
     LJAcc<T> A;
     if (t < n) {
         const uint32_t *L = (const uint32_t *)b.nbr_slot + (size_t)tl.img * cap * n + t;
@@ -685,7 +698,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_lj_nbr(const Tile *tiles, BandDe
                 const T uz = (oj[u].z - oi.z) + (a.z + c.z);
                 const T r2 = ux * ux + uy * uy + uz * uz;
                 // r2 == 0: a padding entry (the atom itself)
-                if (lj_inside(r2, rc2)) A.pair(ux, uy, uz, r2, sig2);
+                if (lj_inside(r2, rc2)) A.pair(ux, uy, uz, r2, sig2, c24);
             }
 #pragma unroll
             for (int u = 0; u < LJ_UNROLL; ++u) e[u] = en[u];
@@ -733,7 +746,7 @@ __global__ void __launch_bounds__(TILE, 4) k_lj_nbr64(const Tile *tiles, BandDev
     const size_t base = (size_t)tl.img * n;
     const T4 *off = (const T4 *)b.slot_off + base;
     const float4 *offf = b.slot_off_lo + base;
-    const double rc2 = g.rc2, sig2 = g.sig2;
+    const double rc2 = g.rc2, sig2 = g.sig2, c24 = g.c24;
     const float screen = g.screen;
     const int l0 = D.l0;
     LJAcc<double> A;
@@ -764,7 +777,7 @@ __global__ void __launch_bounds__(TILE, 4) k_lj_nbr64(const Tile *tiles, BandDev
             lj_disp(D, (uint32_t)(i0 | (i1 << 5) | (i2 << 10)), x, y, z);
             const double r2 = x * x + y * y + z * z;
             // r2 == 0: a padding entry (the atom itself)
-            if (lj_inside(r2, rc2)) A.pair(x, y, z, r2, sig2);
+            if (lj_inside(r2, rc2)) A.pair(x, y, z, r2, sig2, c24);
         }
     }
     A.fx = lane_group_sum(A.fx, lanes);
