@@ -141,9 +141,11 @@ __device__ void skin_decide_one(const BandParams *bp, int nbins_cap, ImgScalars 
 // record is staged in shared memory, updated and written back whole.
 template <typename T>
 __global__ void __launch_bounds__(32) k_mapback(const ImgRef *imgs, int count, BandDev *bands,
-                                                int force) {
+                                                int force_) {
     const ImgRef r = imgs[blockIdx.x];
     BandDev &b = bands[r.band];
+    const bool force =
+        force_ == REBUILD_ALL || (force_ == REBUILD_ENDS && (r.img == 0 || r.img == b.bp->N - 1));
     __shared__ BandParams s_bp;
     __shared__ ImgScalars s_sc;
     stage_copy(&s_bp, b.bp);

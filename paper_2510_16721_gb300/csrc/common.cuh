@@ -935,7 +935,10 @@ __device__ inline void stage_copy(S *dst, const S *src) {
 // ---- launchers (defined in the kernel translation units) ---------------
 
 // map-back and the cell-list decision of every image (the displacements
-// since the last build come from the last move, per row tile)
+// since the last build come from the last move, per row tile); force: every
+// image, or the band's end images, whose rows a caller may have replaced,
+// rebuild whatever the decision
+enum : int { REBUILD_ASKED = 0, REBUILD_ALL = 1, REBUILD_ENDS = 2 };
 template <typename T>
 void launch_mapback(const ImgRef *imgs, int count, BandDev *bands, int force, cudaStream_t s);
 // bins or offsets; with has_cond also sets `cond` (a conditional graph

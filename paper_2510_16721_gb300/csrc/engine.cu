@@ -309,7 +309,7 @@ struct LaunchSet {
     const int *band_ids = nullptr;
     int nbands = 0;
     int max_bins = 0;                    // largest nbins_cap among the bands
-    int force_rebuild = 0;               // rebuild every listed image's cell list
+    int force_rebuild = REBUILD_ASKED;   // which images rebuild their cell lists regardless
     int lj_minb = kLjMinb, ters_minb = kTersMinb;  // force kernel variants
     cudaStream_t s_body = nullptr;       // captures the conditional rebuild body
     const Fork *fork = nullptr;          // side stream and events for the finalize
@@ -538,7 +538,7 @@ void enqueue_eval(cfneb_band *b, Launcher &L, const ImgRef *imgs, int nimg, cons
     // ad-hoc image sets (endpoints, new images, reported energies) are
     // evaluated from freshly built cell lists
     LaunchSet ls = band_set(b, imgs, nimg, atiles, natiles);
-    ls.force_rebuild = 1;
+    ls.force_rebuild = REBUILD_ALL;
     enqueue_eval_set<T>(ls, L, forces);
 }
 
@@ -665,24 +665,20 @@ void eval_images(cfneb_band *b, const std::vector<int> &imgs) {
 // FP64 energies (ImgScalars::E64) of the current coordinates: map-back, cell
 // list and the FP64 energy kernel, no forces.  The interior images keep their
 // lists while those still hold (what moves them leaves the displacements the
-// decision needs); the end images, which a caller may have replaced, are
-// evaluated from new ones.
-void refine_interior(cfneb_band *b) {
-    if (b->N < 3) return;
-    const LaunchSet ls = band_step_set(b);
+// decision needs); the end images, where asked for too, get new ones.
+void refine_energies(cfneb_band *b, bool ends) {
+    LaunchSet ls = band_step_set(b);
+    if (ends) {
+        std::vector<int> all;
+        for (int i = 0; i < b->N; ++i) all.push_back(i);
+        const int nt = upload_images(b, all);
+        ls = band_set(b, b->d_scratch_imgs, b->N, b->d_scratch_tiles, nt);
+        ls.force_rebuild = REBUILD_ENDS;
+    }
+    if (ls.nimg <= 0) return;
     Launcher L;
     if (b->precision == CFNEB_MIXED) enqueue_eval_set<float>(ls, L, false);
     else enqueue_eval_set<double>(ls, L, false);
-    CK(cudaGetLastError());
-}
-void refine_ends(cfneb_band *b) {
-    upload_images(b, {0, b->N - 1});
-    Launcher L;
-    if (b->precision == CFNEB_MIXED)
-        enqueue_eval<float>(b, L, b->d_scratch_imgs, 2, b->d_scratch_tiles, 2 * b->dv.atpi, false);
-    else
-        enqueue_eval<double>(b, L, b->d_scratch_imgs, 2, b->d_scratch_tiles, 2 * b->dv.atpi,
-                             false);
     CK(cudaGetLastError());
 }
 
@@ -1159,7 +1155,7 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
     (lj ? ls.atiles_ljc : pot->kind == CFNEB_NEP ? ls.atiles_nep : ls.atiles_ters) = d_tiles;
     (lj ? ls.n_ljc : pot->kind == CFNEB_NEP ? ls.n_nep : ls.n_ters) = (int)tiles.size();
     ls.max_bins = max_bins;
-    ls.force_rebuild = 1;
+    ls.force_rebuild = REBUILD_ALL;
     if (minb > 0 && pot->kind == CFNEB_TERSOFF) ls.ters_minb = minb;
     launch_points_load<T>(d_tiles, ls.n_atiles, d_bands, s);
     Launcher L;
@@ -2066,9 +2062,8 @@ int cfneb_get_path(const cfneb_band *cb, int32_t *n_images, double *positions, d
             // FP64 energies of the current images (map-back, cell list, energy),
             // then Cartesian positions R = R~ D from the same map-back; the
             // endpoints never move, so theirs are computed once
-            if (!b->ends_e64) refine_ends(b);
+            refine_energies(b, !b->ends_e64);
             b->ends_e64 = true;
-            refine_interior(b);
             if (positions) {
                 if (b->precision == CFNEB_MIXED)
                     launch_cartesian<float>(b->N, b->n, b->d_self, b->s);

@@ -220,7 +220,7 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     const ImgRef *d_img = (const ImgRef *)(base + O_IMG);
     k_noalloc_init<<<32, 256, 0, s>>>(dv, bp, dv.atpi);
     launch_points_load<double>(d_tiles, dv.atpi, d_band, s);
-    launch_mapback<double>(d_img, 1, d_band, 1, s);  // forced: the scratch record is reused
+    launch_mapback<double>(d_img, 1, d_band, REBUILD_ALL, s);  // the scratch record is reused
     launch_bin_assign<double>(d_tiles, dv.atpi, d_band, s);
     launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 0);
     launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 1);
