@@ -191,6 +191,8 @@ __global__ void __launch_bounds__(32) k_mapback(const ImgRef *imgs, int count, B
     // the grid (new or kept) follows the cell; a move that left the cell
     // also left the bin vectors of the kept grid
     if (!fresh || sc.rebuild) bin_vectors_warp(sc, sc.nb[(lane % 9) / 3], sc.h[lane % 9]);
+    if (sizeof(T) == 4 && !fresh && b.shift)
+        grid_warp(sc, b.shift + (size_t)r.img * SHIFTS * 6, sc.h[lane % 9], (float)bp->rl);
     __syncwarp();
     stage_copy(&b.sc[r.img], &s_sc);
 }
@@ -203,8 +205,8 @@ __global__ void __launch_bounds__(32) k_mapback(const ImgRef *imgs, int count, B
 // Both keep the offset to ~1e-14 relative of the cell size, far below the
 // FP32 leading part's rounding.  FP64 bands get the FP32 copy in lo.
 __device__ inline void refresh_offset(const ImgScalars &sc, const BandParams *bp, const double *X,
-                                      const int *wr, const int *bi, double4_32a &o,
-                                      float4 &lo) {
+                                      const int *wr, const int *bi, int, const int *,
+                                      double4_32a &o, float4 &lo) {
     double off[3];
     double s[3];
     for (int a = 0; a < 3; ++a)
@@ -223,32 +225,6 @@ __device__ inline void refresh_offset(const ImgScalars &sc, const BandParams *bp
     lo = make_float4((float)off[0], (float)off[1], (float)off[2], (float)bi[2]);
 }
 
-struct F2 {  // unevaluated sum hi + lo of two floats
-    float hi, lo;
-};
-// a (hi + lo) exactly up to the rounding of the low product
-__device__ inline F2 f2_mul(float a, float bh, float bl) {
-    const float p = __fmul_rn(a, bh);
-    float e = fmaf(a, bh, -p);
-    e = fmaf(a, bl, e);
-    return {p, e};
-}
-__device__ inline F2 f2_add(F2 a, F2 b) {
-    const float s = __fadd_rn(a.hi, b.hi);
-    const float bb = __fsub_rn(s, a.hi);
-    float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
-    e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-    const float hi = __fadd_rn(s, e);
-    return {hi, __fsub_rn(e, __fsub_rn(hi, s))};
-}
-
-// Many-body (Tersoff, NEP-style) bands: the leading part is rounded to a
-// multiple of 2^-20 A (the remainder goes to the low part, exactly), so that
-// the force kernel forms (o_j - o_i) + (bin displacement) exactly with plain
-// FP32 operations: every term sits on the 2^-20 grid (bin vectors on a
-// coarser power-of-two grid) and the sums stay below 2^3 A.
-constexpr float OFF_GRID = 1048576.0f;  // 2^20
-
 __device__ inline F2 f2_prod(float a, float b) {  // a b exactly
     const float p = __fmul_rn(a, b);
     return {p, fmaf(a, b, -p)};
@@ -259,8 +235,44 @@ __device__ inline F2 f2_prod(float a, float b) {  // a b exactly
 // (h_a = nb_a bv_a + dh_a): each m_a bv_a is exact as a pair (bv exact in
 // FP32, m_a a half-integer far below 2^23), the dh terms are tiny and join
 // the low part.
+//
+// Many-body (Tersoff, NEP-style) bands hold the position in the cell, R -
+// sum_a wrap_a h_a, on the image's integer grid instead (see
+// common.cuh; o carries the integers' bits; wk: the wrap's place in the table
+// of lattice shifts, SHIFTS / 2 for none, SHIFTS for one beyond the table).
+__device__ inline int wrap_place(const int *wr) {
+    if ((unsigned)(wr[0] + 1) > 2u || (unsigned)(wr[1] + 1) > 2u || (unsigned)(wr[2] + 1) > 2u)
+        return SHIFTS;
+    return (wr[0] + 1) + 3 * (wr[1] + 1) + 9 * (wr[2] + 1);
+}
 __device__ inline void refresh_offset(const ImgScalars &sc, const BandParams *bp, const float *X,
-                                      const int *wr, const int *bi, float4 &o, float4 &lo) {
+                                      const int *wr, const int *bi, int wk, const int *shift,
+                                      float4 &o, float4 &lo) {
+    if (bp->kind != KIND_LJ) {
+        const float *Dh = sc.dfl, *Dl = sc.dfl + 9, *hh = sc.dfl + 18, *hl = sc.dfl + 27;
+        const float g = sc.grid, ig = sc.igrid;
+        int i[3];
+        float l[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            F2 R = f2_mul(X[0], Dh[c], Dl[c]);
+            R = f2_add(R, f2_mul(X[1], Dh[3 + c], Dl[3 + c]));
+            R = f2_add(R, f2_mul(X[2], Dh[6 + c], Dl[6 + c]));
+            if (wk == SHIFTS) {  // wrapped by more than a cell
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    R = f2_add(R, f2_mul(-(float)wr[a], hh[3 * a + c], hl[3 * a + c]));
+            }
+            grid_split(R, g, ig, i[c], l[c]);
+            if (wk < SHIFTS && wk != SHIFTS / 2) {  // by at most one: the table's shift
+                i[c] -= shift[6 * wk + c];
+                l[c] -= __int_as_float(shift[6 * wk + 3 + c]);
+            }
+        }
+        o = make_float4(__int_as_float(i[0]), __int_as_float(i[1]), __int_as_float(i[2]), 0.0f);
+        lo = make_float4(l[0], l[1], l[2], 0.0f);
+        return;
+    }
     const float *Dh = sc.dfl, *Dl = sc.dfl + 9;
     float m[3];
 #pragma unroll
@@ -278,14 +290,8 @@ __device__ inline void refresh_offset(const ImgScalars &sc, const BandParams *bp
         K.lo = fmaf((float)wr[0], sc.dhf[c],
                     fmaf((float)wr[1], sc.dhf[3 + c], fmaf((float)wr[2], sc.dhf[6 + c], K.lo)));
         const F2 d = f2_add(R, {-K.hi, -K.lo});
-        if (bp->kind != KIND_LJ) {
-            const float q = rintf(d.hi * OFF_GRID) * (1.0f / OFF_GRID);
-            off[0][c] = q;
-            off[1][c] = __fadd_rn(__fsub_rn(d.hi, q), d.lo);  // d.hi - q is exact
-        } else {
-            off[0][c] = d.hi;
-            off[1][c] = d.lo;
-        }
+        off[0][c] = d.hi;
+        off[1][c] = d.lo;
     }
     o = make_float4(off[0][0], off[0][1], off[0][2], (float)bi[2]);
     lo = make_float4(off[1][0], off[1][1], off[1][2], 0.0f);
@@ -349,13 +355,15 @@ __global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev 
         if (t >= b.n) return;
         const size_t st = (size_t)tl.img * b.n + t;
         const int i = b.slot_atom[st];
-        int bi[3];
-        unpack_bin(b.slot_bin[st], bi[0], bi[1], bi[2]);
+        int bi[3] = {0, 0, 0};
         const int *wr = b.atom_wrap + ((size_t)tl.img * b.n + i) * 3;
+        int wk = 0;
+        if (b.shift) wk = b.slot_wrap[st];  // grid positions need no bin, and the wrap's place
+        else unpack_bin(b.slot_bin[st], bi[0], bi[1], bi[2]);
         const T *Xi = (const T *)b.X + ((size_t)tl.img * b.rows + i) * 3;
         T4 o;
         float4 lo;
-        refresh_offset(sc, bp, Xi, wr, bi, o, lo);
+        refresh_offset(sc, bp, Xi, wr, bi, wk, b.shift + (size_t)tl.img * SHIFTS * 6, o, lo);
         ((T4 *)b.slot_off)[st] = o;
         b.slot_off_lo[st] = lo;
         return;
@@ -374,7 +382,8 @@ __global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev 
     // for the row traversal of the LJ kernel)
     T4 o;
     float4 lo;
-    refresh_offset(sc, bp, Xi, wrap, bi, o, lo);
+    refresh_offset(sc, bp, Xi, wrap, bi, wrap_place(wrap), b.shift + (size_t)tl.img * SHIFTS * 6, o,
+                   lo);
     ((T4 *)b.atom_off)[ai] = o;
     b.atom_off_lo[ai] = lo;
     if (b.ref_X) {  // a skin: reference state of the build (row layout of X)
@@ -522,6 +531,9 @@ __global__ void __launch_bounds__(TILE) k_bin_order(const Tile *tiles, int ntile
         b.atom_slot[base + i] = dst;
         ((T4 *)b.slot_off)[base + dst] = o;
         b.slot_off_lo[base + dst] = ol;
+        if (b.slot_wrap) {
+            b.slot_wrap[base + dst] = wrap_place(b.atom_wrap + (base + i) * 3);
+        }
     }
 }
 

@@ -104,6 +104,7 @@ struct ImgScalars {
     float dhf[9];        // dh in FP32 (the offset refresh's wrap term)
     float Dbif[9];       // FP32 inverse of Db (list reuse)
     float skin_e, skin_nD;  // the cell's part of the reuse bound (skin_terms)
+    float grid, igrid;   // FP32 many-body bands: position grid and its inverse (powers of two)
     int nb[3];           // bins per axis
     int m[3];            // stencil half width per axis
     int nbins;
@@ -226,12 +227,16 @@ struct BandDev {
     // (atom_bin: linear bin index; slot_bin: the bin's three indices packed
     // by pack_bin)
     void *atom_off, *slot_off;   // [ncap][n] x 4 T (x, y, z, pad): offsets, leading part
+    // Offsets are FP64 or (FP32 LJ bands) FP32 from the atom's bin centre; FP32
+    // many-body bands hold positions in the cell instead, as integers of the
+    // image's grid (int4) and FP32 remainders (float4): see Grid32.
     // [ncap][n] x float4.  FP32 bands: offset - leading part.  FP64 bands: the
     // offset rounded to FP32 (and the bin index), for distance screens
     float4 *atom_off_lo, *slot_off_lo;
     // neighbour-list reuse: positions and periodic wraps at the last build
     void *ref_X;         // [ncap][rows][3] T: R~ at the build (the layout of X)
     int *atom_wrap;      // [ncap][n][3]: floor(s) at the build
+    int *slot_wrap;      // [ncap][n]: the wrap's place in the table of lattice shifts
     float *skin_part;    // [ncap][rtpi]: per-row-tile max displacement
     // per-slot neighbour lists: Tersoff (slot, code) pairs of MAXN_TERSOFF
     // entries, or LJ packed entries of lj_cap (0: the LJ kernel walks the
@@ -245,6 +250,7 @@ struct BandDev {
     const float *nep_wf;
     void *nbr_P;         // [ncap][MAXN][n] x 4 T: partials (x, y, z, pad)
     // partial sums
+    int *shift;          // [ncap][27][6]: lattice shifts on the grid (FP32 many-body bands)
     double *atom_part;   // [ncap][atpi][NPART]
     double *row_part;    // [ncap][rtpi][NPART]
     // double scratch [ncap][n + 3][3]: Cartesian positions (get_path), state
@@ -594,6 +600,102 @@ __device__ inline bool image_cell_warp(const CellIn &k, double xlat, ImgScalars 
     return ok;
 }
 
+// ---- positions on an integer grid (FP32 many-body bands) --------------------
+//
+// The many-body forces need pair vectors to well below FP32's resolution of a
+// position.  Each atom's position in the cell (R minus the lattice vectors it
+// was wrapped by at the list build) is an integer triple of a power-of-two grid
+// g plus an FP32 remainder of at most g / 2.  A pair's leading part is then an
+// exact integer difference that converts to FP32 exactly (|r| < 2^24 g), its
+// low part a difference of remainders (~2^-24 g), and a periodic image adds a
+// lattice shift of the same form: no bin centres, bin displacements or wrap
+// corrections, which took ~190 of a Tersoff atom's ~1,770 instructions (98,303
+// atoms x 9 images: site terms 83.8 -> 79.8 us, offset refresh 21.1 -> 18.0 us;
+// the table below costs the moving warp 0.6 us, which small bands see).
+// g = 2^-22 A for carbon's 2.25 A lists in any cell up to ~800 A, the least
+// power of two with the cell's extent below 2^30 g and rl below 2^24 g / 1.1.
+constexpr int SHIFTS = 27;  // lattice shifts t_a in {-1, 0, 1}; others are formed on the fly
+struct F2 {  // unevaluated sum hi + lo of two floats
+    float hi, lo;
+};
+// a (hi + lo) exactly up to the rounding of the low product
+__device__ inline F2 f2_mul(float a, float bh, float bl) {
+    const float p = __fmul_rn(a, bh);
+    float e = fmaf(a, bh, -p);
+    e = fmaf(a, bl, e);
+    return {p, e};
+}
+__device__ inline F2 f2_add(F2 a, F2 b) {
+    const float s = __fadd_rn(a.hi, b.hi);
+    const float bb = __fsub_rn(s, a.hi);
+    float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
+    e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
+    const float hi = __fadd_rn(s, e);
+    return {hi, __fsub_rn(e, __fsub_rn(hi, s))};
+}
+// v = i g + lo, |v| < 2^33 g, i modulo 2^32.  Rounding by adding 1.5 2^23 (a
+// rintf and a conversion per step would queue at 16 lanes per clock and SM): in
+// units of g, v.hi gives a multiple of 4096 and an exact rest; the rest is a
+// multiple of v.hi's last place and v.lo at most half of one, so their
+// fast two-sum is exact.  A non-finite v ends in lo.
+__device__ inline void grid_split(F2 v, float g, float ig, int &i, float &lo) {
+    const float M = 12582912.0f;  // 1.5 2^23 = 0x4B400000
+    const float u = v.hi * ig, w = v.lo * ig;
+    const float a = __fadd_rn(u * (1.0f / 4096.0f), M);
+    const float rest = fmaf(__fsub_rn(a, M), -4096.0f, u);
+    const float s = __fadd_rn(rest, w), e = __fsub_rn(w, __fsub_rn(s, rest));
+    const float k = __fadd_rn(s, M);
+    i = (int)(((unsigned)__float_as_int(a) - 0x4B400000u) * 4096u +
+              ((unsigned)__float_as_int(k) - 0x4B400000u));
+    lo = __fadd_rn(__fsub_rn(s, __fsub_rn(k, M)), e) * g;
+}
+// exponent of a positive normal x, and 2^e
+__device__ inline int expo(float x) { return (__float_as_int(x) >> 23) - 127; }
+__device__ inline float pow2f(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
+// The lattice shift t on the grid, from the FP32 pairs of h
+__device__ inline void lattice_shift(const float *hh, const float *hl, float g, float ig, int t0,
+                                     int t1, int t2, int (&s)[3], float (&lo)[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        F2 v = f2_mul((float)t0, hh[c], hl[c]);
+        v = f2_add(v, f2_mul((float)t1, hh[3 + c], hl[3 + c]));
+        v = f2_add(v, f2_mul((float)t2, hh[6 + c], hl[6 + c]));
+        grid_split(v, g, ig, s[c], lo[c]);
+    }
+}
+// The grid of an image's cell and its table of lattice shifts (one warp; h =
+// entry lane % 9 of the cell, rl = the list cutoff).  On the move's critical
+// path: the cell's entries go round by shuffles, not through memory.
+static __device__ __noinline__ void grid_warp(ImgScalars &sc, int *shift, double h, float rl) {
+    const int lane = threadIdx.x & 31;
+    const float mh = (float)h, ml = (float)(h - (double)mh);
+    float hh[9], hl[9], ext = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        hh[k] = __shfl_sync(0xffffffffu, mh, k);
+        hl[k] = __shfl_sync(0xffffffffu, ml, k);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ext = fmaxf(ext, fabsf(hh[c]) + fabsf(hh[3 + c]) + fabsf(hh[6 + c]));
+    // 2^e > 1.25 ext (room for drift between builds)
+    const int e = max(expo(1.25f * ext) + 1 - 30, expo(1.1f * rl) + 1 - 24);
+    const float g = pow2f(e), ig = pow2f(-e);
+    if (lane < SHIFTS) {
+        int s[3];
+        float lo[3];
+        lattice_shift(hh, hl, g, ig, lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1, s, lo);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            shift[6 * lane + c] = s[c];
+            shift[6 * lane + 3 + c] = __float_as_int(lo[c]);
+        }
+    }
+    if (lane == 0) {
+        sc.grid = g;
+        sc.igrid = ig;
+    }
+}
+
 // Bin vectors of the image's grid for its current cell, one entry per lane
 // (lanes 0..8; the whole warp calls): bv_a on a grid of q = 2^(e - 19),
 // 2^e >= max |h_a / nb_a|, so every sum of three products delta_a bv_a
@@ -930,6 +1032,68 @@ __device__ inline void stage_copy(S *dst, const S *src) {
         const int i = threadIdx.x + k * blockDim.x;
         if (i < NW) d[i] = w[k];
     }
+}
+
+// ---- many-body lists ---------------------------------------------------------
+
+// FP32 bands: an image's position grid and its table of lattice shifts, staged
+// by the block.  An entry's code is its lattice shift (t0, t1, t2) as packed by
+// pack_code; CODE_ZERO: none.
+struct GridF {
+    float g, ig;
+    int4 s[SHIFTS];     // shift on the grid
+    float4 lo[SHIFTS];  // its remainder
+};
+constexpr int CODE_ZERO = 16 | (16 << 5) | (16 << 10);
+__device__ inline void grid_stage(GridF &G, const BandDev &b, int img) {
+    const int *sh = b.shift + (size_t)img * SHIFTS * 6;
+    if (threadIdx.x < SHIFTS) {
+        const int *p = sh + 6 * threadIdx.x;
+        G.s[threadIdx.x] = make_int4(p[0], p[1], p[2], 0);
+        G.lo[threadIdx.x] = make_float4(__int_as_float(p[3]), __int_as_float(p[4]),
+                                        __int_as_float(p[5]), 0.0f);
+    }
+    if (threadIdx.x == 32) G.g = b.sc[img].grid;
+    if (threadIdx.x == 33) G.ig = b.sc[img].igrid;
+}
+// The shift of a code: the table's, or (cells narrower than the list cutoff)
+// formed from the cell
+__device__ inline void grid_shift(const GridF &G, const ImgScalars &sc, int code, int (&s)[3],
+                                  float (&lo)[3]) {
+    const int t0 = (code & 31) - 16, t1 = ((code >> 5) & 31) - 16, t2 = ((code >> 10) & 31) - 16;
+    if ((unsigned)(t0 + 1) <= 2u && (unsigned)(t1 + 1) <= 2u && (unsigned)(t2 + 1) <= 2u) {
+        const int k = (t0 + 1) + 3 * (t1 + 1) + 9 * (t2 + 1);
+        s[0] = G.s[k].x; s[1] = G.s[k].y; s[2] = G.s[k].z;
+        lo[0] = G.lo[k].x; lo[1] = G.lo[k].y; lo[2] = G.lo[k].z;
+    } else {
+        lattice_shift(sc.dfl + 18, sc.dfl + 27, G.g, G.ig, t0, t1, t2, s, lo);
+    }
+}
+
+// Bin offset and periodic wrap of a stencil code from bin (b0, b1, b2)
+__device__ inline void ters_code(int code, int b0, int b1, int b2, const int *s_nb, int (&d)[3],
+                                 int (&t)[3]) {
+    const int b[3] = {b0, b1, b2};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        d[a] = ((code >> (5 * a)) & 31) - 16;
+        int w = b[a] + d[a];
+        t[a] = 0;
+        while (w < 0) { w += s_nb[a]; --t[a]; }
+        while (w >= s_nb[a]) { w -= s_nb[a]; ++t[a]; }
+    }
+}
+
+// b = (1 + x)^(-1/2n) for x = (beta zeta)^n: below 2^-10 (carbon: ~1e-4) by
+// the series of log(1 + x) to x^6 and exp(-u) to u^5 (truncation below 1e-18
+// relative)
+__device__ inline double bond_order_x(double x, double inv2n) {
+    if (x < 1.0 / 1024.0) {
+        const double l = x * (1.0 - x * (0.5 - x * (1.0 / 3.0 - x * (0.25 - x * (0.2 - x * (1.0 / 6.0))))));
+        const double u = inv2n * l;
+        return 1.0 - u * (1.0 - u * (0.5 - u * (1.0 / 6.0 - u * (1.0 / 24.0 - u * (1.0 / 120.0)))));
+    }
+    return exp(-inv2n * log1p(x));
 }
 
 // ---- launchers (defined in the kernel translation units) ---------------

@@ -19,128 +19,139 @@
 
 namespace cfneb {
 
-// FP32 bands: two-term offsets (ol, jl the remainders); FP64 bands: the offsets
-__device__ inline void pair_vec64(const float4 &oi, const float4 &oil, const float4 &oj,
-                                  const float4 &ojl, const double *c, double *r) {
-    r[0] = ((double)oj.x + (double)ojl.x) - ((double)oi.x + (double)oil.x) + c[0];
-    r[1] = ((double)oj.y + (double)ojl.y) - ((double)oi.y + (double)oil.y) + c[1];
-    r[2] = ((double)oj.z + (double)ojl.z) - ((double)oi.z + (double)oil.z) + c[2];
+// Unit vectors, lengths and their inverses of the neighbour-list entries of
+// slot t within rc (periodic images included, the atom itself excluded), in
+// FP64; returns their count.  FP32 bands: grid differences are exact in FP32
+// and converted by integer operations, the remainders join with one FP64
+// addition.  FP64 bands: bin displacements exact in FP32, wraps where there are
+// any.
+struct Entries64 {
+    double x[MAXN_TERSOFF], y[MAXN_TERSOFF], z[MAXN_TERSOFF], r[MAXN_TERSOFF];
+};
+__device__ inline bool add_entry(Entries64 &E, int k, double x, double y, double z, double rc2) {
+    const double r2 = x * x + y * y + z * z;
+    if (!(r2 < rc2 && r2 > 0.0)) return false;
+    double r, ir;
+    sqrt_rcp64(r2, r, ir);
+    E.x[k] = x * ir;
+    E.y[k] = y * ir;
+    E.z[k] = z * ir;
+    E.r[k] = r;
+    return true;
 }
-__device__ inline void pair_vec64(const double4_32a &oi, const float4 &, const double4_32a &oj,
-                                  const float4 &, const double *c, double *r) {
-    r[0] = oj.x - oi.x + c[0];
-    r[1] = oj.y - oi.y + c[1];
-    r[2] = oj.z - oi.z + c[2];
-}
-
-// b = (1 + (beta zeta)^n)^(-1/2n) with m2n = -1/2n: x = (beta zeta)^n from
-// log and exp; for x < 1e-3 (carbon: x ~ 1e-5) b = exp(m2n log1p(x)) by
-// their series (log1p to x^5: 2e-13 relative at the bound, exp to y^6);
-// otherwise the library power
-__device__ inline double bond_order64(double bz, double n, double m2n) {
-    if (!(bz > 0.0)) return 1.0;
-    const double x = exp(n * log(bz));
-    if (x >= 1e-3) return pow(1.0 + x, m2n);
-    const double L = x * (1.0 - x * (0.5 - x * (1.0 / 3.0 - x * (0.25 - x * 0.2))));
-    const double y = m2n * L;
-    return 1.0 + y * (1.0 + y * (0.5 + y * (1.0 / 6.0 + y * (1.0 / 24.0 + y * (1.0 / 120.0 + y / 720.0)))));
-}
-
-// FP64 pair vectors of the neighbour-list entries of slot t within rc
-// (periodic images included, the atom itself excluded); returns their count
-template <typename T>
-__device__ inline int list_vectors64(const BandDev &b, int img, int t, const ImgScalars &sc,
-                                     double rc, double *rx, double *ry, double *rz, double *rd) {
-    using T4 = typename Vec4<T>::type;
-    const size_t base = (size_t)img * b.n;
-    const T4 *off = (const T4 *)b.slot_off + base;
-    const float4 *offl = b.slot_off_lo + base;
-    const int *nslot = b.nbr_slot + (size_t)img * MAXN_TERSOFF * b.n;
-    const int *ncode = b.nbr_code + (size_t)img * MAXN_TERSOFF * b.n;
+__device__ inline int entries64(const BandDev &b, const Tile &tl, int t, double rc,
+                                const GridF &G, Entries64 &E, float) {
+    const ImgScalars &sc = b.sc[tl.img];
+    const size_t base = (size_t)tl.img * b.n;
+    const int4 *pos = (const int4 *)b.slot_off + base;
+    const float4 *rem = b.slot_off_lo + base;
+    const int *nslot = b.nbr_slot + base * MAXN_TERSOFF;
+    const int *ncode = b.nbr_code + base * MAXN_TERSOFF;
     const int ne = b.nbr_cnt[base + t];
-    int bb[3];
-    unpack_bin(b.slot_bin[base + t], bb[0], bb[1], bb[2]);
-    const T4 oi = off[t];
-    const float4 oil = offl[t];
+    const int4 pi = pos[t];
+    const float4 li = rem[t];
     int cnt = 0;
     for (int e = 0; e < ne; ++e) {
-        const int q = nslot[(size_t)e * b.n + t];
-        const int code = ncode[(size_t)e * b.n + t];
-        const int dd[3] = {(code & 31) - 16, ((code >> 5) & 31) - 16, ((code >> 10) & 31) - 16};
-        int tt[3];
-        for (int a = 0; a < 3; ++a) {
-            int w = bb[a] + dd[a];
-            tt[a] = 0;
-            while (w < 0) { w += sc.nb[a]; --tt[a]; }
-            while (w >= sc.nb[a]) { w -= sc.nb[a]; ++tt[a]; }
+        const int q = nslot[(size_t)e * b.n + t], code = ncode[(size_t)e * b.n + t];
+        const int4 pj = pos[q];
+        const float4 lj = rem[q];
+        int s[3] = {0, 0, 0};
+        float lo[3] = {0.0f, 0.0f, 0.0f};
+        if (code != CODE_ZERO) grid_shift(G, sc, code, s, lo);
+        const double x = f2d((float)(pj.x - pi.x + s[0]) * G.g) + f2d((lj.x - li.x) + lo[0]);
+        const double y = f2d((float)(pj.y - pi.y + s[1]) * G.g) + f2d((lj.y - li.y) + lo[1]);
+        const double z = f2d((float)(pj.z - pi.z + s[2]) * G.g) + f2d((lj.z - li.z) + lo[2]);
+        cnt += add_entry(E, cnt, x, y, z, rc * rc);
+    }
+    return cnt;
+}
+__device__ inline int entries64(const BandDev &b, const Tile &tl, int t, double rc, const GridF &,
+                                Entries64 &E, double) {
+    const ImgScalars &sc = b.sc[tl.img];
+    const size_t base = (size_t)tl.img * b.n;
+    const double4_32a *off = (const double4_32a *)b.slot_off + base;
+    const int *nslot = b.nbr_slot + base * MAXN_TERSOFF;
+    const int *ncode = b.nbr_code + base * MAXN_TERSOFF;
+    const int ne = b.nbr_cnt[base + t];
+    int b0, b1, b2;
+    unpack_bin(b.slot_bin[base + t], b0, b1, b2);
+    const double4_32a oi = off[t];
+    int cnt = 0;
+    for (int e = 0; e < ne; ++e) {
+        const double4_32a oj = off[nslot[(size_t)e * b.n + t]];
+        int d[3], w[3];
+        ters_code(ncode[(size_t)e * b.n + t], b0, b1, b2, sc.nb, d, w);
+        double v[3] = {oj.x - oi.x, oj.y - oi.y, oj.z - oi.z};
+        for (int c = 0; c < 3; ++c) {
+            v[c] += f2d(d[0] * sc.bvf[c] + d[1] * sc.bvf[3 + c] + d[2] * sc.bvf[6 + c]);
+            if (w[0] | w[1] | w[2])
+                v[c] += f2d((float)w[0]) * sc.dh[c] + f2d((float)w[1]) * sc.dh[3 + c] +
+                        f2d((float)w[2]) * sc.dh[6 + c];
         }
-        double c[3];
-        for (int k = 0; k < 3; ++k)
-            c[k] = dd[0] * sc.bv[k] + dd[1] * sc.bv[3 + k] + dd[2] * sc.bv[6 + k] +
-                   tt[0] * sc.dh[k] + tt[1] * sc.dh[3 + k] + tt[2] * sc.dh[6 + k];
-        double r[3];
-        pair_vec64(oi, oil, off[q], offl[q], c, r);
-        const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-        if (r2 < rc * rc && r2 > 0.0) {
-            rx[cnt] = r[0];
-            ry[cnt] = r[1];
-            rz[cnt] = r[2];
-            rd[cnt] = sqrt(r2);
-            ++cnt;
-        }
+        cnt += add_entry(E, cnt, v[0], v[1], v[2], rc * rc);
     }
     return cnt;
 }
 
+// FP64 site energies.  Bound by the FP64 pipe: angular terms run over unordered
+// pairs (symmetric in j, k), constants derived on the host, reciprocals by
+// Newton steps (98,304 carbon atoms: 152 us; 282 us with ordered pairs,
+// divisions and FP64 conversions of every coordinate).
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_energy64(const Tile *tiles, BandDev *bands) {
     Tile tl = tiles[blockIdx.x];
     BandDev &b = bands[tl.band];
-    const ImgScalars &sc = b.sc[tl.img];
     const BandParams *bp = b.bp;
+    __shared__ GridF G;
+    __shared__ TP<double> q;
+    if (sizeof(T) == 4) grid_stage(G, b, tl.img);
+    stage_copy(&q, &bp->tpd);
+    __syncthreads();
     const int t = tile_atom(b, tl);
     double U = 0.0;
     if (t < b.n) {
+        Entries64 E;
         if (bp->kind == KIND_TERSOFF) {
-            const TersoffParams p = *(const TersoffParams *)bp->pot;
-            const double rc = p.R + p.D;
-            double rx[MAXN_TERSOFF], ry[MAXN_TERSOFF], rz[MAXN_TERSOFF], rd[MAXN_TERSOFF];
-            const int cnt = list_vectors64<T>(b, tl.img, t, sc, rc, rx, ry, rz, rd);
-            const double pi = 3.14159265358979323846;
-            const double c2d2 = p.c * p.c / (p.d * p.d), d2 = p.d * p.d;
-            const double pi_4D = 0.25 * pi / p.D, m2n = -0.5 / p.n;
-            double fc[MAXN_TERSOFF], ir[MAXN_TERSOFF];
+            const int cnt = entries64(b, tl, t, q.R + q.D, G, E, T());
+            double fc[MAXN_TERSOFF], zeta[MAXN_TERSOFF];
             for (int k = 0; k < cnt; ++k) {
-                const double sk = rd[k] - p.R;
-                const double sn = sin_quarter64(pi_4D * (p.D - sk));
-                fc[k] = sk <= -p.D ? 1.0 : (sk >= p.D ? 0.0 : sn * sn);
-                ir[k] = rcp64(rd[k]);
+                const double s = E.r[k] - q.R;
+                fc[k] = 1.0;
+                if (s > -q.D) {
+                    const double sn = s < q.D ? sin_quarter64(q.pi_4D * (q.D - s)) : 0.0;
+                    fc[k] = sn * sn;
+                }
+                zeta[k] = 0.0;
+            }
+            for (int j = 1; j < cnt; ++j) {
+                double zj = 0.0;
+                for (int k = 0; k < j; ++k) {
+                    const double u = q.h - (E.x[j] * E.x[k] + E.y[j] * E.y[k] + E.z[j] * E.z[k]);
+                    const double u2 = u * u;
+                    const double g = fma(q.c2d2 * u2, rcp64_pos(q.d2 + u2), 1.0);
+                    zj = fma(fc[k], g, zj);
+                    zeta[k] = fma(fc[j], g, zeta[k]);
+                }
+                zeta[j] += zj;
             }
             for (int j = 0; j < cnt; ++j) {
                 if (fc[j] == 0.0) continue;  // beyond R + D
-                double zeta = 0.0;
-                for (int k = 0; k < cnt; ++k) {
-                    if (k == j) continue;
-                    const double cs = (rx[j] * rx[k] + ry[j] * ry[k] + rz[j] * rz[k]) * ir[j] * ir[k];
-                    const double u = p.h - cs;
-                    const double g = 1.0 + c2d2 * u * u * rcp64(d2 + u * u);
-                    zeta += fc[k] * g;
-                }
-                U += 0.5 * fc[j] * (p.A * exp(-p.lambda1 * rd[j]) -
-                                    bond_order64(p.beta * zeta, p.n, m2n) * p.B * exp(-p.lambda2 * rd[j]));
+                const double bz = q.beta * zeta[j];
+                const double bij = bz > 0.0 ? bond_order_x(exp(q.n * log(bz)), q.inv2n) : 1.0;
+                U += 0.5 * fc[j] * (q.A * exp(-q.l1 * E.r[j]) - bij * q.B * exp(-q.l2 * E.r[j]));
             }
         } else {
             // NEP-style site energy (descriptors and network as in the force
-            // kernel), in FP64 from the list's pair vectors
-            const double rc = bp->pot[0];
-            double rx[MAXN_TERSOFF], ry[MAXN_TERSOFF], rz[MAXN_TERSOFF], rd[MAXN_TERSOFF];
-            const int cnt = list_vectors64<T>(b, tl.img, t, sc, rc, rx, ry, rz, rd);
+            // kernel)
+            const double rc = bp->pot[0], irc = rcp64_pos(rc);
+            const int cnt = entries64(b, tl, t, rc, G, E, T());
             const double *w = b.nep_w;
             double qd[NEP_ND], gA[MAXN_TERSOFF][NEP_NA];
             for (int d = 0; d < NEP_ND; ++d) qd[d] = 0.0;
             for (int j = 0; j < cnt; ++j) {
-                const double fcj = 0.5 * (1.0 + cospi(rd[j] / rc));
-                const double x = 2.0 * (rd[j] / rc - 1.0) * (rd[j] / rc - 1.0) - 1.0;
+                const double rr = E.r[j] * irc;
+                const double fcj = 0.5 * (1.0 + cospi(rr));
+                const double x = 2.0 * (rr - 1.0) * (rr - 1.0) - 1.0;
                 double f[NEP_K], t0 = 1.0, t1 = x;
                 f[0] = fcj;
                 f[1] = 0.5 * (x + 1.0) * fcj;
@@ -157,15 +168,19 @@ __global__ void __launch_bounds__(TILE) k_energy64(const Tile *tiles, BandDev *b
                     for (int k = 0; k < NEP_K; ++k) gA[j][m] += w[NEP_OCA + m * NEP_K + k] * f[k];
                 }
             }
-            for (int j = 0; j < cnt; ++j)
-                for (int k = 0; k < cnt; ++k) {
-                    const double c = (rx[j] * rx[k] + ry[j] * ry[k] + rz[j] * rz[k]) / (rd[j] * rd[k]);
+            for (int j = 0; j < cnt; ++j) {
+                for (int m = 0; m < NEP_NA; ++m)  // k = j: P_l(1) = 1
+                    for (int l = 0; l < NEP_L; ++l) qd[NEP_NR + m * NEP_L + l] += gA[j][m] * gA[j][m];
+                for (int k = 0; k < j; ++k) {
+                    const double c = E.x[j] * E.x[k] + E.y[j] * E.y[k] + E.z[j] * E.z[k];
                     const double P[4] = {c, 1.5 * c * c - 0.5, (2.5 * c * c - 1.5) * c,
                                          (4.375 * c * c - 3.75) * c * c + 0.375};
-                    for (int m = 0; m < NEP_NA; ++m)
-                        for (int l = 0; l < NEP_L; ++l)
-                            qd[NEP_NR + m * NEP_L + l] += gA[j][m] * gA[k][m] * (j == k ? 1.0 : P[l]);
+                    for (int m = 0; m < NEP_NA; ++m) {
+                        const double gg = 2.0 * gA[j][m] * gA[k][m];
+                        for (int l = 0; l < NEP_L; ++l) qd[NEP_NR + m * NEP_L + l] += gg * P[l];
+                    }
                 }
+            }
             double Ui = -w[NEP_OB1];
             for (int h = 0; h < NEP_H; ++h) {
                 double a = -w[NEP_OB0 + h];

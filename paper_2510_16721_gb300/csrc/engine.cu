@@ -1111,6 +1111,7 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
             ar.add(&d.nbr_code, na * MAXN_TERSOFF * sizeof(int));
             ar.add(&d.nbr_rev, na * MAXN_TERSOFF);
             ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * sizeof(T));
+            if (sizeof(T) == 4) ar.add(&d.shift, SHIFTS * 6 * sizeof(int));
         }
         ar.add(&d.atom_part, (size_t)d.atpi * NPART * sizeof(double));
     }
@@ -1317,6 +1318,7 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
     ar.add(&d.slot_off_lo, na * sizeof(float4));
     if (skin > 0.0) {
         ar.add(&d.atom_wrap, na * 3 * sizeof(int));
+        if (many && b->ts == 4) ar.add(&d.slot_wrap, na * sizeof(int));
         ar.add(&d.skin_part, nc * d.rtpi * sizeof(float));
     }
     if (lj_list) ar.add(&d.nbr_slot, na * d.lj_cap * sizeof(int));
@@ -1328,6 +1330,7 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
         ar.add(&d.nbr_code, na * MAXN_TERSOFF * sizeof(int));
         ar.add(&d.nbr_rev, na * MAXN_TERSOFF);
         ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * b->ts);
+        if (b->ts == 4) ar.add(&d.shift, nc * SHIFTS * 6 * sizeof(int));
     }
     ar.add(&d.atom_part, nc * d.atpi * NPART * sizeof(double));
     ar.add(&d.row_part, nc * d.rtpi * NPART * sizeof(double));
