@@ -36,8 +36,9 @@ namespace cfneb {
 
 template <typename T>
 __global__ void __launch_bounds__(FIN_THREADS) k_image_finalize(const ImgRef *imgs, BandDev *bands) {
-    ImgRef r = imgs[blockIdx.x];
-    BandDev &b = bands[r.band];
+    const ImgRef r = imgs[blockIdx.x];
+    const BandDev b = bands[r.band];
+    dep_sync();
     const BandParams *bp = b.bp;
     ImgScalars &sc = b.sc[r.img];
     // U, V (9), pairs, triples: tile partials summed in FP64, fixed order
@@ -226,7 +227,7 @@ __device__ inline int climbing_image_warp(const BandDev &b, int N, double e0) {
 // energies, FP32 site energies summed in FP64, so that the upwind branch is
 // not chosen by rounding between nearly equal images -- those take the
 // equal-weight tangent dX+ + dX-).
-__device__ inline void image_coef(BandDev &b, int i, int ci, const double *d, double Em,
+__device__ inline void image_coef(const BandDev &b, int i, int ci, const double *d, double Em,
                                   double E0, double Ep, double kspring, double etol) {
     ImgScalars &sc = b.sc[i];
     double wp, wm;
@@ -292,8 +293,9 @@ __device__ inline void st_rows(double *p, const double (&v)[3]) {
 
 template <typename T, bool FUSE>
 __global__ void __launch_bounds__(RTHREADS, sizeof(T) == 4 ? 4 : 2) k_band_dots(const Tile *tiles, BandDev *bands) {
-    Tile tl = tiles[blockIdx.x];
-    BandDev &b = bands[tl.band];
+    const Tile tl = tiles[blockIdx.x];
+    const BandDev b = bands[tl.band];
+    dep_sync();
     Acc<T> acc[10];
     constexpr int RPT = rows_per_thread(sizeof(T));
     const size_t stride = (size_t)b.rows * 3;
@@ -439,8 +441,9 @@ template <> struct UIntOf<double> { using type = unsigned long long; };
 // the FIRE decision on the sums of pass 1.
 template <typename T>
 __global__ void __launch_bounds__(RTHREADS, 4) k_neb_force(const Tile *tiles, BandDev *bands) {
-    Tile tl = tiles[blockIdx.x];
-    BandDev &b = bands[tl.band];
+    const Tile tl = tiles[blockIdx.x];
+    const BandDev b = bands[tl.band];
+    dep_sync();
     constexpr int RPT = rows_per_thread(sizeof(T));
     const size_t stride = (size_t)b.rows * 3;
     const int r0 = tl.t * row_tile(sizeof(T)) + RPT * (int)threadIdx.x;
@@ -553,8 +556,7 @@ __device__ inline void fire_row(T *x, T *v, const T *fn, T cv, T cf, T dt, T ms)
 // next evaluation's map-back finds them ready (cell_fresh) instead of
 // starting its FP64 chain only then.  Runs beside the atom rows' blocks.
 template <typename T>
-__device__ inline void lattice_move_warp(const ImgRef r, BandDev *bands) {
-    BandDev &b = bands[r.band];
+__device__ inline void lattice_move_warp(const ImgRef r, const BandDev &b) {
     const BandParams *bp = b.bp;
     ImgScalars &sc = b.sc[r.img];
     const int lane = threadIdx.x & 31, l = lane % 9;
@@ -609,8 +611,7 @@ __device__ inline void lattice_move_warp(const ImgRef r, BandDev *bands) {
 // rows: lattice_move_warp; padding rows stay zero), and with a skin the
 // tile records its largest displacement since the last list build.
 template <typename T>
-__device__ inline void move_tile(const Tile tl, BandDev *bands) {
-    BandDev &b = bands[tl.band];
+__device__ inline void move_tile(const Tile tl, const BandDev &b) {
     const BandParams *bp = b.bp;
     constexpr int RPT = rows_per_thread(sizeof(T));
     const int r0 = tl.t * row_tile(sizeof(T)) + RPT * (int)threadIdx.x;
@@ -696,11 +697,18 @@ template <typename T>
 __global__ void __launch_bounds__(RTHREADS, sizeof(T) == 4 ? 4 : 2)
     k_fire_update(const Tile *tiles, int ntiles, const ImgRef *imgs, int nimg, BandDev *bands) {
     if ((int)blockIdx.x < nimg) {
-        if (threadIdx.x < 32) lattice_move_warp<T>(imgs[blockIdx.x], bands);
+        const ImgRef r = imgs[blockIdx.x];
+        const BandDev b = bands[r.band];
+        dep_sync();
+        if (threadIdx.x < 32) lattice_move_warp<T>(r, b);
         return;
     }
     const int k0 = ((int)blockIdx.x - nimg) * FU_TILES;
-    for (int k = k0; k < k0 + FU_TILES && k < ntiles; ++k) move_tile<T>(tiles[k], bands);
+    const Tile t0 = tiles[k0];
+    const BandDev b0 = bands[t0.band];
+    dep_sync();
+    move_tile<T>(t0, b0);
+    for (int k = k0 + 1; k < k0 + FU_TILES && k < ntiles; ++k) move_tile<T>(tiles[k], bands[tiles[k].band]);
 }
 
 // X_img <- 1/2 (X_{img-1} + X_{img+1}) (image insertion; all rows)
@@ -909,19 +917,19 @@ void launch_set_control(BandDev *band, double ftol, long long move_limit, cudaSt
 template <typename T>
 void launch_image_finalize(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t s) {
     if (count <= 0) return;
-    k_image_finalize<T><<<count, FIN_THREADS, 0, s>>>(imgs, bands);
+    launch_dep(k_image_finalize<T>, count, FIN_THREADS, s, imgs, bands);
 }
 // pass 1 of the step (fused: per-image dots, NEB coefficients, FIRE sums)
 template <typename T>
 void launch_band_dots(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    k_band_dots<T, true><<<ntiles, RTHREADS, 0, s>>>(tiles, bands);
+    launch_dep(k_band_dots<T, true>, ntiles, RTHREADS, s, tiles, bands);
 }
 // the dots alone (into the tile records; k_dots_reduce sums them per image)
 template <typename T>
 void launch_band_dots_only(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    k_band_dots<T, false><<<ntiles, RTHREADS, 0, s>>>(tiles, bands);
+    launch_dep(k_band_dots<T, false>, ntiles, RTHREADS, s, tiles, bands);
 }
 void launch_dots_reduce(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t s) {
     if (count <= 0) return;
@@ -934,14 +942,13 @@ void launch_shard_fire(BandDev *band, double P, double FF, double VV, double fma
 template <typename T>
 void launch_neb_force(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    k_neb_force<T><<<ntiles, RTHREADS, 0, s>>>(tiles, bands);
+    launch_dep(k_neb_force<T>, ntiles, RTHREADS, s, tiles, bands);
 }
 template <typename T>
 void launch_fire_update(const Tile *tiles, int ntiles, const ImgRef *imgs, int nimg,
                         BandDev *bands, cudaStream_t s) {
     if (ntiles + nimg <= 0) return;
-    k_fire_update<T><<<nimg + (ntiles + FU_TILES - 1) / FU_TILES, RTHREADS, 0, s>>>(
-        tiles, ntiles, imgs, nimg, bands);
+    launch_dep(k_fire_update<T>, nimg + (ntiles + FU_TILES - 1) / FU_TILES, RTHREADS, s,  tiles, ntiles, imgs, nimg, bands);
 }
 template <typename T>
 void launch_midpoint(BandDev *band, int img, int rows, cudaStream_t s) {

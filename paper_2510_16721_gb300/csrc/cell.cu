@@ -143,7 +143,8 @@ template <typename T>
 __global__ void __launch_bounds__(32) k_mapback(const ImgRef *imgs, int count, BandDev *bands,
                                                 int force_) {
     const ImgRef r = imgs[blockIdx.x];
-    BandDev &b = bands[r.band];
+    const BandDev b = bands[r.band];
+    dep_sync();
     const bool force =
         force_ == REBUILD_ALL || (force_ == REBUILD_ENDS && (r.img == 0 || r.img == b.bp->N - 1));
     __shared__ BandParams s_bp;
@@ -338,13 +339,16 @@ __device__ inline void bin_of(const ImgScalars &sc, const BandParams *, const fl
 // In a graph (has_cond), the first tile of every image that rebuilds also
 // switches on the conditional node that holds the rebuild kernels (its
 // value is reset to 0 at every launch of the graph).
+// FP32: 12 blocks per SM (40 registers, 18.4 us at 98,303 atoms x 9 images; 18.9
+// with the 48 that the tables read ahead take).
 template <typename T>
-__global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev *bands,
+__global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 12 : 8) k_bin_assign(const Tile *tiles, BandDev *bands,
                                                      cudaGraphConditionalHandle cond,
                                                      int has_cond) {
     using T4 = typename Vec4<T>::type;
-    Tile tl = tiles[blockIdx.x];
-    BandDev &b = bands[tl.band];
+    const Tile tl = tiles[blockIdx.x];
+    const BandDev b = bands[tl.band];
+    dep_sync();
     const ImgScalars &sc = b.sc[tl.img];
     const BandParams *bp = b.bp;
     if (has_cond && sc.rebuild && tl.t == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 1u);
@@ -368,30 +372,32 @@ __global__ void __launch_bounds__(TILE) k_bin_assign(const Tile *tiles, BandDev 
         b.slot_off_lo[st] = lo;
         return;
     }
-    const int i = tile_atom(b, tl);
-    if (i >= b.n) return;
-    const T *Xi = (const T *)b.X + ((size_t)tl.img * b.rows + i) * 3;
+    // (through the table: what only a rebuild needs holds no registers above)
+    const BandDev &br = bands[tl.band];
+    const int i = tile_atom(br, tl);
+    if (i >= br.n) return;
+    const T *Xi = (const T *)br.X + ((size_t)tl.img * br.rows + i) * 3;
     int bi[3], wrap[3];
     bin_of(sc, bp, Xi, bi, wrap);
     int lin = (bi[0] * sc.nb[1] + bi[1]) * sc.nb[2] + bi[2];
-    size_t ai = (size_t)tl.img * b.n + i;
-    int rank = atomicAdd(&b.bin_count[(size_t)tl.img * b.nbins_cap + lin], 1);
-    b.atom_bin[ai] = lin;
-    b.atom_rank[ai] = rank;
+    size_t ai = (size_t)tl.img * br.n + i;
+    int rank = atomicAdd(&br.bin_count[(size_t)tl.img * br.nbins_cap + lin], 1);
+    br.atom_bin[ai] = lin;
+    br.atom_rank[ai] = rank;
     // offset from the bin centre (the w lane holds the innermost bin index,
     // for the row traversal of the LJ kernel)
     T4 o;
     float4 lo;
-    refresh_offset(sc, bp, Xi, wrap, bi, wrap_place(wrap), b.shift + (size_t)tl.img * SHIFTS * 6, o,
+    refresh_offset(sc, bp, Xi, wrap, bi, wrap_place(wrap), br.shift + (size_t)tl.img * SHIFTS * 6, o,
                    lo);
-    ((T4 *)b.atom_off)[ai] = o;
-    b.atom_off_lo[ai] = lo;
-    if (b.ref_X) {  // a skin: reference state of the build (row layout of X)
-        T *ref = (T *)b.ref_X + ((size_t)tl.img * b.rows + i) * 3;
+    ((T4 *)br.atom_off)[ai] = o;
+    br.atom_off_lo[ai] = lo;
+    if (br.ref_X) {  // a skin: reference state of the build (row layout of X)
+        T *ref = (T *)br.ref_X + ((size_t)tl.img * br.rows + i) * 3;
         ref[0] = Xi[0];
         ref[1] = Xi[1];
         ref[2] = Xi[2];
-        for (int a = 0; a < 3; ++a) b.atom_wrap[ai * 3 + a] = wrap[a];
+        for (int a = 0; a < 3; ++a) br.atom_wrap[ai * 3 + a] = wrap[a];
     }
 }
 
@@ -427,6 +433,7 @@ __device__ inline int block_excl_scan_1024(int v, int *total) {
 }
 
 __global__ void __launch_bounds__(256) k_bin_tilesum(const ImgRef *imgs, BandDev *bands) {
+    dep_sync();
     ImgRef r = imgs[blockIdx.y];
     BandDev &b = bands[r.band];
     if (!b.sc[r.img].rebuild) return;
@@ -452,6 +459,7 @@ __global__ void __launch_bounds__(256) k_bin_tilesum(const ImgRef *imgs, BandDev
 }
 
 __global__ void __launch_bounds__(1024) k_bin_tilescan(const ImgRef *imgs, BandDev *bands) {
+    dep_sync();
     ImgRef r = imgs[blockIdx.x];
     BandDev &b = bands[r.band];
     if (!b.sc[r.img].rebuild) return;
@@ -469,6 +477,7 @@ __global__ void __launch_bounds__(1024) k_bin_tilescan(const ImgRef *imgs, BandD
 }
 
 __global__ void __launch_bounds__(1024) k_bin_scanfill(const ImgRef *imgs, BandDev *bands) {
+    dep_sync();
     ImgRef r = imgs[blockIdx.y];
     BandDev &b = bands[r.band];
     if (!b.sc[r.img].rebuild) return;
@@ -490,6 +499,7 @@ __global__ void __launch_bounds__(1024) k_bin_scanfill(const ImgRef *imgs, BandD
 }
 
 __global__ void __launch_bounds__(TILE) k_bin_scatter(const Tile *tiles, int ntiles, BandDev *bands) {
+    dep_sync();
     for (int k = blockIdx.x; k < ntiles; k += gridDim.x) {
         const Tile tl = tiles[k];
         BandDev &b = bands[tl.band];
@@ -508,6 +518,7 @@ __global__ void __launch_bounds__(TILE) k_bin_scatter(const Tile *tiles, int nti
 // loops: 19,380 atoms in 972 bins, 54 us.)
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_bin_order(const Tile *tiles, int ntiles, BandDev *bands) {
+    dep_sync();
     using T4 = typename Vec4<T>::type;
     for (int k = blockIdx.x; k < ntiles; k += gridDim.x) {
         const Tile tl = tiles[k];
@@ -557,30 +568,30 @@ __global__ void k_cartesian(BandDev *band) {
 template <typename T>
 void launch_mapback(const ImgRef *imgs, int count, BandDev *bands, int force, cudaStream_t s) {
     if (count <= 0) return;
-    k_mapback<T><<<count, 32, 0, s>>>(imgs, count, bands, force);
+    launch_dep(k_mapback<T>, count, 32, s, imgs, count, bands, force);
 }
 template <typename T>
 void launch_bin_assign(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s,
                        cudaGraphConditionalHandle cond, int has_cond) {
     if (ntiles <= 0) return;
-    k_bin_assign<T><<<ntiles, TILE, 0, s>>>(tiles, bands, cond, has_cond);
+    launch_dep(k_bin_assign<T>, ntiles, TILE, s, tiles, bands, cond, has_cond);
 }
 void launch_bin_scan(const ImgRef *imgs, int count, int max_bins, BandDev *bands,
                      cudaStream_t s, int part) {
     if (count <= 0 || max_bins <= 0) return;
     dim3 grid(std::min((max_bins + SCAN_TILE - 1) / SCAN_TILE, 32), count);
-    if (part == 0) k_bin_tilesum<<<grid, 256, 0, s>>>(imgs, bands);
-    else if (part == 1) k_bin_tilescan<<<count, 1024, 0, s>>>(imgs, bands);
-    else k_bin_scanfill<<<grid, 1024, 0, s>>>(imgs, bands);
+    if (part == 0) launch_dep(k_bin_tilesum, grid, 256, s, imgs, bands);
+    else if (part == 1) launch_dep(k_bin_tilescan, count, 1024, s, imgs, bands);
+    else launch_dep(k_bin_scanfill, grid, 1024, s, imgs, bands);
 }
 void launch_bin_scatter(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    k_bin_scatter<<<ntiles < gated_grid() ? ntiles : gated_grid(), TILE, 0, s>>>(tiles, ntiles, bands);
+    launch_dep(k_bin_scatter, ntiles < gated_grid() ? ntiles : gated_grid(), TILE, s, tiles, ntiles, bands);
 }
 template <typename T>
 void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    k_bin_order<T><<<ntiles < gated_grid() ? ntiles : gated_grid(), TILE, 0, s>>>(tiles, ntiles, bands);
+    launch_dep(k_bin_order<T>, ntiles < gated_grid() ? ntiles : gated_grid(), TILE, s, tiles, ntiles, bands);
 }
 template <typename T>
 void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {

@@ -219,7 +219,7 @@ __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandPa
 // Writes the generalised atom force F D^T of slot t (row vector times D^T)
 // and the tile's energy, virial and pair-count partials.
 template <typename T>
-__device__ inline void lj_finish(const LJAcc<T> &A, const LJGeom<T> &g, BandDev &b,
+__device__ inline void lj_finish(const LJAcc<T> &A, const LJGeom<T> &g, const BandDev &b,
                                  const Tile &tl, int t, bool active) {
     const T scale = sizeof(T) == 4 ? (T)1 : g.c24;
     if (active) {
@@ -409,6 +409,7 @@ __device__ inline void lj_disp(const LJDisp &D, uint32_t code, double &x, double
 template <typename T> __global__ void k_lj(const Tile *tiles, BandDev *bands);
 template <>
 __global__ void __launch_bounds__(TILE, 8) k_lj<float>(const Tile *tiles, BandDev *bands) {
+    dep_sync();
     Tile tl = tiles[blockIdx.x];
     BandDev &b = bands[tl.band];
     if (b.lj_cap > 0) return;  // uniform over the block: the list path runs
@@ -443,6 +444,7 @@ __global__ void __launch_bounds__(TILE, 8) k_lj<float>(const Tile *tiles, BandDe
 
 template <>
 __global__ void __launch_bounds__(TILE) k_lj<double>(const Tile *tiles, BandDev *bands) {
+    dep_sync();
     using T4 = typename Vec4<double>::type;
     Tile tl = tiles[blockIdx.x];
     BandDev &b = bands[tl.band];
@@ -558,7 +560,7 @@ __global__ void __launch_bounds__(TILE) k_lj_energy64(const Tile *tiles, BandDev
 // screen on their rounded offsets (entries are tested again in FP64 by the
 // force kernel).
 template <typename T>
-__device__ inline void lj_list_atom(BandDev &b, const Tile &tl, const LJGeom<float> &g, int t) {
+__device__ inline void lj_list_atom(const BandDev &b, const Tile &tl, const LJGeom<float> &g, int t) {
     const int n = b.n, cap = b.lj_cap;
     const size_t base = (size_t)tl.img * n;
     const float4 *off = screen_off<T>(b, base);
@@ -603,6 +605,7 @@ __device__ inline void lj_list_atom(BandDev &b, const Tile &tl, const LJGeom<flo
 
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles, BandDev *bands) {
+    dep_sync();
     __shared__ LJGeom<float> g;
     for (int k = blockIdx.x; k < ntiles; k += gridDim.x) {
         const Tile tl = tiles[k];
@@ -633,8 +636,9 @@ template <int MINB>
 __global__ void __launch_bounds__(TILE, MINB) k_lj_nbr(const Tile *tiles, BandDev *bands) {
     using T = float;
     using T4 = float4;
-    Tile tl = tiles[blockIdx.x];
-    BandDev &b = bands[tl.band];
+    const Tile tl = tiles[blockIdx.x];
+    const BandDev b = bands[tl.band];
+    dep_sync();
     if (b.lj_cap == 0) return;  // uniform over the block: the direct path runs
     const ImgScalars &sc = b.sc[tl.img];
     __shared__ LJGeom<T> g;
@@ -720,8 +724,9 @@ struct LJDispF {  // LJDisp rounded, for the screen
 };
 __global__ void __launch_bounds__(TILE, 4) k_lj_nbr64(const Tile *tiles, BandDev *bands) {
     using T4 = typename Vec4<double>::type;
-    Tile tl = tiles[blockIdx.x];
-    BandDev &b = bands[tl.band];
+    const Tile tl = tiles[blockIdx.x];
+    const BandDev b = bands[tl.band];
+    dep_sync();
     if (b.lj_cap == 0) return;  // uniform over the block: the direct path runs
     const ImgScalars &sc = b.sc[tl.img];
     __shared__ LJGeom<double> g;
@@ -789,7 +794,7 @@ __global__ void __launch_bounds__(TILE, 4) k_lj_nbr64(const Tile *tiles, BandDev
 template <typename T>
 void launch_lj(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    k_lj<T><<<ntiles, TILE, 0, s>>>(tiles, bands);
+    launch_dep(k_lj<T>, ntiles, TILE, s, tiles, bands);
 }
 template <typename T>
 void launch_lj_list(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
@@ -797,20 +802,20 @@ void launch_lj_list(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t 
     // a block per tile: a build walks ~370 candidates per atom, and in a
     // batch of many bands a large share of the images rebuilds at a time
     // (a capped grid was measured slower here)
-    k_lj_list<T><<<ntiles, TILE, 0, s>>>(tiles, ntiles, bands);
+    launch_dep(k_lj_list<T>, ntiles, TILE, s, tiles, ntiles, bands);
 }
 template <typename T>
 void launch_lj_nbr(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s, int minb) {
     if (ntiles <= 0) return;
     if (sizeof(T) == 8) {
-        k_lj_nbr64<<<ntiles, TILE, 0, s>>>(tiles, bands);
+        launch_dep(k_lj_nbr64, ntiles, TILE, s, tiles, bands);
         return;
     }
     switch (minb) {
-        case 5: k_lj_nbr<5><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
-        case 6: k_lj_nbr<6><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
-        case 8: k_lj_nbr<8><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
-        default: k_lj_nbr<7><<<ntiles, TILE, 0, s>>>(tiles, bands); break;
+        case 5: launch_dep(k_lj_nbr<5>, ntiles, TILE, s, tiles, bands); break;
+        case 6: launch_dep(k_lj_nbr<6>, ntiles, TILE, s, tiles, bands); break;
+        case 8: launch_dep(k_lj_nbr<8>, ntiles, TILE, s, tiles, bands); break;
+        default: launch_dep(k_lj_nbr<7>, ntiles, TILE, s, tiles, bands); break;
     }
 }
 template <typename T>
