@@ -449,7 +449,7 @@ int cfneb_get_list_stats(const cfneb_band *band, int64_t *builds, int64_t *evalu
 
 /* Number of kernel launches one cfneb_step makes for this band when it
  * rebuilds cell and neighbour lists (for launch accounting; a step in which
- * every image keeps its lists skips the 6-7 rebuild kernels). */
+ * every image keeps its lists skips the rebuild kernels, or their work). */
 int cfneb_launches_per_step(const cfneb_band *band, int32_t *launches);
 
 /* ---- evaluation without device allocation --------------------------------

@@ -512,6 +512,18 @@ __global__ void __launch_bounds__(TILE) k_bin_scatter(const Tile *tiles, int nti
     }
 }
 
+// Atom i of an image (whose arrays begin at base) takes slot dst of bin pb.
+template <typename T>
+__device__ inline void order_atom(const BandDev &b, size_t base, int i, int dst, int pb,
+                                  const typename Vec4<T>::type &o, const float4 &ol) {
+    b.slot_atom[base + dst] = i;
+    b.slot_bin[base + dst] = pb;
+    b.atom_slot[base + i] = dst;
+    ((typename Vec4<T>::type *)b.slot_off)[base + dst] = o;
+    b.slot_off_lo[base + dst] = ol;
+    if (b.slot_wrap) b.slot_wrap[base + dst] = wrap_place(b.atom_wrap + (base + i) * 3);
+}
+
 // Order each bin's atoms by atom index and write the sorted slot arrays: one
 // thread per atom, its rank among its bin's atoms counted from the unordered
 // slots.  (One thread per bin left the chip to a few threads with quadratic
@@ -537,14 +549,90 @@ __global__ void __launch_bounds__(TILE) k_bin_order(const Tile *tiles, int ntile
         const int s0 = start[bin], s1 = start[bin + 1];
         int dst = s0;
         for (int q = s0; q < s1; ++q) dst += un[q] < i;
-        b.slot_atom[base + dst] = i;
-        b.slot_bin[base + dst] = pack_bin(bin / (nb1 * nb2), (bin / nb2) % nb1, bin % nb2);
-        b.atom_slot[base + i] = dst;
-        ((T4 *)b.slot_off)[base + dst] = o;
-        b.slot_off_lo[base + dst] = ol;
-        if (b.slot_wrap) {
-            b.slot_wrap[base + dst] = wrap_place(b.atom_wrap + (base + i) * 3);
+        order_atom<T>(b, base, i, dst, pack_bin(bin / (nb1 * nb2), (bin / nb2) % nb1, bin % nb2), o,
+                      ol);
+    }
+}
+
+// The scan, scatter and order passes of an image in one launch, for bands of at
+// most SORT_ATOMS atoms and SORT_CAP bins (launch latency bounds those passes
+// there): a cluster of SORT_CL blocks per image, every block scanning the image's
+// counts into its own shared memory (16 bits hold them), the atoms shared out over
+// the blocks, one cluster barrier between the unordered slots and the order.  With
+// more than SORT_BINS bins the scan goes by chunks and the starts are read back
+// from memory.  Same slots as the five passes.
+static_assert(SORT_ATOMS < 65536, "bin starts are kept in 16 bits");
+template <typename T>
+__global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
+    k_bin_sort(const ImgRef *imgs, BandDev *bands) {
+    using T4 = typename Vec4<T>::type;
+    const ImgRef r = imgs[blockIdx.x / SORT_CL];
+    const BandDev b = bands[r.band];
+    const ImgScalars &sc = b.sc[r.img];
+    dep_sync();
+    if (!sc.rebuild) return;  // uniform over the cluster
+    __shared__ unsigned short s_start[SORT_BINS];
+    __shared__ int s_w[SORT_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int first = (int)(blockIdx.x % SORT_CL) * SORT_THREADS + tid;
+    constexpr int STEP = SORT_CL * SORT_THREADS;
+    const int n = b.n, nb = sc.nbins, nb1 = sc.nb[1], nb2 = sc.nb[2];
+    const size_t base = (size_t)r.img * n;
+    int *cnt = b.bin_count + (size_t)r.img * b.nbins_cap;
+    int *start = b.bin_start + (size_t)r.img * (b.nbins_cap + 1);
+    int before = 0;  // atoms of the chunks before
+    for (int c = 0; c < nb; c += SORT_BINS) {
+        const int m = min(SORT_BINS, nb - c);
+        for (int k = tid; k < m; k += SORT_THREADS) s_start[k] = (unsigned short)cnt[c + k];
+        __syncthreads();
+        // an odd number of bins per thread spreads the threads over the banks
+        const int per = ((m + SORT_THREADS - 1) / SORT_THREADS) | 1;
+        const int k0 = min(tid * per, m), k1 = min(k0 + per, m);
+        int sum = 0;
+        for (int k = k0; k < k1; ++k) sum += s_start[k];
+        int inc = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
         }
+        if (lane == 31) s_w[w] = inc;
+        __syncthreads();
+        int run = before + inc - sum;
+        for (int q = 0; q < SORT_THREADS / 32; ++q) {
+            if (q < w) run += s_w[q];
+            before += s_w[q];
+        }
+        for (int k = k0; k < k1; ++k) {
+            const int v = s_start[k];
+            s_start[k] = (unsigned short)run;
+            run += v;
+        }
+        __syncthreads();
+        for (int k = first; k < m; k += STEP) start[c + k] = s_start[k];
+        if (c + m < nb) __syncthreads();  // the next chunk takes this one's place
+    }
+    if (first == 0) start[nb] = n;
+    const bool held = nb <= SORT_BINS;  // uniform over the cluster
+    if (!held) cluster_barrier();
+    // what the cluster's other blocks wrote is read from L2
+    const auto start_of = [&](int k) {
+        return held ? (k < nb ? (int)s_start[k] : n) : __ldcg(start + k);
+    };
+    int *un = b.slot_unsorted + base;
+    for (int i = first; i < n; i += STEP)
+        un[start_of(b.atom_bin[base + i]) + b.atom_rank[base + i]] = i;
+    cluster_barrier();
+    // every block has read the counts: zero for the next build
+    for (int k = first; k < nb; k += STEP) cnt[k] = 0;
+    for (int i = first; i < n; i += STEP) {
+        const int bin = b.atom_bin[base + i];
+        const T4 o = ((const T4 *)b.atom_off)[base + i];
+        const float4 ol = b.atom_off_lo[base + i];
+        const int s0 = start_of(bin), s1 = start_of(bin + 1);
+        int dst = s0;
+        for (int q = s0; q < s1; ++q) dst += __ldcg(un + q) < i;
+        order_atom<T>(b, base, i, dst, pack_bin(bin / (nb1 * nb2), (bin / nb2) % nb1, bin % nb2), o,
+                      ol);
     }
 }
 
@@ -594,6 +682,11 @@ void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_
     launch_dep(k_bin_order<T>, ntiles < gated_grid() ? ntiles : gated_grid(), TILE, s, tiles, ntiles, bands);
 }
 template <typename T>
+void launch_bin_sort(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t s) {
+    if (count <= 0) return;
+    launch_dep(k_bin_sort<T>, count * SORT_CL, SORT_THREADS, s, imgs, bands);
+}
+template <typename T>
 void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {
     if (N <= 0 || n <= 0) return;
     dim3 grid((n + 127) / 128, N);
@@ -605,6 +698,7 @@ void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {
     template void launch_bin_assign<T>(const Tile *, int, BandDev *, cudaStream_t,       \
                                        cudaGraphConditionalHandle, int);                 \
     template void launch_bin_order<T>(const Tile *, int, BandDev *, cudaStream_t);        \
+    template void launch_bin_sort<T>(const ImgRef *, int, BandDev *, cudaStream_t);       \
     template void launch_cartesian<T>(int, int, BandDev *, cudaStream_t);
 CFNEB_INST(float)
 CFNEB_INST(double)

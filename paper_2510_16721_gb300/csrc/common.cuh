@@ -85,6 +85,13 @@ inline void launch_dep(void (*k)(P...), dim3 grid, int block, cudaStream_t s, A.
     c.numAttrs = 1;
     cudaLaunchKernelEx(&c, k, static_cast<P>(a)...);
 }
+// The force kernels go out only once the kernel before is complete: placed among
+// its last blocks, two of theirs would share an SM's arithmetic while other SMs
+// idle (576 carbon atoms, FP64, 126 blocks of site terms: 85 -> 102 us per step).
+template <typename... P, typename... A>
+inline void launch_even(void (*k)(P...), dim3 grid, int block, cudaStream_t s, A... a) {
+    k<<<grid, block, 0, s>>>(static_cast<P>(a)...);
+}
 // In every kernel that launch_dep starts, before its first access to anything a
 // kernel writes: wait until the kernels before are complete and their writes
 // visible, then let the next kernel's blocks be placed as this grid drains.  (The
@@ -96,6 +103,13 @@ __device__ __forceinline__ void dep_sync() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// Barrier of a thread block cluster; what its threads wrote before, to shared or
+// global memory, is visible to all of them after.
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // potential kinds of BandParams::kind (the values of include/cfneb.h)
 constexpr int KIND_LJ = 0, KIND_TERSOFF = 1, KIND_NEP = 2;
 
@@ -1143,6 +1157,11 @@ void launch_bin_assign(const Tile *tiles, int ntiles, BandDev *bands, cudaStream
 void launch_bin_scan(const ImgRef *imgs, int count, int max_bins, BandDev *bands,
                      cudaStream_t s, int part);
 void launch_bin_scatter(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
+// Images that k_bin_sort takes (cell.cu)
+constexpr int SORT_CL = 8, SORT_THREADS = 512, SORT_BINS = 16384;
+constexpr int SORT_ATOMS = 28672, SORT_CAP = 8 * SORT_BINS;
+template <typename T>
+void launch_bin_sort(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t s);
 template <typename T>
 void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s);
 template <typename T>

@@ -309,6 +309,7 @@ struct LaunchSet {
     const int *band_ids = nullptr;
     int nbands = 0;
     int max_bins = 0;                    // largest nbins_cap among the bands
+    int max_n = 0;                       // largest number of atoms among them
     int force_rebuild = REBUILD_ASKED;   // which images rebuild their cell lists regardless
     int lj_minb = kLjMinb, ters_minb = kTersMinb;  // force kernel variants
     cudaStream_t s_body = nullptr;       // captures the conditional rebuild body
@@ -334,6 +335,20 @@ struct Launcher {
     }
 };
 
+// Whether the cell list's scan, scatter and order are one launch (k_bin_sort).
+// Five passes and a conditional node -> one: 40 steps with ~3 rebuilds, per step,
+// mixed LJ 10,975 atoms x 7 images 95.7 -> 88.4 us, 27,435 atoms 131.9 -> 125.5 us;
+// 384 carbon atoms 64.4 -> 54.6, 12,288 x 9 66.2 -> 59.1.  At most seven atoms per
+// thread of the cluster: the gain shrinks beyond (30,720 x 9: 86.1 -> 81.4).
+bool one_sort(const LaunchSet &ls) { return ls.max_n <= SORT_ATOMS && ls.max_bins <= SORT_CAP; }
+
+// Whether a graph holds the rebuild in a conditional node.  A node that is not
+// taken costs 5.0-5.7 us and breaks the chain of overlapped launches; kernels that
+// run and skip cost 0.7 us each and more with their grids.  30,720 carbon atoms x 7
+// images 86.5 us per step with the node and 83.0 without, 61,440 atoms (3,360
+// tiles) 117.2 and 115.9, 98,304 (5,376) 159.4 and 160.2.
+bool cond_rebuild(const LaunchSet &ls) { return !one_sort(ls) && ls.n_atiles > 4096; }
+
 // cell-list scan, scatter and order, then the neighbour lists (they index
 // cell-list slots, so they are rebuilt with every cell list, also by an
 // energy-only evaluation); each kernel skips the images that keep theirs
@@ -341,11 +356,20 @@ template <typename T>
 void enqueue_rebuild(const LaunchSet &ls, Launcher &L) {
     BandDev *d = ls.d_bands;
     cudaStream_t s = ls.s;
-    L.pre(K_BIN_TILESUM); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 0); L.post(K_BIN_TILESUM);
-    L.pre(K_BIN_TILESCAN); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 1); L.post(K_BIN_TILESCAN);
-    L.pre(K_BIN_SCANFILL); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 2); L.post(K_BIN_SCANFILL);
-    L.pre(K_BIN_SCATTER); launch_bin_scatter(ls.atiles, ls.n_atiles, d, s); L.post(K_BIN_SCATTER);
-    L.pre(K_BIN_ORDER); launch_bin_order<T>(ls.atiles, ls.n_atiles, d, s); L.post(K_BIN_ORDER);
+    if (one_sort(ls)) {
+        L.pre(K_BIN_ORDER); launch_bin_sort<T>(ls.imgs, ls.nimg, d, s); L.post(K_BIN_ORDER);
+    } else {
+        L.pre(K_BIN_TILESUM); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 0);
+        L.post(K_BIN_TILESUM);
+        L.pre(K_BIN_TILESCAN); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 1);
+        L.post(K_BIN_TILESCAN);
+        L.pre(K_BIN_SCANFILL); launch_bin_scan(ls.imgs, ls.nimg, ls.max_bins, d, s, 2);
+        L.post(K_BIN_SCANFILL);
+        L.pre(K_BIN_SCATTER); launch_bin_scatter(ls.atiles, ls.n_atiles, d, s);
+        L.post(K_BIN_SCATTER);
+        L.pre(K_BIN_ORDER); launch_bin_order<T>(ls.atiles, ls.n_atiles, d, s);
+        L.post(K_BIN_ORDER);
+    }
     // the neighbour lists index cell-list slots: they are rebuilt with every
     // cell list, also by an energy-only evaluation
     if (ls.n_lj) {
@@ -374,14 +398,14 @@ void enqueue_eval_set(const LaunchSet &ls, Launcher &L, bool forces = true) {
     // (k_fire_update); then map-back and the list decision
     L.pre(K_MAPBACK); launch_mapback<T>(ls.imgs, ls.nimg, d, ls.force_rebuild, s);
     L.post(K_MAPBACK);
-    // the cell-list and neighbour-list rebuild: inside a graph capture it
-    // goes into the body of a conditional node that runs only in steps
-    // where some image rebuilds (most steps keep every list; bin_assign
-    // switches the node on); outside a capture its kernels run and skip the
-    // images that keep their lists
+    // the cell-list and neighbour-list rebuild: its kernels run and skip the
+    // images that keep their lists; inside a graph capture a large set's go
+    // into the body of a conditional node that runs only in steps where some
+    // image rebuilds (bin_assign switches the node on)
     cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(s, &cst));
-    const bool cond_node = cst == cudaStreamCaptureStatusActive && ls.s_body && !L.prof;
+    const bool cond_node = cst == cudaStreamCaptureStatusActive && ls.s_body && !L.prof &&
+                           cond_rebuild(ls);
     cudaGraphConditionalHandle cond = 0;
     if (cond_node) {
         cudaGraph_t graph = nullptr;
@@ -484,13 +508,13 @@ void enqueue_step_set(const LaunchSet &ls, Launcher &L) {
     L.post(K_FIRE_UPDATE);
 }
 
-// launches of a step when it rebuilds lists (the graph's conditional node
-// skips the 5 cell-list and 1-2 neighbour-list kernels in other steps):
-// map-back, bin_assign and the 5 list kernels, the force kernels, the
-// finalize and the three band passes
+// launches of a step when it rebuilds lists (in other steps the 1 or 5 cell-list
+// and 1-2 neighbour-list kernels skip, or the graph's conditional node skips
+// them): map-back, bin_assign and the cell-list kernels, the list and force
+// kernels, the finalize and the three band passes
 int launches_in_set(const LaunchSet &ls) {
-    return 7 + (ls.n_lj ? 2 : 0) + (ls.n_ljc ? 1 : 0) + (ls.n_ters ? 4 : 0) + (ls.n_nep ? 4 : 0) +
-           1 + 3;
+    return (one_sort(ls) ? 3 : 7) + (ls.n_lj ? 2 : 0) + (ls.n_ljc ? 1 : 0) +
+           (ls.n_ters ? 4 : 0) + (ls.n_nep ? 4 : 0) + 1 + 3;
 }
 
 LaunchSet band_set(cfneb_band *b, const ImgRef *imgs, int nimg, const Tile *atiles, int nat) {
@@ -519,6 +543,7 @@ LaunchSet band_set(cfneb_band *b, const ImgRef *imgs, int nimg, const Tile *atil
     ls.band_ids = b->d_band_ids;
     ls.nbands = 1;
     ls.max_bins = b->dv.nbins_cap;
+    ls.max_n = b->n;
     ls.s_body = b->s_body;
     ls.fork = &b->fork;
     if (b->minb > 0) {
@@ -1156,6 +1181,7 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
     (lj ? ls.atiles_ljc : pot->kind == CFNEB_NEP ? ls.atiles_nep : ls.atiles_ters) = d_tiles;
     (lj ? ls.n_ljc : pot->kind == CFNEB_NEP ? ls.n_nep : ls.n_ters) = (int)tiles.size();
     ls.max_bins = max_bins;
+    ls.max_n = (int)big;
     ls.force_rebuild = REBUILD_ALL;
     if (minb > 0 && pot->kind == CFNEB_TERSOFF) ls.ters_minb = minb;
     launch_points_load<T>(d_tiles, ls.n_atiles, d_bands, s);
@@ -1550,9 +1576,10 @@ void batch_rebuild(cfneb_batch *bt) {
     std::vector<ImgRef> im;
     std::vector<Tile> all, lj, ljc, ters, nep, rows;
     std::vector<int> ids;
-    int max_bins = 0;
+    int max_bins = 0, max_n = 0;
     for (size_t k = 0; k < bt->bands.size(); ++k) {
         cfneb_band *b = bt->bands[k];
+        max_n = std::max(max_n, b->n);
         dv.push_back(b->dv);
         ids.push_back((int)k);
         max_bins = std::max(max_bins, b->dv.nbins_cap);
@@ -1617,6 +1644,7 @@ void batch_rebuild(cfneb_batch *bt) {
     ls.band_ids = bt->d_ids;
     ls.nbands = (int)ids.size();
     ls.max_bins = max_bins;
+    ls.max_n = max_n;
     ls.s_body = bt->s_body;
     ls.fork = &bt->fork;
     if (bt->lj_minb) ls.lj_minb = bt->lj_minb;

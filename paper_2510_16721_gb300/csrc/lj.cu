@@ -794,7 +794,7 @@ __global__ void __launch_bounds__(TILE, 4) k_lj_nbr64(const Tile *tiles, BandDev
 template <typename T>
 void launch_lj(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    launch_dep(k_lj<T>, ntiles, TILE, s, tiles, bands);
+    launch_even(k_lj<T>, ntiles, TILE, s, tiles, bands);
 }
 template <typename T>
 void launch_lj_list(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
@@ -808,14 +808,14 @@ template <typename T>
 void launch_lj_nbr(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s, int minb) {
     if (ntiles <= 0) return;
     if (sizeof(T) == 8) {
-        launch_dep(k_lj_nbr64, ntiles, TILE, s, tiles, bands);
+        launch_even(k_lj_nbr64, ntiles, TILE, s, tiles, bands);
         return;
     }
     switch (minb) {
-        case 5: launch_dep(k_lj_nbr<5>, ntiles, TILE, s, tiles, bands); break;
-        case 6: launch_dep(k_lj_nbr<6>, ntiles, TILE, s, tiles, bands); break;
-        case 8: launch_dep(k_lj_nbr<8>, ntiles, TILE, s, tiles, bands); break;
-        default: launch_dep(k_lj_nbr<7>, ntiles, TILE, s, tiles, bands); break;
+        case 5: launch_even(k_lj_nbr<5>, ntiles, TILE, s, tiles, bands); break;
+        case 6: launch_even(k_lj_nbr<6>, ntiles, TILE, s, tiles, bands); break;
+        case 8: launch_even(k_lj_nbr<8>, ntiles, TILE, s, tiles, bands); break;
+        default: launch_even(k_lj_nbr<7>, ntiles, TILE, s, tiles, bands); break;
     }
 }
 template <typename T>

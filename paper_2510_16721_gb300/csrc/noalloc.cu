@@ -222,11 +222,16 @@ extern "C" int cfneb_lj_evaluate_noalloc(const double *d_positions, int32_t n_at
     launch_points_load<double>(d_tiles, dv.atpi, d_band, s);
     launch_mapback<double>(d_img, 1, d_band, REBUILD_ALL, s);  // the scratch record is reused
     launch_bin_assign<double>(d_tiles, dv.atpi, d_band, s);
-    launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 0);
-    launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 1);
-    launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 2);
-    launch_bin_scatter(d_tiles, dv.atpi, d_band, s);
-    launch_bin_order<double>(d_tiles, dv.atpi, d_band, s);
+    static_assert(NA_MAX_BINS <= SORT_CAP, "k_bin_sort takes every grid of the scratch memory");
+    if (n <= SORT_ATOMS) {
+        launch_bin_sort<double>(d_img, 1, d_band, s);
+    } else {
+        launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 0);
+        launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 1);
+        launch_bin_scan(d_img, 1, NA_MAX_BINS, d_band, s, 2);
+        launch_bin_scatter(d_tiles, dv.atpi, d_band, s);
+        launch_bin_order<double>(d_tiles, dv.atpi, d_band, s);
+    }
     launch_lj<double>(d_tiles, dv.atpi, d_band, s);
     launch_image_finalize<double>(d_img, 1, d_band, s);
     if (cudaGetLastError() != cudaSuccess) return CFNEB_ERR_CUDA;
