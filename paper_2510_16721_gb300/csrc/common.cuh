@@ -272,7 +272,8 @@ struct BandDev {
     void *atom_off, *slot_off;   // [ncap][n] x 4 T (x, y, z, pad): offsets, leading part
     // Offsets are FP64 or (FP32 LJ bands) FP32 from the atom's bin centre; FP32
     // many-body bands hold positions in the cell instead, as integers of the
-    // image's grid (int4) and FP32 remainders (float4): see grid_split.
+    // image's grid (int4) and FP32 remainders (float4): see grid_split; by slot one
+    // record of the two, so that a neighbour costs one 32-byte load.
     // [ncap][n] x float4.  FP32 bands: offset - leading part.  FP64 bands: the
     // offset rounded to FP32 (and the bin index), for distance screens
     float4 *atom_off_lo, *slot_off_lo;
@@ -285,7 +286,7 @@ struct BandDev {
     // entries, or LJ packed entries of lj_cap (0: the LJ kernel walks the
     // cell list directly)
     int lj_cap;
-    int *nbr_cnt;        // [ncap][n]
+    int *nbr_cnt;        // [ncap][n]; many-body lists: | NBR_SHIFTED if an entry's code is not CODE_ZERO
     int *nbr_slot;       // [ncap][MAXN or lj_cap][n]
     int *nbr_code;       // [ncap][MAXN][n]
     unsigned char *nbr_rev;  // [ncap][MAXN][n]: entry of j's list pointing back (255: none)
@@ -1088,6 +1089,7 @@ struct GridF {
     float4 lo[SHIFTS];  // its remainder
 };
 constexpr int CODE_ZERO = 16 | (16 << 5) | (16 << 10);
+constexpr int NBR_SHIFTED = 256, NBR_COUNT = 255;
 __device__ inline void grid_stage(GridF &G, const BandDev &b, int img) {
     const int *sh = b.shift + (size_t)img * SHIFTS * 6;
     if (threadIdx.x < SHIFTS) {
@@ -1099,6 +1101,15 @@ __device__ inline void grid_stage(GridF &G, const BandDev &b, int img) {
     if (threadIdx.x == 32) G.g = b.sc[img].grid;
     if (threadIdx.x == 33) G.ig = b.sc[img].igrid;
 }
+// A slot's position record: integers (as float bits) and remainders
+__device__ __forceinline__ void load_pos(const float4 *p, float4 &i, float4 &lo) {
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(i.x), "=f"(i.y), "=f"(i.z), "=f"(i.w), "=f"(lo.x), "=f"(lo.y), "=f"(lo.z), "=f"(lo.w)
+        : "l"(p)
+        : "memory");
+}
+__device__ inline int grid_diff(float a, float b) { return __float_as_int(a) - __float_as_int(b); }
+
 // The shift of a code: the table's, or (cells narrower than the list cutoff)
 // formed from the cell
 __device__ inline void grid_shift(const GridF &G, const ImgScalars &sc, int code, int (&s)[3],

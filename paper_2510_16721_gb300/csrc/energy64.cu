@@ -43,24 +43,23 @@ __device__ inline int entries64(const BandDev &b, const Tile &tl, int t, double 
                                 const GridF &G, Entries64 &E, float) {
     const ImgScalars &sc = b.sc[tl.img];
     const size_t base = (size_t)tl.img * b.n;
-    const int4 *pos = (const int4 *)b.slot_off + base;
-    const float4 *rem = b.slot_off_lo + base;
+    const float4 *pos = (const float4 *)b.slot_off + 2 * base;
     const int *nslot = b.nbr_slot + base * MAXN_TERSOFF;
     const int *ncode = b.nbr_code + base * MAXN_TERSOFF;
-    const int ne = b.nbr_cnt[base + t];
-    const int4 pi = pos[t];
-    const float4 li = rem[t];
+    const int ne = b.nbr_cnt[base + t] & NBR_COUNT;
+    float4 pi, li;
+    load_pos(pos + 2 * t, pi, li);
     int cnt = 0;
     for (int e = 0; e < ne; ++e) {
         const int q = nslot[(size_t)e * b.n + t], code = ncode[(size_t)e * b.n + t];
-        const int4 pj = pos[q];
-        const float4 lj = rem[q];
+        float4 pj, lj;
+        load_pos(pos + 2 * q, pj, lj);
         int s[3] = {0, 0, 0};
         float lo[3] = {0.0f, 0.0f, 0.0f};
         if (code != CODE_ZERO) grid_shift(G, sc, code, s, lo);
-        const double x = f2d((float)(pj.x - pi.x + s[0]) * G.g) + f2d((lj.x - li.x) + lo[0]);
-        const double y = f2d((float)(pj.y - pi.y + s[1]) * G.g) + f2d((lj.y - li.y) + lo[1]);
-        const double z = f2d((float)(pj.z - pi.z + s[2]) * G.g) + f2d((lj.z - li.z) + lo[2]);
+        const double x = f2d((float)(grid_diff(pj.x, pi.x) + s[0]) * G.g) + f2d((lj.x - li.x) + lo[0]);
+        const double y = f2d((float)(grid_diff(pj.y, pi.y) + s[1]) * G.g) + f2d((lj.y - li.y) + lo[1]);
+        const double z = f2d((float)(grid_diff(pj.z, pi.z) + s[2]) * G.g) + f2d((lj.z - li.z) + lo[2]);
         cnt += add_entry(E, cnt, x, y, z, rc * rc);
     }
     return cnt;
@@ -72,7 +71,7 @@ __device__ inline int entries64(const BandDev &b, const Tile &tl, int t, double 
     const double4_32a *off = (const double4_32a *)b.slot_off + base;
     const int *nslot = b.nbr_slot + base * MAXN_TERSOFF;
     const int *ncode = b.nbr_code + base * MAXN_TERSOFF;
-    const int ne = b.nbr_cnt[base + t];
+    const int ne = b.nbr_cnt[base + t] & NBR_COUNT;
     int b0, b1, b2;
     unpack_bin(b.slot_bin[base + t], b0, b1, b2);
     const double4_32a oi = off[t];

@@ -1128,16 +1128,19 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
                         &d.atom_slot})
             ar.add(p, na * sizeof(int));
         ar.add(&d.atom_off, na * 4 * sizeof(T));
-        ar.add(&d.slot_off, na * 4 * sizeof(T));
+        const bool records = !lj && sizeof(T) == 4;  // positions in one 32-byte record
+        ar.add(&d.slot_off, na * 4 * sizeof(T) * (records ? 2 : 1));
         ar.add(&d.atom_off_lo, na * sizeof(float4));
-        ar.add(&d.slot_off_lo, na * sizeof(float4));
+        if (!records) ar.add(&d.slot_off_lo, na * sizeof(float4));
         if (!lj) {
             ar.add(&d.nbr_cnt, na * sizeof(int));
             ar.add(&d.nbr_slot, na * MAXN_TERSOFF * sizeof(int));
             ar.add(&d.nbr_code, na * MAXN_TERSOFF * sizeof(int));
             ar.add(&d.nbr_rev, na * MAXN_TERSOFF);
             ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * sizeof(T));
-            if (sizeof(T) == 4) ar.add(&d.shift, SHIFTS * 6 * sizeof(int));
+            if (records) {
+                ar.add(&d.shift, SHIFTS * 6 * sizeof(int));
+                }
         }
         ar.add(&d.atom_part, (size_t)d.atpi * NPART * sizeof(double));
     }
@@ -1340,9 +1343,10 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
                     &d.atom_slot})
         ar.add(p, na * sizeof(int));
     ar.add(&d.atom_off, na * 4 * b->ts);
-    ar.add(&d.slot_off, na * 4 * b->ts);
+    const bool records = many && b->ts == 4;  // positions in one 32-byte record
+    ar.add(&d.slot_off, na * 4 * b->ts * (records ? 2 : 1));
     ar.add(&d.atom_off_lo, na * sizeof(float4));
-    ar.add(&d.slot_off_lo, na * sizeof(float4));
+    if (!records) ar.add(&d.slot_off_lo, na * sizeof(float4));
     if (skin > 0.0) {
         ar.add(&d.atom_wrap, na * 3 * sizeof(int));
         if (many && b->ts == 4) ar.add(&d.slot_wrap, na * sizeof(int));
@@ -1357,7 +1361,7 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
         ar.add(&d.nbr_code, na * MAXN_TERSOFF * sizeof(int));
         ar.add(&d.nbr_rev, na * MAXN_TERSOFF);
         ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * b->ts);
-        if (b->ts == 4) ar.add(&d.shift, nc * SHIFTS * 6 * sizeof(int));
+        if (records) ar.add(&d.shift, nc * SHIFTS * 6 * sizeof(int));
     }
     ar.add(&d.atom_part, nc * d.atpi * NPART * sizeof(double));
     ar.add(&d.row_part, nc * d.rtpi * NPART * sizeof(double));
