@@ -287,12 +287,18 @@ struct BandDev {
     // cell list directly)
     int lj_cap;
     int *nbr_cnt;        // [ncap][n]; many-body lists: | NBR_SHIFTED if an entry's code is not CODE_ZERO
-    int *nbr_slot;       // [ncap][MAXN or lj_cap][n]
-    int *nbr_code;       // [ncap][MAXN][n]
-    unsigned char *nbr_rev;  // [ncap][MAXN][n]: entry of j's list pointing back (255: none)
+    // many-body lists: [ncap][MAXN / 4][n][4] (ent: four entries of an atom are one
+    // vector); LJ lists: nbr_slot [ncap][lj_cap][n]
+    int *nbr_slot;
+    int *nbr_code;
+    unsigned char *nbr_rev;  // entry of j's list pointing back (255: none)
     const double *nep_w;     // NEP weights [NEP_NW] in FP64 and FP32 (NEP bands)
     const float *nep_wf;
-    void *nbr_P;         // [ncap][MAXN][n] x 4 T: partials (x, y, z, pad)
+    // [ncap][MAXN][n] x 4 T: partials (x, y, z, pad).  FP64: P_ij at atom i's entry
+    // j.  FP32: P_ij at the entry of atom j that points back to i, and the sum over
+    // an atom's own entries in site_P [ncap][n]
+    void *nbr_P;
+    float4 *site_P;
     // partial sums
     int *shift;          // [ncap][27][6]: lattice shifts on the grid (FP32 many-body bands)
     double *atom_part;   // [ncap][atpi][NPART]
@@ -1090,6 +1096,8 @@ struct GridF {
 };
 constexpr int CODE_ZERO = 16 | (16 << 5) | (16 << 10);
 constexpr int NBR_SHIFTED = 256, NBR_COUNT = 255;
+// Place of entry k of atom t in an image's many-body list
+__device__ inline size_t ent(int k, int t, int n) { return ((size_t)(k >> 2) * n + t) * 4 + (k & 3); }
 __device__ inline void grid_stage(GridF &G, const BandDev &b, int img) {
     const int *sh = b.shift + (size_t)img * SHIFTS * 6;
     if (threadIdx.x < SHIFTS) {

@@ -51,7 +51,7 @@ __device__ inline int entries64(const BandDev &b, const Tile &tl, int t, double 
     load_pos(pos + 2 * t, pi, li);
     int cnt = 0;
     for (int e = 0; e < ne; ++e) {
-        const int q = nslot[(size_t)e * b.n + t], code = ncode[(size_t)e * b.n + t];
+        const int q = nslot[ent(e, t, b.n)], code = ncode[ent(e, t, b.n)];
         float4 pj, lj;
         load_pos(pos + 2 * q, pj, lj);
         int s[3] = {0, 0, 0};
@@ -77,9 +77,9 @@ __device__ inline int entries64(const BandDev &b, const Tile &tl, int t, double 
     const double4_32a oi = off[t];
     int cnt = 0;
     for (int e = 0; e < ne; ++e) {
-        const double4_32a oj = off[nslot[(size_t)e * b.n + t]];
+        const double4_32a oj = off[nslot[ent(e, t, b.n)]];
         int d[3], w[3];
-        ters_code(ncode[(size_t)e * b.n + t], b0, b1, b2, sc.nb, d, w);
+        ters_code(ncode[ent(e, t, b.n)], b0, b1, b2, sc.nb, d, w);
         double v[3] = {oj.x - oi.x, oj.y - oi.y, oj.z - oi.z};
         for (int c = 0; c < 3; ++c) {
             v[c] += f2d(d[0] * sc.bvf[c] + d[1] * sc.bvf[3 + c] + d[2] * sc.bvf[6 + c]);

@@ -1140,7 +1140,8 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
             ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * sizeof(T));
             if (records) {
                 ar.add(&d.shift, SHIFTS * 6 * sizeof(int));
-                }
+                ar.add(&d.site_P, na * sizeof(float4));
+            }
         }
         ar.add(&d.atom_part, (size_t)d.atpi * NPART * sizeof(double));
     }
@@ -1361,7 +1362,10 @@ cfneb_band *create(const cfneb_structure *A, const cfneb_structure *B, int N,
         ar.add(&d.nbr_code, na * MAXN_TERSOFF * sizeof(int));
         ar.add(&d.nbr_rev, na * MAXN_TERSOFF);
         ar.add(&d.nbr_P, na * 4 * MAXN_TERSOFF * b->ts);
-        if (records) ar.add(&d.shift, nc * SHIFTS * 6 * sizeof(int));
+        if (records) {
+            ar.add(&d.shift, nc * SHIFTS * 6 * sizeof(int));
+            ar.add(&d.site_P, na * sizeof(float4));
+        }
     }
     ar.add(&d.atom_part, nc * d.atpi * NPART * sizeof(double));
     ar.add(&d.row_part, nc * d.rtpi * NPART * sizeof(double));
