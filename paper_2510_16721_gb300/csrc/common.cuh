@@ -322,6 +322,19 @@ __device__ inline int tile_atom(const BandDev &b, const Tile &tl) {
     return (int)threadIdx.x < b.tile ? tl.t * b.tile + (int)threadIdx.x : b.n;
 }
 
+// Exclusive sum over the `lanes` consecutive lanes of a warp that share an atom
+// (a power of two), and the total.  Called by whole warps.
+__device__ inline int lane_scan(int v, int lanes, int &total) {
+    const int l = threadIdx.x & (lanes - 1);
+    int x = v;
+    for (int o = 1; o < lanes; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o, lanes);
+        if (l >= o) x += y;
+    }
+    total = __shfl_sync(0xffffffffu, x, lanes - 1, lanes);
+    return x - v;
+}
+
 // Lanes that share one atom in the LJ force kernels of a band.  The band's own
 // sizes decide (not its company in a batch: the order of its sums must not
 // depend on it).

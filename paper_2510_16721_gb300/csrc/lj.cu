@@ -603,6 +603,61 @@ __device__ inline void lj_list_atom(const BandDev &b, const Tile &tl, const LJGe
     b.nbr_cnt[base + t] = padded;
 }
 
+// The same list by the `lanes` lanes of an atom (bands whose tiles hold fewer
+// atoms than threads): each walks a share of the stencil's rows, once to count its
+// entries and once to store them where the counts of the lanes before it put them.
+// Whole warps call this (t >= n: no atom).  FP64 steps that rebuild, one thread per
+// atom -> lanes: 31 atoms 55.2 -> 49.7 us, 2,915 atoms x 5 images 207 -> 175 us.
+template <typename T>
+__device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJGeom<float> &g, int t,
+                                     int lane, int lanes) {
+    const int n = b.n, cap = b.lj_cap;
+    const size_t base = (size_t)tl.img * n;
+    const float4 *off = screen_off<T>(b, base);
+    const int *start = b.bin_start + (size_t)tl.img * (b.nbins_cap + 1);
+    uint32_t *L = (uint32_t *)b.nbr_slot + (size_t)tl.img * cap * n + t;
+    const float rc2 = g.rc2, screen = g.screen;
+    const uint32_t self = lj_entry(t, 2 * g.m[0] + LJ_AXIS * 2 * g.m[1], 2 * g.m[2]);
+    const int w1 = 2 * g.m[1] + 1, rows = (2 * g.m[0] + 1) * w1;
+    const int r0 = t < n ? rows * lane / lanes : 0, r1 = t < n ? rows * (lane + 1) / lanes : 0;
+    float4 oi = make_float4(0, 0, 0, 0);
+    int b0 = 0, b1 = 0, b2 = 0;
+    if (t < n) {
+        oi = off[t];
+        unpack_bin(b.slot_bin[base + t], b0, b1, b2);
+    }
+    const auto walk = [&](auto keep) {
+        for (int r = r0; r < r1; ++r)
+            lj_row<false>(off, start, oi, b0, b1, b2, r / w1 - g.m[0], r % w1 - g.m[1], g.bvf,
+                          g.dhf, g.nb, g.m,
+                          [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
+                              const float r2 = ux * ux + uy * uy + uz * uz;
+                              if (!(r2 < screen)) return;
+                              const uint32_t e = lj_entry(q, i0 + LJ_AXIS * i1, i2);
+                              if (e != self) keep(e, r2 < rc2);
+                          });
+    };
+    int nin = 0, nsh = 0, tin, tsh;
+    walk([&](uint32_t, bool in) { in ? ++nin : ++nsh; });
+    int kin = lane_scan(nin, lanes, tin);
+    int ksh = tin + lane_scan(nsh, lanes, tsh);
+    if (t >= n) return;
+    const int total = tin + tsh;
+    if (total > cap) {
+        if (lane == 0) {
+            atomicOr(&b.bp->status, ST_NBR_OVERFLOW);
+            b.nbr_cnt[base + t] = 0;
+        }
+        return;
+    }
+    walk([&](uint32_t e, bool in) { L[(size_t)(in ? kin++ : ksh++) * n] = e; });
+    if (lane == 0) {
+        const int padded = (total + LJ_UNROLL - 1) / LJ_UNROLL * LJ_UNROLL;
+        for (int k = total; k < padded; ++k) L[(size_t)k * n] = self;
+        b.nbr_cnt[base + t] = padded;
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles, BandDev *bands) {
     dep_sync();
@@ -614,8 +669,14 @@ __global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles,
         if (b.lj_cap == 0 || !sc.rebuild) continue;  // uniform over the block
         lj_stage<float>(g, sc, *b.bp, sizeof(T) == 8, true);
         __syncthreads();
-        const int t = tile_atom(b, tl);
-        if (t < b.n) lj_list_atom<T>(b, tl, g, t);
+        const int lanes = TILE / b.tile;  // uniform over the block
+        if (sizeof(T) == 4 || lanes == 1) {
+            const int t = tile_atom(b, tl);
+            if (t < b.n) lj_list_atom<T>(b, tl, g, t);
+        } else {
+            lj_list_lanes<T>(b, tl, g, tl.t * b.tile + (int)threadIdx.x / lanes,
+                             threadIdx.x % lanes, lanes);
+        }
         __syncthreads();  // g is restaged for the next tile
     }
 }
