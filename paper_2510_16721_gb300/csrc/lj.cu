@@ -100,6 +100,15 @@ __device__ inline uint32_t lj_entry(int q, int i01, int i2) {
     return (uint32_t)q | ((uint32_t)i01 << 17) | ((uint32_t)i2 << 27);
 }
 
+// Bins farther than the list cutoff and a bin's half diagonal from the atom hold
+// no candidate.  Of the 125 half-cutoff bins of a stencil about a third are: a row
+// is walked over the part of it inside that sphere (bb = |b|^2 of the innermost
+// bin vector b).  24 bands' lists 183 -> 169 us, the FP32 walk of 62,500 atoms
+// 124.5 -> 115.3 us.
+struct LJTrim {
+    float r2, bb, ibb;
+};
+
 // Visits every cell-list candidate of the atom with FP32 offset oi in bin
 // (b0, b1, b2) along the stencil row (d0, d1): visit(q, ux, uy, uz, i0, i1,
 // i2) with (ux, uy, uz) the FP32 pair vector to slot q and i0, i1, i2 the axis
@@ -113,7 +122,8 @@ __device__ inline uint32_t lj_entry(int q, int i01, int i2) {
 template <bool AHEAD, typename Visit>
 __device__ inline void lj_row(const float4 *off, const int *start, const float4 &oi, int b0, int b1,
                               int b2, int d0, int d1, const float *s_bv, const float *s_dh,
-                              const int *s_nb, const int *s_m, Visit &&visit) {
+                              const int *s_nb, const int *s_m, const LJTrim &trim,
+                              Visit &&visit) {
     const int nb0 = s_nb[0], nb1 = s_nb[1], nb2 = s_nb[2];
     const int m0 = s_m[0], m1 = s_m[1], m2 = s_m[2];
     const bool row_ok = (b2 - m2 >= 0) && (b2 + m2 < nb2);
@@ -129,8 +139,18 @@ __device__ inline void lj_row(const float4 *off, const int *start, const float4 
     const float cx = (d0 * s_bv[0] + d1 * s_bv[3]) + (t0 * s_dh[0] + t1 * s_dh[3]);
     const float cy = (d0 * s_bv[1] + d1 * s_bv[4]) + (t0 * s_dh[1] + t1 * s_dh[4]);
     const float cz = (d0 * s_bv[2] + d1 * s_bv[5]) + (t0 * s_dh[2] + t1 * s_dh[5]);
+    const float px = cx - oi.x, py = cy - oi.y, pz = cz - oi.z;  // to the bin at d2 = 0
     if (row_ok) {
-        const int q0 = start[rowbase + b2 - m2], q1 = start[rowbase + b2 + m2 + 1];
+        // |p + d2 b|^2 <= R^2
+        const float pb = px * s_bv[6] + py * s_bv[7] + pz * s_bv[8];
+        const float disc = pb * pb - trim.bb * (px * px + py * py + pz * pz - trim.r2);
+        if (!(disc >= 0.0f)) return;
+        float h;  // an estimate: R has a margin of 0.1%
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(disc));
+        const int lo = max(-m2, (int)ceilf((-pb - h) * trim.ibb));
+        const int hi = min(m2, (int)floorf((h - pb) * trim.ibb));
+        if (lo > hi) return;
+        const int q0 = start[rowbase + b2 + lo], q1 = start[rowbase + b2 + hi + 1];
         float4 next;
         if (AHEAD && q0 < q1) next = off[q0];
         for (int q = q0; q < q1; ++q) {
@@ -152,6 +172,8 @@ __device__ inline void lj_row(const float4 *off, const int *start, const float4 
             const float ex = cx + (d2 * s_bv[6] + t2 * s_dh[6]);
             const float ey = cy + (d2 * s_bv[7] + t2 * s_dh[7]);
             const float ez = cz + (d2 * s_bv[8] + t2 * s_dh[8]);
+            const float dx = ex - oi.x, dy = ey - oi.y, dz = ez - oi.z;
+            if (dx * dx + dy * dy + dz * dz > trim.r2) continue;
             const int q1 = start[rowbase + w2 + 1];
             for (int q = start[rowbase + w2]; q < q1; ++q) {
                 const float4 oj = off[q];
@@ -186,6 +208,7 @@ struct LJGeom {
     float screen;                 // squared screen radius of the walk, with a margin
     float bvf[9], dhf[9];         // bin vectors and wrap terms in FP32 (the walk)
     int nb[3], m[3];
+    LJTrim trim;                  // which part of a row can hold a candidate
 };
 template <typename T>
 __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandParams &bp,
@@ -202,6 +225,25 @@ __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandPa
         // FP32 rounding)
         if (list) g.screen = fp64_band ? screen_r2<double>(bp.rl, sc) : screen_r2<float>(bp.rl, sc);
         else g.screen = fp64_band ? screen_r2<double>(p.rc, sc) : (float)p.rc2 * 1.001f;
+    }
+    if (threadIdx.x == 32) {
+        // a bin's corners lie within rho of its centre, and so its atoms at the
+        // build; kept bins are walked with atoms that have moved by up to the skin
+        const float *v = sc.bvf;
+        float rho2 = 0.0f;
+        for (int k = 0; k < 4; ++k) {
+            float q = 0.0f;
+            for (int c = 0; c < 3; ++c) {
+                const float x = v[c] + (k & 1 ? v[3 + c] : -v[3 + c]) + (k & 2 ? v[6 + c] : -v[6 + c]);
+                q += 0.25f * x * x;
+            }
+            rho2 = fmaxf(rho2, q);
+        }
+        const float rl = (float)(bp.rl > 0.0 ? bp.rl : bp.rc);
+        const float R = 1.001f * (rl + sqrtf(rho2) + (list ? 0.0f : (float)bp.skin));
+        g.trim.r2 = R * R;
+        g.trim.bb = v[6] * v[6] + v[7] * v[7] + v[8] * v[8];
+        g.trim.ibb = 1.0f / g.trim.bb;
     }
     if (threadIdx.x < 9) {
         g.bv[threadIdx.x] = (T)sc.bv[threadIdx.x];
@@ -335,7 +377,7 @@ __device__ inline void lj_walk_keep(const BandDev &b, const Tile &tl, const LJGe
     for (int r0 = 0; r0 < rows; r0 += lanes, r.step(lanes)) {  // uniform over the block
         if (active && r.more())
             lj_row<true>(
-                off, start, oi, b0, b1, b2, r.d0, r.d1, g.bvf, g.dhf, g.nb, g.m,
+                off, start, oi, b0, b1, b2, r.d0, r.d1, g.bvf, g.dhf, g.nb, g.m, g.trim,
                 [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
                     if (!(ux * ux + uy * uy + uz * uz < g.screen)) return;
                     if (HALF && q < t) return;
@@ -429,7 +471,7 @@ __global__ void __launch_bounds__(TILE, 8) k_lj<float>(const Tile *tiles, BandDe
         unpack_bin(b.slot_bin[base + t], b0, b1, b2);
         const float4 oi = off[t];
         for (LJRows r(g.m, lane); r.more(); r.step(lanes))
-            lj_row<false>(off, start, oi, b0, b1, b2, r.d0, r.d1, g.bvf, g.dhf, g.nb, g.m,
+            lj_row<false>(off, start, oi, b0, b1, b2, r.d0, r.d1, g.bvf, g.dhf, g.nb, g.m, g.trim,
                           [&](int, float ux, float uy, float uz, int, int, int) {
                               const float r2 = ux * ux + uy * uy + uz * uz;
                               // r2 == 0 only for the atom itself at zero shift
@@ -576,7 +618,7 @@ __device__ inline void lj_list_atom(const BandDev &b, const Tile &tl, const LJGe
     unpack_bin(b.slot_bin[base + t], b0, b1, b2);
     for (int d0 = -g.m[0]; d0 <= g.m[0]; ++d0)
         for (int d1 = -g.m[1]; d1 <= g.m[1]; ++d1)
-            lj_row<false>(off, start, oi, b0, b1, b2, d0, d1, g.bvf, g.dhf, g.nb, g.m,
+            lj_row<false>(off, start, oi, b0, b1, b2, d0, d1, g.bvf, g.dhf, g.nb, g.m, g.trim,
                           [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
                               const float r2 = ux * ux + uy * uy + uz * uz;
                               if (!(r2 < screen)) return;
@@ -629,7 +671,7 @@ __device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJG
     const auto walk = [&](auto keep) {
         for (int r = r0; r < r1; ++r)
             lj_row<false>(off, start, oi, b0, b1, b2, r / w1 - g.m[0], r % w1 - g.m[1], g.bvf,
-                          g.dhf, g.nb, g.m,
+                          g.dhf, g.nb, g.m, g.trim,
                           [&](int q, float ux, float uy, float uz, int i0, int i1, int i2) {
                               const float r2 = ux * ux + uy * uy + uz * uz;
                               if (!(r2 < screen)) return;
