@@ -682,7 +682,8 @@ __device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJG
     int nin = 0, nsh = 0, tin, tsh;
     walk([&](uint32_t, bool in) { in ? ++nin : ++nsh; });
     int kin = lane_scan(nin, lanes, tin);
-    int ksh = tin + lane_scan(nsh, lanes, tsh);
+    int ksh = lane_scan(nsh, lanes, tsh);
+    ksh = tin + tsh - 1 - ksh;  // the shell in reverse, as lj_list_atom leaves it
     if (t >= n) return;
     const int total = tin + tsh;
     if (total > cap) {
@@ -692,7 +693,7 @@ __device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJG
         }
         return;
     }
-    walk([&](uint32_t e, bool in) { L[(size_t)(in ? kin++ : ksh++) * n] = e; });
+    walk([&](uint32_t e, bool in) { L[(size_t)(in ? kin++ : ksh--) * n] = e; });
     if (lane == 0) {
         const int padded = (total + LJ_UNROLL - 1) / LJ_UNROLL * LJ_UNROLL;
         for (int k = total; k < padded; ++k) L[(size_t)k * n] = self;
@@ -700,23 +701,27 @@ __device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJG
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles, BandDev *bands) {
+// LANES false: an atom per thread throughout (FP32 sets that fill the GPU; with the
+// other form in the kernel its registers cost 27,435 atoms 2% of a step).
+template <typename T, bool LANES>
+__global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles, BandDev *bands, int split) {
     dep_sync();
     __shared__ LJGeom<float> g;
-    for (int k = blockIdx.x; k < ntiles; k += gridDim.x) {
-        const Tile tl = tiles[k];
+    for (int k = blockIdx.x; k < ntiles * split; k += gridDim.x) {
+        const Tile tl = tiles[k / split];
         BandDev &b = bands[tl.band];
         const ImgScalars &sc = b.sc[tl.img];
         if (b.lj_cap == 0 || !sc.rebuild) continue;  // uniform over the block
         lj_stage<float>(g, sc, *b.bp, sizeof(T) == 8, true);
         __syncthreads();
-        const int lanes = TILE / b.tile;  // uniform over the block
-        if (sizeof(T) == 4 || lanes == 1) {
+        const int lanes = sizeof(T) == 4 ? split : TILE / b.tile;  // uniform over the block
+        if (!LANES || lanes == 1) {
             const int t = tile_atom(b, tl);
             if (t < b.n) lj_list_atom<T>(b, tl, g, t);
-        } else {
-            lj_list_lanes<T>(b, tl, g, tl.t * b.tile + (int)threadIdx.x / lanes,
+        } else if constexpr (LANES) {
+            lj_list_lanes<T>(b, tl, g,
+                             tl.t * b.tile + (k % split) * (TILE / split) +
+                                 (int)threadIdx.x / lanes,
                              threadIdx.x % lanes, lanes);
         }
         __syncthreads();  // g is restaged for the next tile
@@ -905,7 +910,15 @@ void launch_lj_list(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t 
     // a block per tile: a build walks ~370 candidates per atom, and in a
     // batch of many bands a large share of the images rebuilds at a time
     // (a capped grid was measured slower here)
-    launch_dep(k_lj_list<T>, ntiles, TILE, s, tiles, ntiles, bands);
+    // FP32 tiles (an atom per thread) of a small set are split over several blocks
+    // with as many lanes per atom: the two end images of a band, 8 to 116 tiles,
+    // 125-175 us with one thread per atom
+    int split = 1;
+    if (sizeof(T) == 4)
+        while (split < 16 && 2 * split * ntiles <= 4 * sm_count()) split *= 2;
+    const int grid = ntiles * split;
+    if (sizeof(T) == 4 && split == 1) launch_dep(k_lj_list<T, false>, grid, TILE, s, tiles, ntiles, bands, 1);
+    else launch_dep(k_lj_list<T, true>, grid, TILE, s, tiles, ntiles, bands, split);
 }
 template <typename T>
 void launch_lj_nbr(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s, int minb) {

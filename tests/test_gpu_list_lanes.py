@@ -73,3 +73,20 @@ def test_overflow_is_reported(g, precision):
                       cell_filter=True, precision=g.MIXED if precision == "mixed" else g.FP64)
         gb.step(1)
     assert e.value.status == g.ERR_NBR_OVERFLOW
+
+
+@pytest.mark.parametrize("reps", [(2, 2, 2), (5, 5, 5), (8, 8, 9), (17, 17, 17)])
+def test_lj_mixed(g, oracle_mod, reps):
+    """Mixed LJ bands: sets of 3 to 462 tiles, split over 16 blocks to none."""
+    R0, h0, R1, h1 = ci.lj_vacancy_hop(ci.LJ_A, reps)
+    n = len(R0)
+    gb = gpu_band(g, R0, h0, R1, h1, 5, g.lj_potential(), k=1.0, dt=0.01, cell_filter=False,
+                  precision=g.MIXED, noise=ci.interior_noise(4, 5, n, 0.03))
+    gb.step(2)
+    X = gb.get_state()["X"]
+    gb.step(1)
+    F = gb.get_state()["F"]
+    idx = np.random.default_rng(7).choice(n, min(n, 40), replace=False)
+    for i in (1, 2, 3):
+        Fo = oracle_mod.LJ().forces_sampled(X[i][:n], h0, idx)
+        assert np.max(np.abs(F[i][idx] - Fo)) <= 1e-4, i
