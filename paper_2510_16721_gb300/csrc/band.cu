@@ -35,7 +35,8 @@
 namespace cfneb {
 
 template <typename T>
-__global__ void __launch_bounds__(FIN_THREADS) k_image_finalize(const ImgRef *imgs, BandDev *bands) {
+__global__ void __launch_bounds__(FIN_THREADS)
+    k_image_finalize(const ImgRef *imgs, BandDev *bands) {
     const ImgRef r = imgs[blockIdx.x];
     const BandDev b = bands[r.band];
     dep_sync();
@@ -292,7 +293,8 @@ __device__ inline void st_rows(double *p, const double (&v)[3]) {
 }
 
 template <typename T, bool FUSE>
-__global__ void __launch_bounds__(RTHREADS, sizeof(T) == 4 ? 4 : 2) k_band_dots(const Tile *tiles, BandDev *bands) {
+__global__ void __launch_bounds__(RTHREADS, sizeof(T) == 4 ? 4 : 2)
+    k_band_dots(const Tile *tiles, BandDev *bands) {
     const Tile tl = tiles[blockIdx.x];
     const BandDev b = bands[tl.band];
     dep_sync();
@@ -708,7 +710,8 @@ __global__ void __launch_bounds__(RTHREADS, sizeof(T) == 4 ? 4 : 2)
     const BandDev b0 = bands[t0.band];
     dep_sync();
     move_tile<T>(t0, b0);
-    for (int k = k0 + 1; k < k0 + FU_TILES && k < ntiles; ++k) move_tile<T>(tiles[k], bands[tiles[k].band]);
+    for (int k = k0 + 1; k < k0 + FU_TILES && k < ntiles; ++k)
+        move_tile<T>(tiles[k], bands[tiles[k].band]);
 }
 
 // X_img <- 1/2 (X_{img-1} + X_{img+1}) (image insertion; all rows)
@@ -948,7 +951,8 @@ template <typename T>
 void launch_fire_update(const Tile *tiles, int ntiles, const ImgRef *imgs, int nimg,
                         BandDev *bands, cudaStream_t s) {
     if (ntiles + nimg <= 0) return;
-    launch_dep(k_fire_update<T>, nimg + (ntiles + FU_TILES - 1) / FU_TILES, RTHREADS, s,  tiles, ntiles, imgs, nimg, bands);
+    launch_dep(k_fire_update<T>, nimg + (ntiles + FU_TILES - 1) / FU_TILES, RTHREADS, s, tiles,
+               ntiles, imgs, nimg, bands);
 }
 template <typename T>
 void launch_midpoint(BandDev *band, int img, int rows, cudaStream_t s) {

@@ -16,7 +16,8 @@
 // lattice vector and nb_a rounded bin vectors.  For |delta| <= 1 in an
 // orthorhombic cell every term is exact in FP32, so the only roundings are
 // those of the two small offsets and of the final sums: pair vectors keep
-// ~6e-8 A absolute accuracy whatever the cell size.  Enumerating delta over
+// ~6e-8 A absolute accuracy whatever the cell size.  (FP32 many-body bands store
+// integer grid positions instead, see refresh_offset.)  Enumerating delta over
 // [-m_a, m_a] with m_a = ceil(rc / bin width) visits every periodic image
 // of every atom within rc exactly once, also when rc exceeds half the cell
 // width (no minimum-image assumption; the neighbourhoods of Sec. II.B are
@@ -363,9 +364,9 @@ __device__ inline void bin_of(const ImgScalars &sc, const BandParams *, const fl
 // FP32: 12 blocks per SM (40 registers, 18.4 us at 98,303 atoms x 9 images; 18.9
 // with the 48 that the tables read ahead take).
 template <typename T>
-__global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 12 : 8) k_bin_assign(const Tile *tiles, BandDev *bands,
-                                                     cudaGraphConditionalHandle cond,
-                                                     int has_cond) {
+__global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 12 : 8)
+    k_bin_assign(const Tile *tiles, BandDev *bands, cudaGraphConditionalHandle cond,
+                 int has_cond) {
     using T4 = typename Vec4<T>::type;
     const Tile tl = tiles[blockIdx.x];
     const BandDev b = bands[tl.band];
@@ -693,12 +694,12 @@ void launch_bin_scan(const ImgRef *imgs, int count, int max_bins, BandDev *bands
 }
 void launch_bin_scatter(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    launch_dep(k_bin_scatter, ntiles < gated_grid() ? ntiles : gated_grid(), TILE, s, tiles, ntiles, bands);
+    launch_dep(k_bin_scatter, std::min(ntiles, gated_grid()), TILE, s, tiles, ntiles, bands);
 }
 template <typename T>
 void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s) {
     if (ntiles <= 0) return;
-    launch_dep(k_bin_order<T>, ntiles < gated_grid() ? ntiles : gated_grid(), TILE, s, tiles, ntiles, bands);
+    launch_dep(k_bin_order<T>, std::min(ntiles, gated_grid()), TILE, s, tiles, ntiles, bands);
 }
 template <typename T>
 void launch_bin_sort(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t s) {

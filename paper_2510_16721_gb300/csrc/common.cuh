@@ -286,7 +286,7 @@ struct BandDev {
     // entries, or LJ packed entries of lj_cap (0: the LJ kernel walks the
     // cell list directly)
     int lj_cap;
-    int *nbr_cnt;        // [ncap][n]; many-body lists: | NBR_SHIFTED if an entry's code is not CODE_ZERO
+    int *nbr_cnt;        // [ncap][n]; many-body: | NBR_SHIFTED if a code is not CODE_ZERO
     // many-body lists: [ncap][MAXN / 4][n][4] (ent: four entries of an atom are one
     // vector); LJ lists: nbr_slot [ncap][lj_cap][n]
     int *nbr_slot;

@@ -234,7 +234,8 @@ __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandPa
         for (int k = 0; k < 4; ++k) {
             float q = 0.0f;
             for (int c = 0; c < 3; ++c) {
-                const float x = v[c] + (k & 1 ? v[3 + c] : -v[3 + c]) + (k & 2 ? v[6 + c] : -v[6 + c]);
+                const float x =
+                    v[c] + (k & 1 ? v[3 + c] : -v[3 + c]) + (k & 2 ? v[6 + c] : -v[6 + c]);
                 q += 0.25f * x * x;
             }
             rho2 = fmaxf(rho2, q);
@@ -602,7 +603,8 @@ __global__ void __launch_bounds__(TILE) k_lj_energy64(const Tile *tiles, BandDev
 // screen on their rounded offsets (entries are tested again in FP64 by the
 // force kernel).
 template <typename T>
-__device__ inline void lj_list_atom(const BandDev &b, const Tile &tl, const LJGeom<float> &g, int t) {
+__device__ inline void lj_list_atom(const BandDev &b, const Tile &tl, const LJGeom<float> &g,
+                                    int t) {
     const int n = b.n, cap = b.lj_cap;
     const size_t base = (size_t)tl.img * n;
     const float4 *off = screen_off<T>(b, base);
@@ -651,8 +653,8 @@ __device__ inline void lj_list_atom(const BandDev &b, const Tile &tl, const LJGe
 // Whole warps call this (t >= n: no atom).  FP64 steps that rebuild, one thread per
 // atom -> lanes: 31 atoms 55.2 -> 49.7 us, 2,915 atoms x 5 images 207 -> 175 us.
 template <typename T>
-__device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJGeom<float> &g, int t,
-                                     int lane, int lanes) {
+__device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJGeom<float> &g,
+                                     int t, int lane, int lanes) {
     const int n = b.n, cap = b.lj_cap;
     const size_t base = (size_t)tl.img * n;
     const float4 *off = screen_off<T>(b, base);
@@ -704,7 +706,8 @@ __device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJG
 // LANES false: an atom per thread throughout (FP32 sets that fill the GPU; with the
 // other form in the kernel its registers cost 27,435 atoms 2% of a step).
 template <typename T, bool LANES>
-__global__ void __launch_bounds__(TILE) k_lj_list(const Tile *tiles, int ntiles, BandDev *bands, int split) {
+__global__ void __launch_bounds__(TILE)
+    k_lj_list(const Tile *tiles, int ntiles, BandDev *bands, int split) {
     dep_sync();
     __shared__ LJGeom<float> g;
     for (int k = blockIdx.x; k < ntiles * split; k += gridDim.x) {
@@ -824,7 +827,8 @@ __global__ void __launch_bounds__(TILE, MINB) k_lj_nbr(const Tile *tiles, BandDe
 // and in bands of few atoms by the chain of one thread's entries (31 atoms, 110
 // entries each: 129 us with one thread per atom, four warps busy; 11 us with 32
 // lanes.  2,915 atoms x 5 images: 146 us, now 108 us of which the FP64 pipe's
-// share is 65 us).  An atom's entries are dealt to its lanes (BandDev::tile), every entry is screened in
+// share is 65 us).  An atom's entries are dealt to its lanes (BandDev::tile), every
+// entry is screened in
 // FP32 on the rounded offsets first, and only entries inside the screen (78 of
 // 110; the shell entries stand last in a list, so a warp skips most of them
 // together) reach FP64.
@@ -918,8 +922,10 @@ void launch_lj_list(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t 
     if (sizeof(T) == 4)
         while (split < 16 && 2 * split * ntiles <= 4 * sm_count()) split *= 2;
     const int grid = ntiles * split;
-    if (sizeof(T) == 4 && split == 1) launch_dep(k_lj_list<T, false>, grid, TILE, s, tiles, ntiles, bands, 1);
-    else launch_dep(k_lj_list<T, true>, grid, TILE, s, tiles, ntiles, bands, split);
+    if (sizeof(T) == 4 && split == 1)
+        launch_dep(k_lj_list<T, false>, grid, TILE, s, tiles, ntiles, bands, 1);
+    else
+        launch_dep(k_lj_list<T, true>, grid, TILE, s, tiles, ntiles, bands, split);
 }
 template <typename T>
 void launch_lj_nbr(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_t s, int minb) {
