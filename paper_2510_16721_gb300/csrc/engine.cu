@@ -37,13 +37,19 @@ struct CudaFail {
     cudaError_t e;
 };
 
+// A failed call leaves its error with the runtime until it is asked for: it is
+// taken off here, or the next call's own check after its launches would find it
+// and fail (an allocation that did not fit, then a smaller one that does).
+[[noreturn]] void cuda_fail(cudaError_t e, const char *what) {
+    g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
+    cudaGetLastError();
+    throw CudaFail{e};
+}
+
 #define CK(x)                                                                            \
     do {                                                                                 \
         cudaError_t _e = (x);                                                            \
-        if (_e != cudaSuccess) {                                                         \
-            g_last_error = std::string(#x) + ": " + cudaGetErrorString(_e);              \
-            throw CudaFail{_e};                                                          \
-        }                                                                                \
+        if (_e != cudaSuccess) cuda_fail(_e, #x);                                        \
     } while (0)
 
 static_assert(NEP_NW == CFNEB_NEP_N_WEIGHTS, "NEP weight count of the header and kernels");
@@ -194,11 +200,7 @@ struct Arena {
 
 void *device_alloc(size_t bytes) {
     void *p = nullptr;
-    const cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) {
-        g_last_error = std::string("cudaMalloc: ") + cudaGetErrorString(e);
-        throw CudaFail{e};
-    }
+    CK(cudaMalloc(&p, bytes));
     return p;
 }
 
