@@ -825,12 +825,12 @@ __global__ void __launch_bounds__(TILE) k_points_store(const Tile *tiles, BandDe
 
 // State exchange on the device: the band's padded T rows against [N][n + 3][3]
 // doubles in the scratch array (converted by one thread per value: host loops
-// over 98,304-atom bands took as long as tens of steps).  blockIdx.y = image.
+// over 98,304-atom bands took as long as tens of steps).  `blocks` per image.
 template <typename T>
-__global__ void k_state_load(BandDev *band, int n, double c) {
+__global__ void k_state_load(BandDev *band, int n, double c, int blocks) {
     BandDev &b = *band;
-    const size_t img = blockIdx.y;
-    const int per = (n + 3) * 3, e = blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t img = blockIdx.x / blocks;
+    const int per = (n + 3) * 3, e = (blockIdx.x % blocks) * blockDim.x + threadIdx.x;
     if (e >= b.rows * 3) return;
     double v = 0.0;
     if (e < per) {
@@ -841,10 +841,10 @@ __global__ void k_state_load(BandDev *band, int n, double c) {
     ((T *)b.X)[img * (size_t)b.rows * 3 + e] = (T)v;
 }
 template <typename T>
-__global__ void k_state_store(BandDev *band, int which, int N, int n, double c) {
+__global__ void k_state_store(BandDev *band, int which, int N, int n, double c, int blocks) {
     BandDev &b = *band;
-    const size_t img = blockIdx.y;
-    const int per = (n + 3) * 3, e = blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t img = blockIdx.x / blocks;
+    const int per = (n + 3) * 3, e = (blockIdx.x % blocks) * blockDim.x + threadIdx.x;
     if (e >= per) return;
     const void *src = which == 0 ? b.X : which == 1 ? b.F : b.Fneb;
     double v = (double)((const T *)src)[img * (size_t)b.rows * 3 + e];
@@ -905,12 +905,13 @@ void launch_points_store(const Tile *tiles, int ntiles, BandDev *bands, cudaStre
 }
 template <typename T>
 void launch_state_load(BandDev *band, int N, int n, double c, cudaStream_t s) {
-    const int rows = (n + 3 + 3) / 4 * 4;
-    k_state_load<T><<<dim3((rows * 3 + 255) / 256, N), 256, 0, s>>>(band, n, c);
+    const int rows = (n + 3 + 3) / 4 * 4, blocks = (rows * 3 + 255) / 256;
+    k_state_load<T><<<N * blocks, 256, 0, s>>>(band, n, c, blocks);
 }
 template <typename T>
 void launch_state_store(BandDev *band, int which, int N, int n, double c, cudaStream_t s) {
-    k_state_store<T><<<dim3(((n + 3) * 3 + 255) / 256, N), 256, 0, s>>>(band, which, N, n, c);
+    const int blocks = ((n + 3) * 3 + 255) / 256;
+    k_state_store<T><<<N * blocks, 256, 0, s>>>(band, which, N, n, c, blocks);
 }
 void launch_fire_reset(BandDev *band, cudaStream_t s) { k_fire_reset<<<1, 1, 0, s>>>(band); }
 void launch_set_control(BandDev *band, double ftol, long long move_limit, cudaStream_t s) {

@@ -455,7 +455,7 @@ __device__ inline int block_excl_scan_1024(int v, int *total) {
 
 __global__ void __launch_bounds__(256) k_bin_tilesum(const ImgRef *imgs, BandDev *bands) {
     dep_sync();
-    ImgRef r = imgs[blockIdx.y];
+    ImgRef r = imgs[blockIdx.x];
     BandDev &b = bands[r.band];
     if (!b.sc[r.img].rebuild) return;
     const int nb = b.sc[r.img].nbins;
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(256) k_bin_tilesum(const ImgRef *imgs, BandDev
     __shared__ int ws[8];
     // a fixed grid strides over the tiles: images that keep their cell list
     // cost one read per block
-    for (int c = blockIdx.x; c * SCAN_TILE < nb; c += gridDim.x) {
+    for (int c = blockIdx.y; c * SCAN_TILE < nb; c += gridDim.y) {
         const int t0 = c * SCAN_TILE;
         int s = 0;
         for (int k = threadIdx.x; k < SCAN_TILE && t0 + k < nb; k += blockDim.x) s += cnt[t0 + k];
@@ -499,13 +499,13 @@ __global__ void __launch_bounds__(1024) k_bin_tilescan(const ImgRef *imgs, BandD
 
 __global__ void __launch_bounds__(1024) k_bin_scanfill(const ImgRef *imgs, BandDev *bands) {
     dep_sync();
-    ImgRef r = imgs[blockIdx.y];
+    ImgRef r = imgs[blockIdx.x];
     BandDev &b = bands[r.band];
     if (!b.sc[r.img].rebuild) return;
     const int nb = b.sc[r.img].nbins;
     int *cnt = b.bin_count + (size_t)r.img * b.nbins_cap;
     int *start = b.bin_start + (size_t)r.img * (b.nbins_cap + 1);
-    for (int c = blockIdx.x; c * SCAN_TILE < nb; c += gridDim.x) {
+    for (int c = blockIdx.y; c * SCAN_TILE < nb; c += gridDim.y) {
         const int bin = c * SCAN_TILE + threadIdx.x;
         const int v = bin < nb ? cnt[bin] : 0;
         int tot;
@@ -656,13 +656,13 @@ __global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
     }
 }
 
-// Cartesian positions R = R~ D (FP64) of a band's images (blockIdx.y), for
+// Cartesian positions R = R~ D (FP64) of a band's images (`per` blocks each), for
 // output.
 template <typename T>
-__global__ void k_cartesian(BandDev *band) {
-    const ImgRef r = {0, (int)blockIdx.y};
+__global__ void k_cartesian(BandDev *band, int per) {
+    const ImgRef r = {0, (int)(blockIdx.x / per)};
     BandDev &b = *band;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int i = (blockIdx.x % per) * blockDim.x + threadIdx.x;
     if (i >= b.n) return;
     const ImgScalars &sc = b.sc[r.img];
     const T *Xi = (const T *)b.X + ((size_t)r.img * b.rows + i) * 3;
@@ -687,7 +687,7 @@ void launch_bin_assign(const Tile *tiles, int ntiles, BandDev *bands, cudaStream
 void launch_bin_scan(const ImgRef *imgs, int count, int max_bins, BandDev *bands,
                      cudaStream_t s, int part) {
     if (count <= 0 || max_bins <= 0) return;
-    dim3 grid(std::min((max_bins + SCAN_TILE - 1) / SCAN_TILE, 32), count);
+    dim3 grid(count, std::min((max_bins + SCAN_TILE - 1) / SCAN_TILE, 32));
     if (part == 0) launch_dep(k_bin_tilesum, grid, 256, s, imgs, bands);
     else if (part == 1) launch_dep(k_bin_tilescan, count, 1024, s, imgs, bands);
     else launch_dep(k_bin_scanfill, grid, 1024, s, imgs, bands);
@@ -709,8 +709,8 @@ void launch_bin_sort(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t
 template <typename T>
 void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {
     if (N <= 0 || n <= 0) return;
-    dim3 grid((n + 127) / 128, N);
-    k_cartesian<T><<<grid, 128, 0, s>>>(band);
+    const int per = (n + 127) / 128;
+    k_cartesian<T><<<N * per, 128, 0, s>>>(band, per);
 }
 
 #define CFNEB_INST(T)                                                                     \

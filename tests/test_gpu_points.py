@@ -109,3 +109,19 @@ def test_state_and_path_in_any_order(g, pot, precision):
     np.testing.assert_allclose(p1["energies"], p3["energies"], rtol=1e-12)
     assert p1["energies"][0] == p2["energies"][0] and p1["energies"][-1] == p2["energies"][-1]
     np.testing.assert_allclose(p1["positions"][0], R0, atol=2e-5 if precision else 1e-12)
+
+
+def test_more_structures_than_a_grid_axis_holds(g):
+    """66,001 structures in one call, the last of them large enough to take the
+    five-pass cell list for all: a kernel's grid holds 65,535 blocks along its
+    second and third axes only."""
+    pot = g.lj_potential()
+    few = [(np.array([[0.1 * k, 0.0, 0.0], [1.05 + 0.11 * k, 0.2, 0.0]]), np.eye(3) * 4.0)
+           for k in range(8)]
+    R, h = ci.fcc(ci.LJ_A, 20, 20, 18)
+    R = R + np.random.default_rng(5).normal(0.0, 0.02, R.shape)
+    want = [g.evaluate([s], pot, g.FP64) for s in few + [(R, h)]]
+    E, F, V = g.evaluate(few * 8250 + [(R, h)], pot, g.FP64)
+    assert np.array_equal(E, np.concatenate([np.tile([w[0][0] for w in want[:8]], 8250), want[8][0]]))
+    for k, w in list(enumerate(want[:8])) + [(65528 + j, want[j]) for j in range(8)] + [(66000, want[8])]:
+        assert np.array_equal(F[k], w[1][0]) and np.array_equal(V[k], w[2][0])
