@@ -1028,7 +1028,15 @@ std::tuple<int, int, int, int> tune_class(const cfneb_potential *pot, int precis
 // to 480 atoms 3.1 ms, a 98,304-atom one 3.4 ms.)  The FP64 energies come from
 // the same cell list; an FP64 evaluation's own energy is one already.
 
-constexpr long long POINT_GROUP_ATOMS = 1LL << 18;
+// A group ends at this many atoms (~0.25 GB) or cell-list bins (4 GB: up to 2^26
+// bins per structure, whatever its atoms, where a box is mostly empty).
+constexpr long long POINT_GROUP_ATOMS = 1LL << 18, POINT_GROUP_BINS = 1LL << 29;
+
+// bins reserved for a structure's cell list: room for the finest tuned grid
+int point_bins(const double *cell, double rc) {
+    const int nb = bins_for(cell, rc * kTuneScales[0]);
+    return (int)std::min<long long>((long long)(1.5 * nb) + 64, 1LL << 26);
+}
 
 // every reason to refuse a structure (all CFNEB_ERR_INVALID_ARG)
 int check_point(const cfneb_structure &S, const cfneb_potential *pot, int precision) {
@@ -1077,8 +1085,7 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
         d.rows = (n + 3 + 3) / 4 * 4;
         d.ncap = P.N = 1;
         const auto key = tune_class(pot, precision, n, vol, rc);
-        const int nb = bins_for(S[k].cell, rc * kTuneScales[0]);
-        d.nbins_cap = (int)std::min<long long>((long long)(1.5 * nb) + 64, 1LL << 26);
+        d.nbins_cap = point_bins(S[k].cell, rc);
         d.tsum_cap = (d.nbins_cap + 1023) / 1024 + 1;
         d.tile = atom_tile(pot, precision, n, 1, vol, rc, lj);
         d.atpi = (n + d.tile - 1) / d.tile;
@@ -2385,10 +2392,14 @@ int cfneb_evaluate(const cfneb_structure *structures, int32_t count,
     int k = 0;
     while (k < count) {
         int e = k, st = CFNEB_OK;
-        long long n = 0;
+        long long n = 0, bins = 0;
+        double rc = 0.0;
         while (e < count && (st = check_point(structures[e], potential, precision)) == CFNEB_OK) {
-            if (e > k && n + structures[e].n_atoms > POINT_GROUP_ATOMS) break;
-            n += structures[e++].n_atoms;
+            check_potential(potential, &rc);
+            n += structures[e].n_atoms;
+            bins += point_bins(structures[e].cell, rc);
+            if (e > k && (n > POINT_GROUP_ATOMS || bins > POINT_GROUP_BINS)) break;
+            ++e;
         }
         const int refused = st;
         int done = 0;

@@ -53,3 +53,29 @@ def test_points_that_fit_one_by_one(g):
     for k, (e, f, v) in enumerate(want):
         assert E[k] == e[0]
         assert np.array_equal(F[k], f[0]) and np.array_equal(V[k], v[0])
+
+
+def test_a_group_of_points_is_bounded(g):
+    """40 structures with 0.54 GB of bins each: a group takes 4 GB of them and
+    little else, as another thread sees it."""
+    import threading
+
+    import torch
+    S = [_dimer(1.05 + 0.01 * k, 460.0) for k in range(40)]
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    least, done = [before], threading.Event()
+
+    def watch():
+        while not done.is_set():
+            least[0] = min(least[0], torch.cuda.mem_get_info()[0])
+
+    w = threading.Thread(target=watch)
+    w.start()
+    try:
+        g.evaluate(S, g.lj_potential(), g.FP64)
+    finally:
+        done.set()
+        w.join()
+    assert before - least[0] <= 5 << 30
