@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import cfneb_inputs as ci
-from _cases import f32_structure
+from _cases import f32_structure, gpu_band
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +49,36 @@ def test_points(g, oracle_mod, kind, reps, drop):
     assert np.max(np.abs(F[0] - Fo)) <= max(1e-4, 1e-6 * np.max(np.abs(Fo)))
     assert abs(E[0] - e.sum()) <= 1e-10 * max(1.0, np.abs(e).sum())
     assert np.max(np.abs(V[0] - Vo)) <= 1e-4 * len(R)
+
+
+def _sharp(g, oracle_mod):
+    """Carbon's constants with a cutoff of no width (D = 0) at 2 A."""
+    q = dict(oracle_mod.TERSOFF_C1988, R=2.0, D=0.0)
+    order = ["A", "B", "lambda1", "lambda2", "beta", "n", "c", "d", "h", "R", "D"]
+    return g.tersoff_potential([q[k] for k in order]), oracle_mod.Tersoff(q)
+
+
+@pytest.mark.parametrize("kind,reps,drop", [("graphite", (2, 1, 2), 1), ("diamond", (3, 2, 3), 15),
+                                            ("dense", (2, 2, 2), 0), ("sparse", (4, 4, 4), 0)])
+def test_sharp_cutoff_points(g, oracle_mod, kind, reps, drop):
+    """Entries that an atom does not have stay outside a cutoff of no width."""
+    pot, o = _sharp(g, oracle_mod)
+    R, h = f32_structure(*_carbon(kind, reps, drop, 3))
+    e, Fo, Vo = o.evaluate(R, h)
+    E, F, V = g.evaluate([(R, h)], pot, g.MIXED)
+    assert np.max(np.abs(F[0] - Fo)) <= max(1e-4, 1e-6 * np.max(np.abs(Fo)))
+    assert np.max(np.abs(V[0] - Vo)) <= 1e-4 * len(R)
+
+
+def test_sharp_cutoff_step_energies(g, oracle_mod):
+    """The end images' step energies: 63 atoms leave half of a block without one.
+    FP32 site energies: a few 1e-7 of each atom's energy and of a warp's sum."""
+    pot, o = _sharp(g, oracle_mod)
+    R0, h0, R1, h1 = ci.diamond_vacancy_hop(reps=(2, 2, 2))
+    R0, R1 = f32_structure(R0, h0)[0], f32_structure(R1, h1)[0]
+    band = gpu_band(g, R0, h0, R1, h1, 3, pot, k=0.1, dt=0.05, precision=g.MIXED)
+    E = band.image_scalars()["E"]
+    band.destroy()
+    e0, e1 = o.evaluate(R0, h0)[0].sum(), o.evaluate(R1, h1)[0].sum()
+    assert abs(E[0] - e0) <= 1e-6 * abs(e0)
+    assert abs(E[2] - e1) <= 1e-6 * abs(e1)
