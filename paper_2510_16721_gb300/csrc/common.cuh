@@ -167,7 +167,8 @@ struct __align__(8) TP {  // Tersoff constants in T (derived once per band, on t
     T AeR, BeR;        // A exp(-l1 R), B exp(-l2 R)
     T R2hi, R2lo;      // R^2 as a two-term sum
     T Dlo;             // D - (T)D
-    T pad_;            // (a whole number of 8-byte words: staged by word copies)
+    T xs;              // (beta zeta)^n below which the bond order is a series
+                       // (and a whole number of 8-byte words: staged by word copies)
     // host only (std::exp of the host library): the device reads the result
     __host__ void load(const TersoffParams &p) {
         A = (T)p.A; B = (T)p.B; l1 = (T)p.lambda1; l2 = (T)p.lambda2; beta = (T)p.beta;
@@ -182,6 +183,8 @@ struct __align__(8) TP {  // Tersoff constants in T (derived once per band, on t
         R2hi = (T)(p.R * p.R);
         R2lo = (T)(p.R * p.R - (double)R2hi);
         Dlo = (T)(p.D - (double)D);
+        // x below 2^-10 and x / 2n below 2^-9 (FP32: 2^-8)
+        xs = (T)std::fmin(1.0 / 1024.0, std::fabs(p.n) / (sizeof(T) == 8 ? 256.0 : 128.0));
     }
 };
 
@@ -1159,11 +1162,11 @@ __device__ inline void ters_code(int code, int b0, int b1, int b2, const int *s_
     }
 }
 
-// b = (1 + x)^(-1/2n) for x = (beta zeta)^n: below 2^-10 (carbon: ~1e-4) by
-// the series of log(1 + x) to x^6 and exp(-u) to u^5 (truncation below 1e-18
-// relative)
-__device__ inline double bond_order_x(double x, double inv2n) {
-    if (x < 1.0 / 1024.0) {
+// b = (1 + x)^(-1/2n) for x = (beta zeta)^n: below xs (2^-10, carbon: x ~ 1e-4; less
+// where n < 1/4, so that u = x / 2n stays below 2^-9) by the series of log(1 + x) to
+// x^6 and exp(-u) to u^5 (truncation below 1e-18 relative)
+__device__ inline double bond_order_x(double x, double inv2n, double xs) {
+    if (x < xs) {
         const double l = x * (1.0 - x * (0.5 - x * (1.0 / 3.0 - x * (0.25 - x * (0.2 - x * (1.0 / 6.0))))));
         const double u = inv2n * l;
         return 1.0 - u * (1.0 - u * (0.5 - u * (1.0 / 6.0 - u * (1.0 / 24.0 - u * (1.0 / 120.0)))));

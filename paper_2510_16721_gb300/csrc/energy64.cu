@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(TILE) k_energy64(const Tile *tiles, BandDev *b
             for (int j = 0; j < cnt; ++j) {
                 if (fc[j] == 0.0) continue;  // beyond R + D
                 const double bz = q.beta * zeta[j];
-                const double bij = bz > 0.0 ? bond_order_x(exp(q.n * log(bz)), q.inv2n) : 1.0;
+                const double bij = bz > 0.0 ? bond_order_x(exp(q.n * log(bz)), q.inv2n, q.xs) : 1.0;
                 U += 0.5 * fc[j] * (q.A * exp(-q.l1 * E.r[j]) - bij * q.B * exp(-q.l2 * E.r[j]));
             }
         } else {

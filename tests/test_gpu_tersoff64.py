@@ -58,3 +58,21 @@ def test_both_forms_agree(g, kind):
     assert np.max(np.abs(F2[0].reshape(27, -1, 3) - F1[0])) <= 1e-10 * s
     assert abs(E2[0] - 27 * E1[0]) <= 1e-10 * abs(E2[0])
     assert np.max(np.abs(V2[0] - 27 * V1[0])) <= 1e-9 * max(1.0, np.max(np.abs(V2[0])))
+
+
+@pytest.mark.parametrize("n", [0.01, 0.0125, 0.05, 0.2, 0.25, 0.72751])
+@pytest.mark.parametrize("x", [2e-5, 9e-4, 1.1e-3, 0.3])
+def test_bond_order_over_n(g, n, x):
+    """Three atoms whose bond order is (1 + x)^(-1/2n) with x given (g = 1, one other
+    neighbour: zeta = 1): FP64 energy to a few roundings for any n, with x on both
+    sides of the series' limit."""
+    A, B, l1, l2, r = 1393.6, 346.74, 3.4879, 2.2119, 1.5
+    par = [A, B, l1, l2, x ** (1.0 / n), n, 0.0, 1.0, -0.57, 1.95, 0.15]
+    R = 5.0 + r * np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [0.5, 0.75 ** 0.5, 0.0]])
+    E, F, V = g.evaluate([(R, np.eye(3) * 12.0)], g.tersoff_potential(par), g.FP64)
+    d = [np.linalg.norm(R[i] - R[j]) for i, j in ((0, 1), (0, 2), (1, 2))]
+    b = np.exp(-np.log1p(par[4] ** n) / (2.0 * n))  # (a beta below 1e-308 is 0: b = 1)
+    rep, att = (sum(c * np.exp(-l * v) for v in d) for c, l in ((A, l1), (B, l2)))
+    # x ** (1/n) and back: 2^-53 (|log x| + 1) of x, u of that in b
+    tol = 1e-14 * (rep + att) * (1.0 + x / (2.0 * n) * abs(np.log(x)))
+    assert abs(E[0] - (rep - b * att)) <= tol
