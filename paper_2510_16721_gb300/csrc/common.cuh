@@ -434,13 +434,14 @@ __device__ inline float d2f_pos(double x) {  // a positive x truncated to FP32
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
 }
-// x lies in FP32's normal range (and is positive), with room for a square
+// 2^-126 <= x < 2^126: x and 1 / x are normal in FP32, and __fdividef divides by x
+// (by 2^126 and more it gives 0)
 __device__ inline bool in_f32_range(double x) {
-    return (unsigned)__double2hiint(x) - 0x38100000u < 0x47E00000u - 0x38100000u;
+    return (unsigned)__double2hiint(x) - 0x38100000u < 0x47D00000u - 0x38100000u;
 }
 // Reciprocal of a positive x from an FP32 seed (error e ~ 2^-22) and one
 // third-order step r (1 + e + e^2): ~1 ulp in three FP64 instructions; outside
-// FP32's range a divide.
+// in_f32_range a divide.
 __device__ inline double rcp64_pos(double x) {
     if (!in_f32_range(x)) return 1.0 / x;
     const double r = f2d(__fdividef(1.0f, d2f_pos(x)));

@@ -76,3 +76,19 @@ def test_bond_order_over_n(g, n, x):
     # x ** (1/n) and back: 2^-53 (|log x| + 1) of x, u of that in b
     tol = 1e-14 * (rep + att) * (1.0 + x / (2.0 * n) * abs(np.log(x)))
     assert abs(E[0] - (rep - b * att)) <= tol
+
+
+@pytest.mark.parametrize("product", [4e37, 8.6e37, 1.2e38, 1.6e38, 1.8e38, 1e39])
+def test_large_bond_order_argument(g, oracle_mod, product):
+    """Three atoms in the cutoff's edge with (beta zeta)^n zeta about 2^126 to 2^127,
+    where FP32 has no normal reciprocal: forces through db/dzeta against the oracle."""
+    n, zeta = 50.0, 0.5  # f_C = 1/2 at r = R, g = 1
+    beta = (product / zeta) ** (1.0 / n) / zeta
+    par = [1393.6, 346.74, 3.4879, 2.2119, beta, n, 0.0, 1.0, -0.57, 1.95, 0.15]
+    R = 5.0 + 1.95 * np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [0.5, 0.75 ** 0.5, 0.0]])
+    h = np.eye(3) * 12.0
+    names = ["A", "B", "lambda1", "lambda2", "beta", "n", "c", "d", "h", "R", "D"]
+    e, Fo, Vo = oracle_mod.Tersoff(dict(zip(names, par))).evaluate(R, h)
+    E, F, V = g.evaluate([(R, h)], g.tersoff_potential(par), g.FP64)
+    assert np.max(np.abs(F[0] - Fo)) <= 1e-10 * np.max(np.abs(Fo))
+    assert abs(E[0] - e.sum()) <= 1e-10 * abs(e).sum()
