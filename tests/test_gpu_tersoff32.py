@@ -82,3 +82,18 @@ def test_sharp_cutoff_step_energies(g, oracle_mod):
     e0, e1 = o.evaluate(R0, h0)[0].sum(), o.evaluate(R1, h1)[0].sum()
     assert abs(E[0] - e0) <= 1e-6 * abs(e0)
     assert abs(E[2] - e1) <= 1e-6 * abs(e1)
+
+
+@pytest.mark.parametrize("product", [4e37, 8.6e37, 1.2e38, 1.6e38])
+def test_large_bond_order_argument(g, oracle_mod, product):
+    """Three atoms in the cutoff's edge with (beta zeta)^n zeta about 2^126 to 2^127,
+    where FP32 has no normal reciprocal: forces through db/dzeta."""
+    n, zeta = 50.0, 0.5  # f_C = 1/2 at r = R, g = 1
+    beta = (product / zeta) ** (1.0 / n) / zeta
+    par = [1393.6, 346.74, 3.4879, 2.2119, beta, n, 0.0, 1.0, -0.57, 1.95, 0.15]
+    R = 5.0 + 1.95 * np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [0.5, 0.75 ** 0.5, 0.0]])
+    R, h = f32_structure(R, np.eye(3) * 12.0)
+    names = ["A", "B", "lambda1", "lambda2", "beta", "n", "c", "d", "h", "R", "D"]
+    e, Fo, Vo = oracle_mod.Tersoff(dict(zip(names, par))).evaluate(R, h)
+    E, F, V = g.evaluate([(R, h)], g.tersoff_potential(par), g.MIXED)
+    assert np.max(np.abs(F[0] - Fo)) <= 1e-4
