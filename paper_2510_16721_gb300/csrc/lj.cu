@@ -102,11 +102,11 @@ __device__ inline uint32_t lj_entry(int q, int i01, int i2) {
 
 // Bins farther than the list cutoff and a bin's half diagonal from the atom hold
 // no candidate.  Of the 125 half-cutoff bins of a stencil about a third are: a row
-// is walked over the part of it inside that sphere (bb = |b|^2 of the innermost
+// is walked over the part of it inside that sphere (ibb = 1 / |b|^2 of the innermost
 // bin vector b).  24 bands' lists 183 -> 169 us, the FP32 walk of 62,500 atoms
 // 124.5 -> 115.3 us.
 struct LJTrim {
-    float r2, bb, ibb;
+    float r2, ibb;
 };
 
 // Visits every cell-list candidate of the atom with FP32 offset oi in bin
@@ -141,14 +141,15 @@ __device__ inline void lj_row(const float4 *off, const int *start, const float4 
     const float cz = (d0 * s_bv[2] + d1 * s_bv[5]) + (t0 * s_dh[2] + t1 * s_dh[5]);
     const float px = cx - oi.x, py = cy - oi.y, pz = cz - oi.z;  // to the bin at d2 = 0
     if (row_ok) {
-        // |p + d2 b|^2 <= R^2
-        const float pb = px * s_bv[6] + py * s_bv[7] + pz * s_bv[8];
-        const float disc = pb * pb - trim.bb * (px * px + py * py + pz * pz - trim.r2);
+        // |p + d2 b|^2 <= R^2, in units of |b|: fourth powers of a length in metres
+        // would leave FP32's range
+        const float pb = (px * s_bv[6] + py * s_bv[7] + pz * s_bv[8]) * trim.ibb;
+        const float disc = pb * pb - (px * px + py * py + pz * pz - trim.r2) * trim.ibb;
         if (!(disc >= 0.0f)) return;
         float h;  // an estimate: R has a margin of 0.1%
         asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(disc));
-        const int lo = max(-m2, (int)ceilf((-pb - h) * trim.ibb));
-        const int hi = min(m2, (int)floorf((h - pb) * trim.ibb));
+        const int lo = max(-m2, (int)ceilf(-pb - h));
+        const int hi = min(m2, (int)floorf(h - pb));
         if (lo > hi) return;
         const int q0 = start[rowbase + b2 + lo], q1 = start[rowbase + b2 + hi + 1];
         float4 next;
@@ -243,8 +244,7 @@ __device__ inline void lj_stage(LJGeom<T> &g, const ImgScalars &sc, const BandPa
         const float rl = (float)(bp.rl > 0.0 ? bp.rl : bp.rc);
         const float R = 1.001f * (rl + sqrtf(rho2) + (list ? 0.0f : (float)bp.skin));
         g.trim.r2 = R * R;
-        g.trim.bb = v[6] * v[6] + v[7] * v[7] + v[8] * v[8];
-        g.trim.ibb = 1.0f / g.trim.bb;
+        g.trim.ibb = 1.0f / (v[6] * v[6] + v[7] * v[7] + v[8] * v[8]);
     }
     if (threadIdx.x < 9) {
         g.bv[threadIdx.x] = (T)sc.bv[threadIdx.x];
