@@ -61,8 +61,9 @@ namespace cfneb {
 // stencil half widths m from the perpendicular widths and the list cutoff.
 // Between rebuilds the grid stays as built and only the bin vectors follow
 // the cell (bin_vectors_warp).
+// status: the band's word in memory (bp may be a staged copy).
 __device__ void bin_grid(const BandParams *bp, int nbins_cap, const double *h, double omega,
-                         ImgScalars &sc) {
+                         ImgScalars &sc, int *status) {
     const double rl = bp->rl > 0.0 ? bp->rl : bp->rc;
     int nb[3];
     float w[3];
@@ -74,6 +75,13 @@ __device__ void bin_grid(const BandParams *bp, int nbins_cap, const double *h, d
         const double cx = u[1] * v[2] - u[2] * v[1], cy = u[2] * v[0] - u[0] * v[2],
                      cz = u[0] * v[1] - u[1] * v[0];
         w[a] = (float)omega / sqrtf((float)(cx * cx + cy * cy + cz * cz)) * 0.9999f;
+        // a cell whose volume or areas leave FP32's range: refused, and on with a
+        // grid that is safe (a NaN here would give no bin at all, and the walks
+        // that wrap by the bin count would not end)
+        if (!(w[a] > 0.0f && w[a] <= 3e38f)) {
+            atomicOr(status, ST_NBR_OVERFLOW);
+            w[a] = (float)rl;
+        }
     }
     for (int a = 0; a < 3; ++a) {
         // the innermost axis may be binned finer: the LJ kernel walks it
@@ -84,7 +92,7 @@ __device__ void bin_grid(const BandParams *bp, int nbins_cap, const double *h, d
         // MAX_STENCIL bins per side (coarser bins are always correct)
         const float q = fminf(floorf(w[a] / bw),
                               floorf(w[a] * (float)MAX_STENCIL / (float)rl * 0.9999f));
-        nb[a] = q < 1.0f ? 1 : (q > 1024.0f ? 1024 : (int)q);
+        nb[a] = q >= 1.0f ? (q > 1024.0f ? 1024 : (int)q) : 1;
     }
     // keep within the bin capacity: coarser bins are always correct
     while ((long long)nb[0] * nb[1] * nb[2] > nbins_cap) {
@@ -96,7 +104,7 @@ __device__ void bin_grid(const BandParams *bp, int nbins_cap, const double *h, d
         const int m = (int)ceilf((float)rl / bw);
         // a cell narrower than rl / MAX_STENCIL: periodic images beyond the
         // stencil would be missed
-        if (m > MAX_STENCIL) atomicOr(const_cast<int *>(&bp->status), ST_NBR_OVERFLOW);
+        if (m > MAX_STENCIL) atomicOr(status, ST_NBR_OVERFLOW);
         sc.m[a] = m < 1 ? 1 : (m > MAX_STENCIL ? MAX_STENCIL : m);
         sc.nb[a] = nb[a];
     }
@@ -109,7 +117,7 @@ __device__ void bin_grid(const BandParams *bp, int nbins_cap, const double *h, d
 // or while autotuning).  d = the largest displacement since the build; the
 // cell's part of the bound (skin_terms) is current in sc.
 __device__ void skin_decide_one(const BandParams *bp, int nbins_cap, ImgScalars &sc, double d,
-                                int force) {
+                                int force, int *status) {
     bool rebuild = force || bp->stale || bp->tune_rebuild || sc.builds == 0;
     if (!rebuild) {
         const double bound = bp->rl * (1.0 - 1e-5) * (1.0 - (double)sc.skin_e) -
@@ -117,7 +125,7 @@ __device__ void skin_decide_one(const BandParams *bp, int nbins_cap, ImgScalars 
         rebuild = !(bound > bp->rc);
     }
     if (rebuild) {
-        bin_grid(bp, nbins_cap, sc.h, sc.omega, sc);
+        bin_grid(bp, nbins_cap, sc.h, sc.omega, sc, status);
         float Db[9];
         for (int k = 0; k < 9; ++k) {
             sc.Db[k] = sc.D[k];
@@ -181,12 +189,12 @@ __global__ void __launch_bounds__(32) k_mapback(const ImgRef *imgs, int count, B
         if (!fresh && bp->skin > 0.0) skin_terms(sc, sc.Dbif);
         if (bp->skin <= 0.0) {
             // no skin: the cell list is rebuilt at every evaluation
-            bin_grid(bp, b.nbins_cap, sc.h, sc.omega, sc);
+            bin_grid(bp, b.nbins_cap, sc.h, sc.omega, sc, &b.bp->status);
             sc.rebuild = 1;
             sc.builds += 1;
             sc.evals += 1;
         } else {
-            skin_decide_one(bp, b.nbins_cap, sc, dmax, force);
+            skin_decide_one(bp, b.nbins_cap, sc, dmax, force, &b.bp->status);
         }
     }
     __syncwarp();

@@ -57,3 +57,22 @@ def test_reflected_end_cell_is_not_spd_for_the_deformation_gradient(g):
     with pytest.raises(g.CfnebError) as e:
         gpu_band(g, R0, h0, R1, h1, 5, g.lj_potential(), k=1.0, dt=0.01, variant=1)
     assert e.value.status == g.ERR_NOT_SPD
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("scale", [2.0 ** -50, 2.0 ** 45])
+def test_cells_beyond_the_bin_arithmetic(g, scale, precision):
+    """Cells whose volume or areas leave FP32's range, in which the bins are
+    counted, end with a status; the next call is unharmed."""
+    R0, h0, _, _ = ci.lj_vacancy_hop()
+    lj = g.lj_potential(1.0, scale, 2.5 * scale)
+    with pytest.raises(g.CfnebError) as e:
+        g.evaluate([(scale * R0, scale * h0)], lj, precision)
+    assert e.value.status in (g.ERR_NBR_OVERFLOW, g.ERR_NONFINITE)
+    q = [1393.6, 346.74, 3.4879 / scale, 2.2119 / scale, 1.5724e-7, 0.72751, 38049.0, 4.3484,
+         -0.57058, 1.95 * scale, 0.15 * scale]
+    _, _, R, h = ci.tersoff_endpoint_cells()
+    with pytest.raises(g.CfnebError) as e:
+        g.evaluate([(scale * R, scale * h)], g.tersoff_potential(q), precision)
+    assert e.value.status in (g.ERR_NBR_OVERFLOW, g.ERR_NONFINITE)
+    assert math.isfinite(g.evaluate([(R0, h0)], g.lj_potential(), precision)[0][0])
