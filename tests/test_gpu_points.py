@@ -125,3 +125,37 @@ def test_more_structures_than_a_grid_axis_holds(g):
     assert np.array_equal(E, np.concatenate([np.tile([w[0][0] for w in want[:8]], 8250), want[8][0]]))
     for k, w in list(enumerate(want[:8])) + [(65528 + j, want[j]) for j in range(8)] + [(66000, want[8])]:
         assert np.array_equal(F[k], w[1][0]) and np.array_equal(V[k], w[2][0])
+
+
+@pytest.mark.parametrize("what", ["path", "X", "F", "Fneb"])
+def test_read_back_follows_the_stream(g, what):
+    """A pinned array whose copy to the device is still queued on the band's stream
+    is the target of a read-back: the queued copy gets the array's old bytes."""
+    import torch
+    R0, h0, R1, h1 = ci.lj_vacancy_hop(reps=(6, 6, 6))
+    s = torch.cuda.Stream()
+    n, N = len(R0), 5
+    opt = g.default_options()
+    opt.k_spring, opt.dt, opt.n_max = 1.0, 0.01, N
+    band = g.create_band((R0, h0), (R1, h1), N, g.lj_potential(), None, opt, stream=s)
+    band.step(1)
+    torch.cuda.synchronize()
+    size = N * (n if what == "path" else n + 3) * 3
+    host = torch.from_numpy(np.random.default_rng(2).uniform(size=size)).pin_memory()
+    old, dev = host.clone(), torch.zeros(size, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(100000000)  # ~50 ms
+        dev.copy_(host, non_blocking=True)
+    ptr = ctypes.cast(host.data_ptr(), ctypes.POINTER(ctypes.c_double))
+    arg = {k: ptr if k == what else None for k in ("X", "F", "Fneb")}
+    if what == "path":
+        st = g.lib().cfneb_get_path(band.handle, None, ptr, None, None, None)
+    else:
+        st = g.lib().cfneb_get_state(band.handle, arg["X"], arg["F"], arg["Fneb"], None, None, None)
+    assert st == g.OK
+    torch.cuda.synchronize()
+    assert torch.equal(dev.cpu(), old)
+    want = band.get_path()["positions"] if what == "path" else band.get_state()[what]
+    assert np.array_equal(host.numpy(), want.ravel())
+    band.destroy()
