@@ -167,7 +167,7 @@ struct __align__(8) TP {  // Tersoff constants in T (derived once per band, on t
     T AeR, BeR;        // A exp(-l1 R), B exp(-l2 R)
     T R2hi, R2lo;      // R^2 as a two-term sum
     T Dlo;             // D - (T)D
-    T xs;              // (beta zeta)^n below which the bond order is a series
+    T xs;              // FP64: (beta zeta)^n below which the bond order is a series
                        // (and a whole number of 8-byte words: staged by word copies)
     // host only (std::exp of the host library): the device reads the result
     __host__ void load(const TersoffParams &p) {
@@ -183,8 +183,7 @@ struct __align__(8) TP {  // Tersoff constants in T (derived once per band, on t
         R2hi = (T)(p.R * p.R);
         R2lo = (T)(p.R * p.R - (double)R2hi);
         Dlo = (T)(p.D - (double)D);
-        // x below 2^-10 and x / 2n below 2^-9 (FP32: 2^-8)
-        xs = (T)std::fmin(1.0 / 1024.0, std::fabs(p.n) / (sizeof(T) == 8 ? 256.0 : 128.0));
+        xs = (T)std::fmin(1.0 / 1024.0, std::fabs(p.n) / 256.0);  // x / 2n below 2^-9
     }
 };
 
