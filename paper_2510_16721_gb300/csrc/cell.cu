@@ -591,23 +591,17 @@ __global__ void __launch_bounds__(TILE) k_bin_order(const Tile *tiles, int ntile
 // from memory.  Same slots as the five passes.
 static_assert(SORT_ATOMS < 65536, "bin starts are kept in 16 bits");
 template <typename T>
-__global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
-    k_bin_sort(const ImgRef *imgs, BandDev *bands) {
+__device__ __forceinline__ void sort_image(const BandDev &b, int img, unsigned short *s_start,
+                                           int *s_w) {
     using T4 = typename Vec4<T>::type;
-    const ImgRef r = imgs[blockIdx.x / SORT_CL];
-    const BandDev b = bands[r.band];
-    const ImgScalars &sc = b.sc[r.img];
-    dep_sync();
-    if (!sc.rebuild) return;  // uniform over the cluster
-    __shared__ unsigned short s_start[SORT_BINS];
-    __shared__ int s_w[SORT_THREADS / 32];
+    const ImgScalars &sc = b.sc[img];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int first = (int)(blockIdx.x % SORT_CL) * SORT_THREADS + tid;
     constexpr int STEP = SORT_CL * SORT_THREADS;
     const int n = b.n, nb = sc.nbins, nb1 = sc.nb[1], nb2 = sc.nb[2];
-    const size_t base = (size_t)r.img * n;
-    int *cnt = b.bin_count + (size_t)r.img * b.nbins_cap;
-    int *start = b.bin_start + (size_t)r.img * (b.nbins_cap + 1);
+    const size_t base = (size_t)img * n;
+    int *cnt = b.bin_count + (size_t)img * b.nbins_cap;
+    int *start = b.bin_start + (size_t)img * (b.nbins_cap + 1);
     int before = 0;  // atoms of the chunks before
     for (int c = 0; c < nb; c += SORT_BINS) {
         const int m = min(SORT_BINS, nb - c);
@@ -664,6 +658,38 @@ __global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
     }
 }
 
+// Sets of more images than SMs are shared out over a cluster per SM, which reads 32
+// images' decisions at once: with a cluster per image, the blocks that find nothing
+// to rebuild were a fifth of a step (256 bands of 31 atoms x 5 images, mixed: 168 us per step, 141 so).
+template <typename T>
+__global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
+    k_bin_sort(const ImgRef *imgs, int count, BandDev *bands) {
+    __shared__ unsigned short s_start[SORT_BINS];
+    __shared__ int s_w[SORT_THREADS / 32];
+    const int clusters = gridDim.x / SORT_CL, step = 32 * clusters;
+    int k = blockIdx.x / SORT_CL;  // uniform over the cluster, as all that follows from it
+    const auto flag = [&](int i) {
+        const ImgRef r = imgs[min(i, count - 1)];
+        return &bands[r.band].sc[r.img].rebuild;
+    };
+    const int l = (int)(threadIdx.x & 31) * clusters;
+    const int *f = flag(k + l);
+    dep_sync();
+    for (;;) {
+        unsigned todo = __ballot_sync(0xffffffffu, k + l < count && *f);
+        while (todo) {
+            const ImgRef r = imgs[k + (__ffs(todo) - 1) * clusters];
+            sort_image<T>(bands[r.band], r.img, s_start, s_w);
+            todo &= todo - 1;
+            if (todo) __syncthreads();  // the next image takes this one's place
+        }
+        k += step;
+        if (k >= count) return;
+        f = flag(k + l);
+        __syncthreads();
+    }
+}
+
 // Cartesian positions R = R~ D (FP64) of a band's images (`per` blocks each), for
 // output.
 template <typename T>
@@ -712,7 +738,8 @@ void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_
 template <typename T>
 void launch_bin_sort(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t s) {
     if (count <= 0) return;
-    launch_dep(k_bin_sort<T>, count * SORT_CL, SORT_THREADS, s, imgs, bands);
+    launch_dep(k_bin_sort<T>, std::min(count, sm_count()) * SORT_CL, SORT_THREADS, s, imgs, count,
+               bands);
 }
 template <typename T>
 void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {

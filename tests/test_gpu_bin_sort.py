@@ -61,3 +61,45 @@ def test_sorted_order_is_the_same(g, bin_scale, skin):
         gb.step(12)
         st.append(gb.get_state())
     assert np.array_equal(st[0]["X"], st[1]["X"]) and np.array_equal(st[0]["F"], st[1]["F"])
+
+
+def test_more_images_than_clusters_points(g):
+    """9,000 structures: each cluster sorts several, in more than one round of 32."""
+    pot = g.lj_potential()
+    few = [(np.array([[0.1 * k, 0.0, 0.0], [1.05 + 0.11 * k, 0.2, 0.0], [2.0, 2.0 + 0.05 * k, 1.0]]),
+            np.eye(3) * (4.0 + 0.3 * k)) for k in range(9)]
+    want = [g.evaluate([s], pot, g.FP64) for s in few]
+    E, F, V = g.evaluate(few * 1000, pot, g.FP64)
+    assert np.array_equal(E, np.tile([w[0][0] for w in want], 1000))
+    for k in range(0, 9000, 7):
+        w = want[k % 9]
+        assert np.array_equal(F[k], w[1][0]) and np.array_equal(V[k], w[2][0])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_more_images_than_clusters_bands(g, precision):
+    """60 bands of 5 moving images whose lists are rebuilt at different steps:
+    bit for bit as alone."""
+    R0, h0, R1, h1 = ci.lj_vacancy_hop(ci.LJ_A, (2, 2, 2))
+    kw = dict(k=1.0, dt=0.01, cell_filter=False, precision=precision, skin=0.1)
+
+    def make(k):
+        return gpu_band(g, R0, h0, R1, h1, 7, g.lj_potential(),
+                        noise=ci.interior_noise(k, 7, len(R0), 0.002 * (k % 20)), **kw)
+
+    bt = g.Batch(precision)
+    bands = [make(k) for k in range(60)]
+    for b in bands:
+        bt.add(b)
+    bt.step(40)
+    stats = set()
+    for k in (0, 7, 19, 31, 32, 33, 58, 59):
+        alone = make(k)
+        alone.step(40)
+        a, b = alone.get_state(), bands[k].get_state()
+        assert all(np.array_equal(a[q], b[q]) for q in ("X", "F", "Fneb", "virials"))
+        stats.add(alone.list_stats()[0] if not isinstance(alone.list_stats(), dict)
+                  else alone.list_stats()["builds"])
+        alone.destroy()
+    assert len(stats) > 2  # rebuilds differ between the bands
+    bt.destroy()
