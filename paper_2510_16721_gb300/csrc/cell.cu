@@ -370,7 +370,9 @@ __device__ inline void bin_of(const ImgScalars &sc, const BandParams *, const fl
 // switches on the conditional node that holds the rebuild kernels (its
 // value is reset to 0 at every launch of the graph).
 // FP32: 12 blocks per SM (40 registers, 18.4 us at 98,303 atoms x 9 images; 18.9
-// with the 48 that the tables read ahead take).
+// with the 48 that the tables read ahead take).  An atom per thread also where the
+// force kernel's tiles hold few atoms (500 FP64 bands of 31 atoms x 5 images, tiles
+// of 4: 62 us with a tile's atoms per block, 29 so).
 template <typename T>
 __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 12 : 8)
     k_bin_assign(const Tile *tiles, BandDev *bands, cudaGraphConditionalHandle cond,
@@ -385,7 +387,7 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 12 : 8)
     if (!sc.rebuild) {
         // keep the bins of the build: thread = slot, offset from the centre
         // of the slot's bin at the current position (unwrapped as at the build)
-        const int t = tile_atom(b, tl);
+        const int t = block_atom(b, tl);
         if (t >= b.n) return;
         const size_t st = (size_t)tl.img * b.n + t;
         const int i = b.slot_atom[st];
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 12 : 8)
     }
     // (through the table: what only a rebuild needs holds no registers above)
     const BandDev &br = bands[tl.band];
-    const int i = tile_atom(br, tl);
+    const int i = block_atom(br, tl);
     if (i >= br.n) return;
     const T *Xi = (const T *)br.X + ((size_t)tl.img * br.rows + i) * 3;
     int bi[3], wrap[3];
@@ -660,7 +662,8 @@ __device__ __forceinline__ void sort_image(const BandDev &b, int img, unsigned s
 
 // Sets of more images than SMs are shared out over a cluster per SM, which reads 32
 // images' decisions at once: with a cluster per image, the blocks that find nothing
-// to rebuild were a fifth of a step (256 bands of 31 atoms x 5 images, mixed: 168 us per step, 141 so).
+// to rebuild were a fifth of a step (256 bands of 31 atoms x 5 images, mixed: 168 us
+// per step, 141 so; 64 bands of 256 to 28,000 atoms x 7 images: 1,545 us either way).
 template <typename T>
 __global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
     k_bin_sort(const ImgRef *imgs, int count, BandDev *bands) {
@@ -679,7 +682,8 @@ __global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
         unsigned todo = __ballot_sync(0xffffffffu, k + l < count && *f);
         while (todo) {
             const ImgRef r = imgs[k + (__ffs(todo) - 1) * clusters];
-            sort_image<T>(bands[r.band], r.img, s_start, s_w);
+            const BandDev b = bands[r.band];
+            sort_image<T>(b, r.img, s_start, s_w);
             todo &= todo - 1;
             if (todo) __syncthreads();  // the next image takes this one's place
         }

@@ -324,6 +324,13 @@ __device__ inline int tile_atom(const BandDev &b, const Tile &tl) {
     return (int)threadIdx.x < b.tile ? tl.t * b.tile + (int)threadIdx.x : b.n;
 }
 
+// As tile_atom, with the atoms of TILE / tile consecutive tiles on the first one's
+// block, one per thread; the other tiles' blocks have none.
+__device__ inline int block_atom(const BandDev &b, const Tile &tl) {
+    const int first = tl.t * b.tile;  // (tile divides TILE)
+    return first % TILE == 0 ? first + (int)threadIdx.x : b.n;
+}
+
 // Exclusive sum over the `lanes` consecutive lanes of a warp that share an atom
 // (a power of two), and the total.  Called by whole warps.
 __device__ inline int lane_scan(int v, int lanes, int &total) {
