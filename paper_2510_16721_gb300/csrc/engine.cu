@@ -973,6 +973,9 @@ void to_host(void *dst, const void *src, size_t bytes, cudaStream_t s) {
     CK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
 }
 
+// state arrays of up to this many bytes on the device are converted on the host
+constexpr size_t STATE_HOST_BYTES = 96 << 10;
+
 // no NaN or Inf among n doubles (exponent bits, four at a time)
 bool all_finite(const double *x, size_t n) {
     const uint64_t E = 0x7ff0000000000000ull;
@@ -2153,19 +2156,46 @@ int cfneb_get_state(const cfneb_band *cb, double *X, double *F, double *Fneb, do
     if (!b) return CFNEB_ERR_INVALID_ARG;
     try {
         enter(b);
-        // converted on the device, then one copy into the caller's array
         double *dst[3] = {X, F, Fneb};
+        const void *src[3] = {b->dv.X, b->dv.F, b->dv.Fneb};
+        // large bands: converted on the device, then one copy into the caller's
+        // array; small ones: the arrays, adjacent in the band's memory, in one copy,
+        // converted here (FP64, 7 images, all three: 31 atoms 38 us, 68 on the device;
+        // 499 atoms 55 and 69, 1,371 atoms 85 and 73; one array: 32 and 36, 37 and
+        // 36, 47 and 36)
+        const size_t per = (size_t)(b->n + 3) * 3, stride = (size_t)b->dv.rows * 3;
+        const char *lo = nullptr, *hi = nullptr;  // from the first wanted array to the last
         for (int which = 0; which < 3; ++which) {
             if (!dst[which]) continue;
+            if (!lo) lo = (const char *)src[which];
+            hi = (const char *)src[which] + b->N * stride * b->ts;
+        }
+        std::vector<char> host(b->N * stride * b->ts <= STATE_HOST_BYTES ? hi - lo : 0);
+        if (!host.empty())
+            CK(cudaMemcpyAsync(host.data(), lo, host.size(), cudaMemcpyDeviceToHost, b->s));
+        for (int which = 0; which < 3; ++which) {
+            if (!dst[which] || !host.empty()) continue;
             if (b->ts == 4) launch_state_store<float>(b->d_self, which, b->N, b->n, b->c, b->s);
             else launch_state_store<double>(b->d_self, which, b->N, b->n, b->c, b->s);
             CK(cudaGetLastError());
-            to_host(dst[which], b->dv.cart, (size_t)b->N * (b->n + 3) * 3 * sizeof(double), b->s);
+            to_host(dst[which], b->dv.cart, b->N * per * sizeof(double), b->s);
         }
         std::vector<ImgScalars> sc(b->N);
         CK(cudaMemcpyAsync(sc.data(), b->dv.sc, b->N * sizeof(ImgScalars),
                            cudaMemcpyDeviceToHost, b->s));
         read_params(b);
+        for (int which = 0; which < 3; ++which) {
+            if (!dst[which] || host.empty()) continue;
+            const char *p = host.data() + ((const char *)src[which] - lo);
+            for (int im = 0; im < b->N; ++im) {
+                double *x = dst[which] + im * per;
+                for (size_t i = 0; i < per; ++i)
+                    x[i] = b->ts == 4 ? (double)((const float *)p)[im * stride + i]
+                                      : ((const double *)p)[im * stride + i];
+                if (which == 0) lattice_rows_public(b, x, 1.0);
+                if (which == 2 && (im == 0 || im == b->N - 1)) std::memset(x, 0, per * sizeof(double));
+            }
+        }
         if (virials)
             for (int i = 0; i < b->N; ++i) std::memcpy(virials + 9 * i, sc[i].V, 9 * sizeof(double));
         if (fire) {

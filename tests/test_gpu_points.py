@@ -127,12 +127,13 @@ def test_more_structures_than_a_grid_axis_holds(g):
         assert np.array_equal(F[k], w[1][0]) and np.array_equal(V[k], w[2][0])
 
 
+@pytest.mark.parametrize("reps", [(6, 6, 6), (10, 10, 10)])
 @pytest.mark.parametrize("what", ["path", "X", "F", "Fneb"])
-def test_read_back_follows_the_stream(g, what):
+def test_read_back_follows_the_stream(g, what, reps):
     """A pinned array whose copy to the device is still queued on the band's stream
     is the target of a read-back: the queued copy gets the array's old bytes."""
     import torch
-    R0, h0, R1, h1 = ci.lj_vacancy_hop(reps=(6, 6, 6))
+    R0, h0, R1, h1 = ci.lj_vacancy_hop(reps=reps)
     s = torch.cuda.Stream()
     n, N = len(R0), 5
     opt = g.default_options()
@@ -158,4 +159,27 @@ def test_read_back_follows_the_stream(g, what):
     assert torch.equal(dev.cpu(), old)
     want = band.get_path()["positions"] if what == "path" else band.get_state()[what]
     assert np.array_equal(host.numpy(), want.ravel())
+    band.destroy()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("reps", [(2, 2, 2), (5, 5, 5), (6, 6, 6), (7, 7, 8)])
+def test_state_read_at_once_or_by_array(g, reps, precision):
+    """Read-backs converted on the host and on the device (arrays above 96 kB): all
+    arrays at once and each by itself are the same values, with zero f_NEB on the end
+    images and the lattice rows c B = c I of the end image."""
+    R0, h0, R1, h1 = ci.lj_vacancy_hop(reps=reps)
+    n, N = len(R0), 5
+    band = gpu_band(g, R0, h0, R1, h1, N, g.lj_potential(), k=1.0, dt=0.01, precision=precision)
+    band.step(2)
+    st = band.get_state()
+    for what in ("X", "F", "Fneb"):
+        a = np.full((N, n + 3, 3), np.nan)
+        arg = {k: g._dptr(a) if k == what else None for k in ("X", "F", "Fneb")}
+        assert g.lib().cfneb_get_state(band.handle, arg["X"], arg["F"], arg["Fneb"], None, None,
+                                       None) == g.OK
+        assert np.array_equal(a, st[what])
+    # (B of the initial cell is I to a few roundings, in units of c = n)
+    assert np.max(np.abs(st["X"][0, n:] - n * np.eye(3))) <= 1e-14 * n and np.any(st["Fneb"][1])
+    assert not np.any(st["Fneb"][[0, -1]])
     band.destroy()
