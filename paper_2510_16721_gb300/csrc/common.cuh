@@ -165,6 +165,8 @@ template <typename T>
 struct __align__(8) TP {  // Tersoff constants in T (derived once per band, on the host)
     T A, B, l1, l2, beta, n, c2, d2, h, R, D, Rhi, pi_2D, pi_4D, inv2n, c2d2;
     T AeR, BeR;        // A exp(-l1 R), B exp(-l2 R)
+    T AeRl, BeRl;      // FP64: what rounding left off (the same for every bond: in a
+                       // total it does not average out)
     T R2hi, R2lo;      // R^2 as a two-term sum
     T Dlo;             // D - (T)D
     T xs;              // FP64: (beta zeta)^n below which the bond order is a series
@@ -180,6 +182,15 @@ struct __align__(8) TP {  // Tersoff constants in T (derived once per band, on t
         c2d2 = (T)(p.c * p.c / (p.d * p.d));
         AeR = (T)(p.A * std::exp(-p.lambda1 * p.R));
         BeR = (T)(p.B * std::exp(-p.lambda2 * p.R));
+        AeRl = BeRl = (T)0;
+        if (sizeof(T) == 8) {
+            const long double a = p.A * std::exp(-(long double)p.lambda1 * p.R),
+                              b = p.B * std::exp(-(long double)p.lambda2 * p.R);
+            AeR = (T)a;
+            BeR = (T)b;
+            AeRl = (T)(a - AeR);
+            BeRl = (T)(b - BeR);
+        }
         R2hi = (T)(p.R * p.R);
         R2lo = (T)(p.R * p.R - (double)R2hi);
         Dlo = (T)(p.D - (double)D);

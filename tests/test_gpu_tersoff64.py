@@ -92,3 +92,55 @@ def test_large_bond_order_argument(g, oracle_mod, product):
     E, F, V = g.evaluate([(R, h)], g.tersoff_potential(par), g.FP64)
     assert np.max(np.abs(F[0] - Fo)) <= 1e-10 * np.max(np.abs(Fo))
     assert abs(E[0] - e.sum()) <= 1e-10 * abs(e).sum()
+
+
+def _energy_long(R, h, q):
+    """Tersoff energy in long double (the oracle's g, as published, cancels to 1e-8:
+    2e-15 of a total)."""
+    L = np.longdouble
+    rc, W = q["R"] + q["D"], h.astype(L)
+    I, D = [], []
+    for t in np.ndindex(3, 3, 3):
+        d = R[None, :, :] + (np.array(t) - 1) @ h - R[:, None, :]
+        i, j = np.nonzero(((d * d).sum(2) < (rc + 0.01) ** 2) & ((d * d).sum(2) > 1e-6))
+        I.append(i)
+        D.append(R[j].astype(L) + (np.array(t) - 1).astype(L) @ W - R[i].astype(L))
+    I, D = np.concatenate(I), np.concatenate(D)
+    r = np.sqrt((D * D).sum(1))
+    q = {k: L(v) for k, v in q.items()}
+    half_pi = 2 * np.arctan(L(1))
+    fc = np.where(r < q["R"] - q["D"], L(1), (1 - np.sin(half_pi * (r - q["R"]) / q["D"])) / 2)
+    fc = np.where(r < q["R"] + q["D"], fc, L(0))
+    E, u = L(0), D / r[:, None]
+    for i in range(len(R)):
+        e = np.nonzero((I == i) & (fc > 0))[0]
+        x = q["h"] - u[e] @ u[e].T
+        c2, d2 = q["c"] ** 2, q["d"] ** 2
+        z = ((1 + c2 / d2 * x * x / (d2 + x * x)) * (1 - np.eye(len(e)))) @ fc[e]
+        b = np.where(z > 0, (1 + (q["beta"] * z) ** q["n"]) ** (-1 / (2 * q["n"])), L(1))
+        fr, fa = (q[a] * np.exp(-q[l] * r[e]) for a, l in (("A", "lambda1"), ("B", "lambda2")))
+        E += (fc[e] * (fr - b * fa)).sum() / 2
+    return E
+
+
+@pytest.mark.parametrize("kind,reps", [("diamond", (5, 4, 6)), ("graphite", (6, 4, 5)),
+                                       ("disordered", (4, 3, 4))])
+@pytest.mark.parametrize("images", [0, 84])
+def test_total_energy_to_roundings(g, oracle_mod, kind, reps, images):
+    """FP64 totals against long double: roundings of single bonds average out, those
+    of constants shared by all bonds would not (8e-16 of the total).  Four lanes per
+    atom (images = 0: a single point) and, with 84 images, one thread (the end
+    image's step energy)."""
+    R, h = _carbon(kind, reps, 0, 3)
+    want = _energy_long(R, h, oracle_mod.TERSOFF_C1988)
+    if images:
+        R1 = R.copy()
+        R1[0, 0] += 0.1
+        o = g.default_options()
+        o.n_max = images
+        band = g.create_band((R, h), (R1, h), images, g.tersoff_potential(), None, o)
+        E = band.image_scalars()["E"][0]
+        band.destroy()
+    else:
+        E = g.evaluate([(R, h)], g.tersoff_potential(), g.FP64)[0][0]
+    assert abs(E - want) <= 4e-16 * abs(want)
