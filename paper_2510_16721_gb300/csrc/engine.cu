@@ -1011,9 +1011,16 @@ int atom_tile(const cfneb_potential *pot, int precision, long long n, long long 
     if (pot->kind == CFNEB_LJ && precision == CFNEB_FP64)
         lanes = fp64_lanes(n, images, lj_fp64_instr((double)n, volume, rc), cells ? 2 : 1);
     else if (cells) lanes = lanes_per_atom(atoms, LJ_LANES_FP32);
-    // FP64 many-body kernels take four lanes per atom (32 atoms per block)
-    // where the band's blocks would leave SMs idle, else one
-    if (pot->kind != CFNEB_LJ && precision == CFNEB_FP64 && atoms < 152 * 2 * TILE) lanes = 4;
+    // FP64 many-body bands whose blocks would leave SMs idle: 32 atoms per tile.  The
+    // Tersoff site kernel and the lists then work with four lanes per atom; the network
+    // kernel, the energy pass and the gather leave three quarters of a block's threads
+    // without an atom, which is still the faster spread for the network kernel while
+    // its blocks are all resident, three per SM (FP64, per step, tiles of 32 and 128:
+    // 576 atoms x 7 images 246 and 255 us, 1,728 x 7 272 and 278, 2,520 x 7 391 and 319)
+    if (precision == CFNEB_FP64 &&
+        ((pot->kind == CFNEB_TERSOFF && atoms < 152 * 2 * TILE) ||
+         (pot->kind == CFNEB_NEP && atoms <= 152 * 3 * TILE / 4)))
+        lanes = 4;
     return TILE / lanes;
 }
 

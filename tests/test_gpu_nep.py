@@ -145,3 +145,18 @@ def test_large_nep_band_image_properties(g):
     _, Fm, _ = g.evaluate([(R, h)], pot, g.MIXED)
     idx = rng.choice(len(R), 64, replace=False)
     assert np.max(np.abs(Fm[0][idx] - F[idx])) <= 1e-4
+
+
+def test_small_and_large_tiles_agree(g):
+    """FP64: a disordered cell with 32 atoms per tile and tiled past the line of that
+    rule (128 per tile): per-atom forces agree and the totals scale."""
+    _, _, Rd, hd = ci.tersoff_endpoint_cells()
+    R, h = ci.tile(Rd, hd, (5, 5, 5))
+    R = R + np.random.default_rng(8).normal(0.0, 0.06, R.shape)
+    Rt, ht = ci.tile(R, h, (3, 3, 2))
+    assert len(R) <= 152 * 3 * 32 < len(Rt)
+    pot = g.nep_potential(_weights(), RC)
+    (E1, F1, V1), (E2, F2, V2) = (g.evaluate([s], pot, g.FP64) for s in ((R, h), (Rt, ht)))
+    assert np.max(np.abs(F2[0].reshape(18, -1, 3) - F1[0])) <= 1e-10 * max(1.0, np.max(np.abs(F1[0])))
+    assert abs(E2[0] - 18 * E1[0]) <= 1e-10 * abs(E2[0])
+    assert np.max(np.abs(V2[0] - 18 * V1[0])) <= 1e-9 * max(1.0, np.max(np.abs(V2[0])))
