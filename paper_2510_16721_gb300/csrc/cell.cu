@@ -370,9 +370,10 @@ __device__ inline void bin_of(const ImgScalars &sc, const BandParams *, const fl
 // switches on the conditional node that holds the rebuild kernels (its
 // value is reset to 0 at every launch of the graph).
 // FP32: 12 blocks per SM (40 registers, 18.4 us at 98,303 atoms x 9 images; 18.9
-// with the 48 that the tables read ahead take).  An atom per thread also where the
-// force kernel's tiles hold few atoms (500 FP64 bands of 31 atoms x 5 images, tiles
-// of 4: 62 us with a tile's atoms per block, 29 so).
+// with the 48 that the tables read ahead take).  Where the force kernel's tiles hold
+// few atoms, large sets put an atom on every thread (500 FP64 bands of 31 atoms x 5
+// images, tiles of 4: 62 us with a tile's atoms per block, 29 so), small ones a tile's
+// atoms on a block (2,915 FP64 atoms x 5 images, tiles of 32: 10.2 us, 12.8 packed).
 template <typename T>
 __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 12 : 8)
     k_bin_assign(const Tile *tiles, BandDev *bands, cudaGraphConditionalHandle cond,
@@ -660,37 +661,39 @@ __device__ __forceinline__ void sort_image(const BandDev &b, int img, unsigned s
     }
 }
 
+template <typename T>
+__global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
+    k_bin_sort(const ImgRef *imgs, BandDev *bands) {
+    __shared__ unsigned short s_start[SORT_BINS];
+    __shared__ int s_w[SORT_THREADS / 32];
+    const ImgRef r = imgs[blockIdx.x / SORT_CL];
+    const BandDev b = bands[r.band];
+    dep_sync();
+    if (b.sc[r.img].rebuild) sort_image<T>(b, r.img, s_start, s_w);  // uniform over the cluster
+}
 // Sets of more images than SMs are shared out over a cluster per SM, which reads 32
 // images' decisions at once: with a cluster per image, the blocks that find nothing
 // to rebuild were a fifth of a step (256 bands of 31 atoms x 5 images, mixed: 168 us
 // per step, 141 so; 64 bands of 256 to 28,000 atoms x 7 images: 1,545 us either way).
 template <typename T>
 __global__ void __cluster_dims__(SORT_CL, 1, 1) __launch_bounds__(SORT_THREADS)
-    k_bin_sort(const ImgRef *imgs, int count, BandDev *bands) {
+    k_bin_sort_many(const ImgRef *imgs, int count, BandDev *bands) {
     __shared__ unsigned short s_start[SORT_BINS];
     __shared__ int s_w[SORT_THREADS / 32];
     const int clusters = gridDim.x / SORT_CL, step = 32 * clusters;
-    int k = blockIdx.x / SORT_CL;  // uniform over the cluster, as all that follows from it
-    const auto flag = [&](int i) {
-        const ImgRef r = imgs[min(i, count - 1)];
-        return &bands[r.band].sc[r.img].rebuild;
-    };
     const int l = (int)(threadIdx.x & 31) * clusters;
-    const int *f = flag(k + l);
     dep_sync();
-    for (;;) {
-        unsigned todo = __ballot_sync(0xffffffffu, k + l < count && *f);
-        while (todo) {
+    // k: uniform over the cluster, as all that follows from it
+    for (int k = blockIdx.x / SORT_CL; k < count; k += step) {
+        const ImgRef f = imgs[min(k + l, count - 1)];
+        unsigned todo =
+            __ballot_sync(0xffffffffu, k + l < count && bands[f.band].sc[f.img].rebuild);
+        for (; todo; todo &= todo - 1) {
             const ImgRef r = imgs[k + (__ffs(todo) - 1) * clusters];
             const BandDev b = bands[r.band];
             sort_image<T>(b, r.img, s_start, s_w);
-            todo &= todo - 1;
-            if (todo) __syncthreads();  // the next image takes this one's place
+            __syncthreads();  // the next image takes this one's place
         }
-        k += step;
-        if (k >= count) return;
-        f = flag(k + l);
-        __syncthreads();
     }
 }
 
@@ -742,8 +745,10 @@ void launch_bin_order(const Tile *tiles, int ntiles, BandDev *bands, cudaStream_
 template <typename T>
 void launch_bin_sort(const ImgRef *imgs, int count, BandDev *bands, cudaStream_t s) {
     if (count <= 0) return;
-    launch_dep(k_bin_sort<T>, std::min(count, sm_count()) * SORT_CL, SORT_THREADS, s, imgs, count,
-               bands);
+    if (count <= sm_count())
+        launch_dep(k_bin_sort<T>, count * SORT_CL, SORT_THREADS, s, imgs, bands);
+    else
+        launch_dep(k_bin_sort_many<T>, sm_count() * SORT_CL, SORT_THREADS, s, imgs, count, bands);
 }
 template <typename T>
 void launch_cartesian(int N, int n, BandDev *band, cudaStream_t s) {

@@ -335,10 +335,12 @@ __device__ inline int tile_atom(const BandDev &b, const Tile &tl) {
     return (int)threadIdx.x < b.tile ? tl.t * b.tile + (int)threadIdx.x : b.n;
 }
 
-// As tile_atom, with the atoms of TILE / tile consecutive tiles on the first one's
-// block, one per thread; the other tiles' blocks have none.
+// As tile_atom; in grids of more blocks than fit at a time, with the atoms of TILE /
+// tile consecutive tiles on the first one's block, one per thread, and none on the
+// other tiles' blocks.
 __device__ inline int block_atom(const BandDev &b, const Tile &tl) {
     const int first = tl.t * b.tile;  // (tile divides TILE)
+    if (gridDim.x <= 152 * 16) return tile_atom(b, tl);
     return first % TILE == 0 ? first + (int)threadIdx.x : b.n;
 }
 
