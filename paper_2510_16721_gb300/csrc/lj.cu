@@ -704,9 +704,12 @@ __device__ inline void lj_list_lanes(const BandDev &b, const Tile &tl, const LJG
 }
 
 // LANES false: an atom per thread throughout (FP32 sets that fill the GPU; with the
-// other form in the kernel its registers cost 27,435 atoms 2% of a step).
+// other form in the kernel its registers cost 27,435 atoms 2% of a step).  FP32 with
+// lanes: five blocks per SM, which leave 96 registers and no spills (2,915 atoms x 5
+// images 44.9 us; 51.1 with the 72 that the compiler takes by itself.  FP64 lists, also
+// of large sets, keep those: 59,999 atoms 3% of a step).
 template <typename T, bool LANES>
-__global__ void __launch_bounds__(TILE)
+__global__ void __launch_bounds__(TILE, LANES && sizeof(T) == 4 ? 5 : 0)
     k_lj_list(const Tile *tiles, int ntiles, BandDev *bands, int split) {
     dep_sync();
     __shared__ LJGeom<float> g;
