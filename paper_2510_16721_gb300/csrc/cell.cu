@@ -1,7 +1,7 @@
 // Cell filter inverse map and cell-list build.
 //
 // Map-back (Sec. II.C): the lattice rows of X hold c B; B = X_lat / c is
-// symmetrised and D = B^(1/2) taken with a cyclic Jacobi eigen-solve in FP64
+// symmetrised and D = B^(1/2) taken with a coupled Newton-Schulz iteration in FP64
 // (rotation-free variant), or D = X_lat / c (deformation-gradient variant).
 // Then h = h0 D, and the bin geometry of the image is derived from the
 // perpendicular widths of h.

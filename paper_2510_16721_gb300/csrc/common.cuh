@@ -557,10 +557,6 @@ __device__ inline double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ inline double warp_max(double v) {
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
 
 // ---- lane-parallel 3x3 algebra (map-back, lattice force) -------------------
 //
@@ -698,8 +694,9 @@ __device__ inline bool image_cell_warp(const CellIn &k, double xlat, ImgScalars 
 // corrections, which took ~190 of a Tersoff atom's ~1,770 instructions (98,303
 // atoms x 9 images: site terms 83.8 -> 79.8 us, offset refresh 21.1 -> 18.0 us;
 // the table below costs the moving warp 0.6 us, which small bands see).
-// g = 2^-22 A for carbon's 2.25 A lists in any cell up to ~800 A, the least
-// power of two with the cell's extent below 2^30 g and rl below 2^24 g / 1.1.
+// g is the least power of two with 1.25 times the cell's extent below 2^30 g and rl
+// below 2^24 g / 1.1: 2^-22 A for carbon's 2.25 A lists in cells up to 204 A, 2^-21 A
+// up to 409 A, and so on; the remainders keep the precision.
 constexpr int SHIFTS = 27;  // lattice shifts t_a in {-1, 0, 1}; others are formed on the fly
 struct F2 {  // unevaluated sum hi + lo of two floats
     float hi, lo;
@@ -964,35 +961,11 @@ __device__ inline void block_sum(double (&v)[K], double *out) {
     __syncthreads();  // red[] may be reused by a later call
 }
 
-// Sum K per-thread values of type T over a TILE-thread block: within each
-// warp in T (fixed butterfly), across warps in FP64; thread 0 receives the
-// totals.  With T = float the long accumulations (across warps, tiles and
-// images) stay FP64 while the per-element work avoids FP64 arithmetic.
-template <int K, typename T>
-__device__ inline void block_sum_t(T (&v)[K], double *out) {
-    __shared__ double red[TILE / 32][K > 0 ? K : 1];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        T s = v[k];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) red[w][k] = (double)s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            double s = 0.0;
-            for (int q = 0; q < TILE / 32; ++q) s += red[q][k];
-            out[k] = s;
-        }
-    }
-    __syncthreads();
-}
-
-// As block_sum_t, but the totals go straight to dst[0..K-1]: lane k of warp
-// 0 sums value k across the warps, in the same order (so the same bits), and
-// the FP64 additions take K/32 warp instructions instead of K in thread 0
+// Sum K per-thread values of type T over a TILE-thread block: within each warp in T
+// (fixed butterfly), across warps in FP64.  With T = float the long accumulations
+// (across warps, tiles and images) stay FP64 while the per-element work avoids FP64
+// arithmetic.  The totals go to dst[0..K-1]: lane k of warp 0 sums value k across the
+// warps, so the FP64 additions take K/32 warp instructions instead of K in thread 0
 // (an FP64 instruction occupies a warp's FP64 pipe for ~64 cycles here).
 template <int K, typename T>
 __device__ inline void block_sum_store(T (&v)[K], double *dst) {
@@ -1071,20 +1044,6 @@ __device__ inline void block_sum_any(double (&v)[K], double *out) {
         }
     }
     __syncthreads();
-}
-
-// block-wide maximum; thread 0 receives it
-__device__ inline double block_max_any(double v) {
-    __shared__ double red[32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    v = warp_max(v);
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    double m = red[0];
-    if (threadIdx.x == 0)
-        for (int q = 1; q < nw; ++q) m = fmax(m, red[q]);
-    __syncthreads();
-    return m;
 }
 
 // threads of the per-image / per-band reduction kernels

@@ -5,12 +5,11 @@
 // and to pick the climbing image, but a total over ~1e5 atoms carries errors
 // of ~1e-2 eV (in a perfect crystal every atom makes the same rounding
 // error).  Reported energies therefore come from these kernels, which redo
-// the energy -- and only the energy -- in FP64 from the cell list of the
-// configuration being reported: pair vectors from the two-term offsets (exact
-// positions), bin displacements and wrap corrections in FP64, then the
-// Tersoff or NEP-style energy of Sec. II.B's per-atom split (Lennard-Jones:
-// k_lj_energy64, beside its force kernels) summed over atoms in FP64.  Used by cfneb_get_path and cfneb_evaluate, never inside a
-// relaxation step.
+// the energy -- and only the energy -- in FP64 from the neighbour lists of the
+// configuration being reported: pair vectors in FP64 (entries64), then the Tersoff
+// or NEP-style energy of Sec. II.B's per-atom split (Lennard-Jones: k_lj_energy64,
+// beside its force kernels) summed over atoms in FP64.  Used by cfneb_get_path and,
+// in mixed precision, by cfneb_evaluate, never inside a relaxation step.
 //
 // FP64 arithmetic is scarce on this GPU, so it is spent on the terms only:
 // the atom's neighbour list (rebuilt with the cell list) is walked instead of
@@ -57,9 +56,12 @@ __device__ inline int entries64(const BandDev &b, const Tile &tl, int t, double 
         int s[3] = {0, 0, 0};
         float lo[3] = {0.0f, 0.0f, 0.0f};
         if (code != CODE_ZERO) grid_shift(G, sc, code, s, lo);
-        const double x = f2d((float)(grid_diff(pj.x, pi.x) + s[0]) * G.g) + f2d((lj.x - li.x) + lo[0]);
-        const double y = f2d((float)(grid_diff(pj.y, pi.y) + s[1]) * G.g) + f2d((lj.y - li.y) + lo[1]);
-        const double z = f2d((float)(grid_diff(pj.z, pi.z) + s[2]) * G.g) + f2d((lj.z - li.z) + lo[2]);
+        const auto component = [&](float j, float i, float jl, float il, int c) {
+            return f2d((float)(grid_diff(j, i) + s[c]) * G.g) + f2d((jl - il) + lo[c]);
+        };
+        const double x = component(pj.x, pi.x, lj.x, li.x, 0);
+        const double y = component(pj.y, pi.y, lj.y, li.y, 1);
+        const double z = component(pj.z, pi.z, lj.z, li.z, 2);
         cnt += add_entry(E, cnt, x, y, z, rc * rc);
     }
     return cnt;

@@ -594,9 +594,9 @@ __global__ void __launch_bounds__(TILE) k_lj_energy64(const Tile *tiles, BandDev
     if (threadIdx.x == 0) b.atom_part[((size_t)tl.img * b.atpi + tl.t) * NPART] = tot[0];
 }
 
-// Neighbour list of a rebuilt image (bands with a skin): one thread per atom
-// walks the cell-list stencil and keeps every candidate within rl, coalesced
-// as [entry][atom].  Entries inside rc at the build come first and those of
+// Neighbour list of a rebuilt image (bands with a skin): one thread per atom (or
+// several lanes, lj_list_lanes) walks the cell-list stencil and keeps every candidate
+// within rl, coalesced as [entry][atom].  Entries inside rc at the build come first and those of
 // the skin shell after them, so that the force kernel's warps mostly agree
 // on which entries have a pair term.  Images that keep their cell list keep
 // their list too.  The walk runs in FP32 in both precisions: FP64 bands

@@ -59,6 +59,18 @@ def test_single_points(g, oracle_mod, pot, kind, reps, shear, wraps):
     assert abs(E[0] - np.sum(e)) <= 1e-10 * np.sum(np.abs(e))
 
 
+@pytest.mark.parametrize("reps", [(75, 1, 2), (90, 1, 2), (170, 1, 1), (2, 200, 1)])
+def test_long_cells(g, oracle_mod, reps):
+    """Extents on both sides of 205 A, where the grid becomes coarser, and of 410 and
+    820 A."""
+    R, h, kh = _carbon("diamond", reps, 0.0, 1, 11)
+    R, h = f32_structure(R, h)
+    e, Fo, _ = oracle_mod.Tersoff().evaluate(R, h)
+    E, F, V = g.evaluate([(R, h)], g.tersoff_potential(), g.MIXED)
+    assert np.max(np.abs(F[0] - Fo)) <= max(1e-4, 1e-6 * np.max(np.abs(Fo)))
+    assert abs(E[0] - np.sum(e)) <= 1e-10 * np.sum(np.abs(e))
+
+
 @pytest.mark.parametrize("wraps", [1, 3])
 @pytest.mark.parametrize("reps", [(2, 1, 1), (6, 4, 3)])
 def test_moving_band(g, oracle_mod, reps, wraps):
