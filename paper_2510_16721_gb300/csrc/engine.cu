@@ -1088,12 +1088,15 @@ void eval_points_t(const cfneb_structure *S, int count, const cfneb_potential *p
     std::vector<ImgRef> imgs;
     size_t atoms = 0, big = 0;
     int max_bins = 0, minb = 0;
+    BandParams same;  // what all structures have in common
+    std::memset(&same, 0, sizeof(same));
+    const double rc = fill_potential(pot, same);
     for (int k = 0; k < count; ++k) {
         BandDev &d = dv[k];
         BandParams &P = bp[k];
         std::memset(&d, 0, sizeof(d));
-        std::memset(&P, 0, sizeof(P));
-        const double rc = fill_potential(pot, P), vol = std::fabs(det3(S[k].cell));
+        P = same;
+        const double vol = std::fabs(det3(S[k].cell));
         const int n = S[k].n_atoms;
         d.n = P.n = n;
         d.rows = (n + 3 + 3) / 4 * 4;
