@@ -10,6 +10,8 @@
 // spacings and energies the kernels computed, because they change the launch
 // shape.
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <chrono>
@@ -960,16 +962,29 @@ double fill_potential(const cfneb_potential *pot, BandParams &P) {
     return rc;
 }
 
-// Device to caller's memory, in stream order.  A fresh array's pages are touched
-// first: a copy into pages that nobody has written yet faults them in one by one
-// from the device (26 MB: 24 ms, against ~1 ms once touched).  The touch leaves
-// every byte as it is, also against writers: what the stream still does to the
-// array before this copy (a pinned array may be the source of an earlier one) is
-// not disturbed.
-void to_host(void *dst, const void *src, size_t bytes, cudaStream_t s) {
+// Maps the pages of an array without changing a byte of it: what the caller's stream
+// still does to the array (a pinned one may be the source of a queued copy) is not
+// disturbed.  Asked of the kernel in one call (28 MB of fresh pages: 0.5 ms more than
+// mapped ones; a write of nothing to each page, the form for small arrays and the
+// fallback, faults twice: 9 ms).
+void map_pages(void *dst, size_t bytes) {
+    if (!bytes) return;
+#ifndef MADV_POPULATE_WRITE
+    constexpr int MADV_POPULATE_WRITE = 23;  // Linux 5.14
+#endif
+    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE), first = (uintptr_t)dst / page * page;
+    const size_t span = ((uintptr_t)dst + bytes - first + page - 1) / page * page;
+    if (bytes > 65536 && madvise((void *)first, span, MADV_POPULATE_WRITE) == 0) return;
     unsigned char *p = (unsigned char *)dst;
     for (size_t i = 0; i < bytes; i += 4096) __atomic_fetch_or(p + i, 0, __ATOMIC_RELAXED);
-    if (bytes) __atomic_fetch_or(p + bytes - 1, 0, __ATOMIC_RELAXED);
+    __atomic_fetch_or(p + bytes - 1, 0, __ATOMIC_RELAXED);
+}
+
+// Device to caller's memory, in stream order.  The pages are mapped first: a copy into
+// pages that nobody has written yet faults them in one by one from the device (26 MB:
+// 24 ms, against ~1 ms once mapped).
+void to_host(void *dst, const void *src, size_t bytes, cudaStream_t s) {
+    map_pages(dst, bytes);
     CK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
 }
 
