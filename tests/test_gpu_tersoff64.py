@@ -144,3 +144,18 @@ def test_total_energy_to_roundings(g, oracle_mod, kind, reps, images):
     else:
         E = g.evaluate([(R, h)], g.tersoff_potential(), g.FP64)[0][0]
     assert abs(E - want) <= 4e-16 * abs(want)
+
+
+@pytest.mark.parametrize("lam", [0.01, 0.5, 40.0, 250.0, 300.0, 340.0])
+def test_bond_constants_over_exponents(g, oracle_mod, lam):
+    """A exp(-lambda1 R) over the exponents that a potential may have: the two-term
+    constant (lambda1 R up to 600) and, at the largest, the plain one.  A repulsion's
+    exponent is rounded at lambda1 R and lambda1 (r - R), units of up to 663 and 240
+    (3e-13 with r's own), and takes lambda1 times the error of r: positions below 16 A
+    rounded twice for each atom, 4e-15 A."""
+    q = dict(oracle_mod.TERSOFF_C1988)
+    q["lambda1"], q["A"] = lam, float(np.exp(lam * 1.45))
+    R, h = _carbon("graphite", (3, 3, 2), 0, 3)
+    E = g.evaluate([(R, h)], g.tersoff_potential([q[k] for k in q]), g.FP64)[0][0]
+    want = _energy_long(R, h, q)
+    assert abs(E - want) <= (3e-13 + 4e-15 * lam) * abs(want)
